@@ -4,7 +4,9 @@
 // temperature == 0 (greedy): one launch.  Block (chunk, row, sequence) finds the arg-max of its
 // chunk of a target row; the last block of the sequence merges the rows' arg-maxes and walks.
 //
-// temperature > 0 (multi-round speculative sampling over siblings): two launches.
+// temperature > 0 (multi-round speculative sampling over siblings): one launch that walks every sequence's
+// tree with a cluster of its own (accept_walk.cuh), as long as a cluster's registers hold the vocabulary.
+// Larger vocabularies (131073 entries and more): two launches.
 //   chain kernel  One thread-block cluster per (sequence, expanded node).  The cluster keeps the
 //     node's target and draft distributions in shared memory (each block a slice of the vocabulary,
 //     read from HBM once) and runs the node's whole rejection chain over its selected children: the
@@ -244,6 +246,10 @@ __device__ __forceinline__ float exp_scaled(float zs, float gmax) {
 __device__ __forceinline__ float prob_of(float z, float inv_t, float gmax, float c) {
     return __fmul_rn(exp_scaled(scale_logit(z, inv_t), gmax), c);
 }
+
+}  // namespace eagle2
+#include "accept_walk.cuh"
+namespace eagle2 {
 
 template <bool RESIDENT, bool VEC>
 __global__ void __launch_bounds__(kChainThreads)
@@ -822,6 +828,43 @@ accept_bonus_kernel(const float* __restrict__ target_logits, long long t_stride,
     }
 }
 
+// A cluster's registers hold the two rows of a node up to 8 blocks x 512 threads x 32 tokens.  The walk reads
+// the rows of two or three nodes of a sequence where the chain kernel reads those of every expanded node:
+// per call at V = 128256 and B = 1 / 4 / 8 / 16 / 32 37.8 / 74 / 138 / 257 / 483 -> 34.2 / 39 / 45 / 58 / 89 us,
+// with the candidates as proposal 31 / 63 / 115 / 218 / 408 -> 13 / 18.5 / 21 / 27 / 41 us; at V = 32000
+// 24 / 37 / 49 / 81 / 140 -> 26 / 32 / 33 / 42 / 38 us, one launch less in the batch-1 cycle.
+static bool walk_holds(int V) { return V <= kWalkMaxCluster * kWalkThreads * 32; }
+
+// The slice of a block is the shortest that leaves every sequence a cluster at once on nine tenths of the
+// SMs (clusters do not tile the rest); more sequences than that take the longest slices.
+static int launch_walk(int B, int V, bool vec, const float* target, long long t_stride, const float* draft, long long d_stride,
+                       const int32_t* sel_index, const int32_t* sel_parent, const int32_t* sel_token, const int32_t* n_sel,
+                       const float* u_accept, const float* u_bonus, int k, int D, int m, float inv_t, int32_t* acc_len,
+                       int32_t* acc_path, int32_t* bonus_token, int32_t* d_status, cudaStream_t st) {
+    int nf = 1, cs = 1;
+    for (;; nf *= 2) {
+        cs = (V + kWalkThreads * 4 * nf - 1) / (kWalkThreads * 4 * nf);
+        if (nf == 8 || cs == 1 || (cs <= kWalkMaxCluster && (long long)B * cs <= sm_count() * 9 / 10)) break;
+    }
+    if ((long long)B * cs > 0x7fffffffLL) return EAGLE2_ERR_SHAPE;
+#define EAGLE2_WALK_CASE(NF_)                                                                                        \
+    case NF_: {                                                                                                      \
+        auto kern = draft ? (vec ? accept_walk_kernel<NF_, true, true> : accept_walk_kernel<NF_, false, true>)        \
+                          : (vec ? accept_walk_kernel<NF_, true, false> : accept_walk_kernel<NF_, false, false>);      \
+        return launch_chained(kern, dim3((unsigned)(B * cs)), dim3(kWalkThreads), 0, st, (unsigned)cs, target, t_stride, \
+                              draft, d_stride, sel_index, sel_parent, sel_token, n_sel, u_accept, u_bonus, V, k, D, m,  \
+                              inv_t, acc_len, acc_path, bonus_token, d_status);                                       \
+    }
+    switch (nf) {
+        EAGLE2_WALK_CASE(1)
+        EAGLE2_WALK_CASE(2)
+        EAGLE2_WALK_CASE(4)
+        EAGLE2_WALK_CASE(8)
+    }
+#undef EAGLE2_WALK_CASE
+    return EAGLE2_ERR_SHAPE;
+}
+
 }  // namespace eagle2
 
 using namespace eagle2;
@@ -875,6 +918,9 @@ extern "C" int eagle2_accept(const float* target_logits, long long t_stride,
 
     // ---- temperature > 0 --------------------------------------------------------------------------
     const float inv_t = 1.0f / temperature;
+    if (walk_holds(V)) return launch_walk(B, V, vec, target_logits, t_stride, draft_logits_all, d_stride, sel_index, sel_parent,
+                                            sel_token, n_sel, u_accept, u_bonus, k, D, m, inv_t, acc_len, acc_path, bonus_token,
+                                            d_status, st);
     // Cluster size.  One sequence: the smallest power of two whose vocabulary slices fit in shared
     // memory (many short slices: the chain of the root's children sets the time).  A batch has more
     // nodes than clusters fit on the device at once, so the fewest blocks that can hold the rows give

@@ -104,7 +104,8 @@ class CycleBuffers:
         """Kernel launches of this library in one cycle (for bookkeeping in benchmarks)."""
         s = self.shape
         per_layer = e2.tree_attention_launches(s.B, s.m, s.Hq, s.Hkv, s.d, s.max_kv_len)
-        return s.D + 1 + s.n_layers * per_layer + (2 if s.temperature > 0 else 1) + 2
+        accept = 2 if s.temperature > 0 and s.V > 131072 else 1  # larger vocabularies: chains, then the walk
+        return s.D + 1 + s.n_layers * per_layer + accept + 2
 
 
 def enqueue_cycle(buf: CycleBuffers, draft_rows, target_logits, u_accept, u_bonus, q_layers, k_layers,
