@@ -835,7 +835,7 @@ accept_bonus_kernel(const float* __restrict__ target_logits, long long t_stride,
 // 24 / 37 / 49 / 81 / 140 -> 26 / 32 / 33 / 42 / 38 us, one launch less in the batch-1 cycle.
 static bool walk_holds(int V) { return V <= kWalkMaxCluster * kWalkThreads * 32; }
 
-// The slice of a block is the shortest that leaves every sequence a cluster at once on nine tenths of the
+// The slice of a block is the shortest that leaves every sequence a cluster at once on four fifths of the
 // SMs (clusters do not tile the rest); more sequences than that take the longest slices.
 static int launch_walk(int B, int V, bool vec, const float* target, long long t_stride, const float* draft, long long d_stride,
                        const int32_t* sel_index, const int32_t* sel_parent, const int32_t* sel_token, const int32_t* n_sel,
@@ -844,7 +844,7 @@ static int launch_walk(int B, int V, bool vec, const float* target, long long t_
     int nf = 1, cs = 1;
     for (;; nf *= 2) {
         cs = (V + kWalkThreads * 4 * nf - 1) / (kWalkThreads * 4 * nf);
-        if (nf == 8 || cs == 1 || (cs <= kWalkMaxCluster && (long long)B * cs <= sm_count() * 9 / 10)) break;
+        if (nf == 8 || cs == 1 || (cs <= kWalkMaxCluster && (long long)B * cs <= sm_count() * 4 / 5)) break;
     }
     if ((long long)B * cs > 0x7fffffffLL) return EAGLE2_ERR_SHAPE;
 #define EAGLE2_WALK_CASE(NF_)                                                                                        \

@@ -113,6 +113,12 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity) && clock64() - t0 < kWaitCycles) {}
 }
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
 __device__ __forceinline__ void fence_proxy_async() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -307,6 +313,19 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
+}
+// this shared-memory address in block `rank` of the cluster
+__device__ __forceinline__ uint32_t in_block(uint32_t addr, uint32_t rank) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    return remote;
+}
+// Bulk copy from this block's shared memory to a block of the cluster, counted by a barrier there (addresses
+// and size multiples of 16).
+__device__ __forceinline__ void bulk_copy_to(uint32_t remote_dst, uint32_t src, uint32_t bytes, uint32_t remote_bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(remote_dst), "r"(src), "r"(bytes), "r"(remote_bar)
+                 : "memory");
 }
 // arrive on the barrier at this shared-memory offset in block `rank` of the cluster
 __device__ __forceinline__ void mbar_arrive_in(uint32_t bar, uint32_t rank) {

@@ -5,15 +5,20 @@
 // g = Hq/Hkv query heads that share a KV head are packed into M = m*g query rows, so every K/V tile
 // read from HBM serves all of them.  A block owns (sequence, KV head, row block, KV split) with up
 // to 256 packed rows (two 128-row UMMA tiles) and is warp specialised:
-//   softmax warps  one thread per query row.  S = Q.K^T arrives in tensor memory; the thread reads
-//                  its row, applies scale, tree mask and a lazily rescaled running maximum, and
-//                  writes P as bf16 back into tensor memory over the scores it consumed.
-//   TMA warp       streams 128-key K and V tiles (128-byte swizzled) through a ring of stages.
-//   MMA warp       one thread issues tcgen05.mma: S = Q.K^T (operands in shared memory) and
-//                  O += P.V (P from tensor memory, V in shared memory, MN-major), two score slots
-//                  in flight so that the tensor pipe and the softmax warps overlap.
-// The block writes final rows when its sequence needs a single split, otherwise an unnormalised
-// fp32 partial plus (max, sum) that a merge kernel combines.
+//   softmax warps  one thread per query row.  S = Q.K^T arrives in tensor memory; the thread takes
+//                  its row into registers, applies scale, tree mask and a lazily rescaled running
+//                  maximum, and writes P as bf16 back into tensor memory over the scores.
+//   K, V warps     stream 128-key tiles (TMA, 128-byte swizzled) through a ring of stages each.
+//   MMA warp       issues tcgen05.mma: S = Q.K^T (operands in shared memory) and O += P.V (P from
+//                  tensor memory, V in shared memory, MN-major), two score slots in flight so that
+//                  the tensor pipe and the softmax warps overlap.
+// What bounds a block: the chain scores -> probabilities -> P.V -> next scores of a slot (0.9 us for 128 x 128
+// with both slots busy: 1.75 us per tile of 128 keys x 256 rows, where the tensor pipe alone needs 1.06 us, the
+// exponentials 1.04 us and the K/V tile's 64 KB 1.5 us).  It was 2.3 us with sixteen softmax warps that read the
+// scores twice and exchanged half rows' maxima, and MMAs issued by a diverged lane (92 instead of 55 cycles each).
+// The block writes final rows when it serves its sequence alone; otherwise the blocks of a cluster combine
+// their rows among themselves, or partial rows go to L2 and are combined by a merge kernel or by the last
+// block to finish.
 //
 // Every wait on an mbarrier is bounded: when it runs out the block raises EAGLE2_STATUS_TIMEOUT,
 // drains its own copies, frees its tensor memory and returns.
@@ -34,9 +39,25 @@ constexpr int kRowsPerTile = 128;     // M of every tcgen05.mma
 constexpr int kMaxTilesPerSplit = 16; // sequences that would need longer blocks are served longest first (batches)
 constexpr int kMaxTilesPerSplitOrdered = 64;  // a block never streams more than 8192 keys
 constexpr int kTmemCols = 512;
+constexpr int kMaxCluster = 8;
 constexpr int kSlots = 2;             // score slots in tensor memory
-constexpr int kSoftmaxThreads = 512;  // 16 softmax warps: four per SM sub-partition
-constexpr int kAttnThreads = kSoftmaxThreads + 64;  // ... the TMA warp, the MMA warp
+constexpr int kSoftmaxThreads = 256;  // 8 softmax warps: two per SM sub-partition, one of each group
+constexpr int kAttnThreads = kSoftmaxThreads + 96;  // ... the warps that request K (and Q), issue MMAs, request V
+
+// Division of 31-bit numbers by a launch constant: a multiplication and a shift instead of the ~100 dependent
+// cycles of a run-time division (a block works out its place with half a dozen of them before its first request).
+struct FastDiv {
+    uint32_t d, mul, shift;
+    FastDiv() = default;
+    explicit FastDiv(int by) : d((uint32_t)by), shift(0) {
+        while ((1u << shift) < d) ++shift;
+        mul = (uint32_t)((((1ull << shift) - d) << 32) / d + 1);
+    }
+#ifdef __CUDACC__
+    __device__ __forceinline__ int div(int n) const { return (int)((__umulhi((uint32_t)n, mul) + (uint32_t)n) >> shift); }
+    __device__ __forceinline__ int mod(int n) const { return n - div(n) * (int)d; }
+#endif
+};
 
 struct AttnPlan {
     int g, M;
@@ -56,13 +77,67 @@ struct AttnPlan {
     int ordered;    // 1: a small kernel first lists the (sequence, split) items that have tiles, longest
                     // first, and blocks take their item from that list (ragged batches: the last wave
                     // is then made of the shortest blocks, and idle splits cost nothing)
+    int cluster;    // > 1: the blocks of a (sequence, KV head, row block) form a cluster, share out the sequence's
+                    // tiles evenly and combine their partial rows through distributed shared memory
+    int own;        // cluster launches: packed rows that each block of the cluster combines (even)
     int fused_merge;  // 1 (ordered launches with several splits): the last block of a (sequence, KV head, row
                       // block) to finish combines the splits' partials itself, while other blocks still run
+    int tile_tok;   // query rows by TMA: tree tokens per 128-row tile
+    FastDiv by_g, by_splits, by_n_rb, by_hkv, by_per_split;
     size_t smem;
     long long wait_limit;  // bound of every device-side wait of the launch, in clock cycles
 };
 
-static void attention_plan(int B, int m, int Hq, int Hkv, int d, int max_kv_len, AttnPlan* p) {
+// Clusters of `size` attention blocks (one block per SM) that the device holds at once.  It depends on how
+// many SMs each of a GPU's processing clusters has, which differs from one GPU to the next.
+static int resident_clusters(int size);
+
+static void ring_of(AttnPlan* p, int d) {
+    const size_t unit = (size_t)(d / 64) * kTK * 128;  // one 128-row operand tile
+    int stages = (int)((220 * 1024 - p->mt * unit) / (2 * unit));
+    p->stages = stages > 4 ? 4 : (stages < 2 ? 2 : stages);
+    p->smem = (p->mt + 2 * (size_t)p->stages) * unit + 1024;
+}
+
+// Launches that the device holds at once with every (sequence, KV head, row block) on one block or one cluster of
+// blocks: which way is cheapest, by the items (128 rows x 128 keys) that one block goes through.  Combining a
+// cluster's partial rows costs about as much as two of them and, for 128 rows, one and a half more (measured: four
+// tiles of 128 rows are quicker on one block, 9.0 against 9.7 us per layer, of 40 rows on four blocks, 7.2 against
+// 8.2 us), so sequences of a few tiles stay on one block each.  Row blocks of 128 rows read the K/V tiles once more than those of 256, from L2, and give twice
+// the blocks.  Launches whose blocks would be long are left to the plans below, which put more SMs to work.
+// (Measured against partial rows and a merge launch, per layer: B = 1, 1024 keys, 8 KV heads of 4 query heads
+// 11.8 -> 10.5 us, 4096 keys 15.5 -> 14.8 us, 32 KV heads, 1024 keys 12.4 -> 12.0 us.)
+constexpr double kMaxItemsPerBlock = 24.0;
+static bool single_wave_plan(int B, int m, int Hkv, int d, int tiles, AttnPlan* p) {
+    const long long groups = (long long)B * Hkv;
+    int best_c = 0, best_tok = 0;
+    double best = kMaxItemsPerBlock + 3.5;
+    for (int mt = 1; mt <= 2; ++mt) {
+        const int tok_max = mt * kRowsPerTile / p->g, n_rb = (m + tok_max - 1) / tok_max, per_tok = (m + n_rb - 1) / n_rb;
+        if ((per_tok * p->g > kRowsPerTile) != (mt == 2)) continue;
+        for (int c = 1; c <= kMaxCluster && c <= tiles; ++c) {
+            if (groups * n_rb > (c == 1 ? sm_count() : resident_clusters(c))) continue;
+            const double cost = (double)((tiles + c - 1) / c) * mt + (c > 1 ? 2.0 + 1.5 * per_tok * p->g / kRowsPerTile : 0.0);
+            if (cost < best) best = cost, best_c = c, best_tok = per_tok;
+        }
+    }
+    if (!best_c) return false;
+    p->cluster = best_c;
+    p->per_tok = best_tok;
+    p->per = best_tok * p->g;
+    p->n_rb = (m + best_tok - 1) / best_tok;
+    p->mt = p->per > kRowsPerTile ? 2 : 1;
+    p->own = ((p->per + best_c - 1) / best_c + 1) / 2 * 2;
+    p->splits = best_c;
+    p->per_split = (tiles + best_c - 1) / best_c;
+    p->pair = p->ordered = p->fused_merge = 0;
+    p->wait_limit = wait_limit_cycles();
+    p->setup_first = B == 1;
+    ring_of(p, d);
+    return true;
+}
+
+static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_kv_len, AttnPlan* p) {
     p->g = Hq / Hkv;
     p->M = m * p->g;
     // A block holds at most 256 packed rows, i.e. at most 256/g whole tokens (g need not divide 256).
@@ -82,6 +157,8 @@ static void attention_plan(int B, int m, int Hq, int Hkv, int d, int max_kv_len,
     // against 8 per single block: 35.6 against 34.2 us; LLaMA3-8B-shaped layer, 4 against 2: 18.5
     // against 19.7 us).
     const int tiles = (max_kv_len + m + kTK - 1) / kTK;
+    p->cluster = 1, p->own = 0;
+    if (single_wave_plan(B, m, Hkv, d, tiles, p)) return;
     p->pair = (p->mt == 2 && p->q_tma && d == 128 && items * 2 <= tpcs &&
                (tiles + tpcs / items - 1) / (tpcs / items) <= 8) ? 1 : 0;
     long long s = (p->pair ? tpcs : sms) / (items > 0 ? items : 1);
@@ -118,16 +195,21 @@ static void attention_plan(int B, int m, int Hq, int Hkv, int d, int max_kv_len,
     p->per_split = per_split;
     p->splits = (tiles + per_split - 1) / per_split;
     p->fused_merge = (p->ordered && p->splits > 1) ? 1 : 0;
-    const size_t unit = (size_t)(d / 64) * kTK * 128;  // one 128-row operand tile
-    int stages = (int)((220 * 1024 - p->mt * unit) / (2 * unit));
-    p->stages = stages > 4 ? 4 : (stages < 2 ? 2 : stages);
-    p->smem = (p->mt + 2 * (size_t)p->stages) * unit + 1024;
+    ring_of(p, d);
     p->wait_limit = wait_limit_cycles();
     p->setup_first = B == 1;  // ragged batches leave many splits without tiles: those leave at once
     if (p->pair) {  // per block: one 128-row query tile, half-size K and V stages
+        const size_t unit = (size_t)(d / 64) * kTK * 128;
         p->stages = p->ordered ? 5 : 4;
         p->smem = unit + (size_t)p->stages * unit + 1024;
     }
+}
+
+static void attention_plan(int B, int m, int Hq, int Hkv, int d, int max_kv_len, AttnPlan* p) {
+    attention_plan_sizes(B, m, Hq, Hkv, d, max_kv_len, p);
+    p->by_g = FastDiv(p->g), p->by_splits = FastDiv(p->splits), p->by_n_rb = FastDiv(p->n_rb), p->by_hkv = FastDiv(Hkv);
+    p->by_per_split = FastDiv(p->per_split);
+    p->tile_tok = kRowsPerTile / p->g;
 }
 
 struct AttnWs {
@@ -138,7 +220,7 @@ struct AttnWs {
 };
 
 static size_t attention_ws_layout(int B, int Hkv, int d, const AttnPlan& p, void* base, AttnWs* w) {
-    if (p.splits == 1 && !p.ordered) return 0;
+    if (p.cluster > 1 || (p.splits == 1 && !p.ordered)) return 0;
     // every operation keeps its arrival counters (B ints) at the start of the workspace and leaves
     // them zero; everything else goes behind that region so that a shared workspace stays valid
     size_t off = round_up(sizeof(int) * (size_t)B, kWsAlign);
@@ -215,45 +297,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-// Largest raw score of a 32-column chunk (TAIL: only over the columns whose visibility bit is set).
-template <bool TAIL>
-__device__ __forceinline__ float chunk_rowmax(const uint32_t (&r)[32], uint32_t visw, float mx) {
-    float m0 = mx, m1 = -INFINITY;
-#pragma unroll
-    for (int c = 0; c < 32; c += 4) {
-        float a[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            a[e] = __uint_as_float(r[c + e]);
-            if (TAIL && !((visw >> (c + e)) & 1u)) a[e] = -INFINITY;
-        }
-        m0 = max3(m0, a[0], a[1]);
-        m1 = max3(m1, a[2], a[3]);
-    }
-    return fmaxf(m0, m1);
-}
-// p = 2^(s * scale - reference) for a chunk of NC columns, packed to NC/2 bf16 pairs; the sums of the
-// unrounded probabilities accumulate in two packed registers.
-template <bool TAIL, int NC>
-__device__ __forceinline__ void chunk_probs(const uint32_t (&r)[NC], uint32_t visw, float2 scale2, float2 neg_ref2,
-                                            float2& sum_a, float2& sum_b, uint32_t (&pk)[NC / 2]) {
-#pragma unroll
-    for (int c = 0; c < NC; c += 4) {
-        float2 a = __ffma2_rn(make_float2(__uint_as_float(r[c]), __uint_as_float(r[c + 1])), scale2, neg_ref2);
-        float2 bq = __ffma2_rn(make_float2(__uint_as_float(r[c + 2]), __uint_as_float(r[c + 3])), scale2, neg_ref2);
-        if (TAIL) {
-            if (!((visw >> c) & 1u)) a.x = -INFINITY;
-            if (!((visw >> (c + 1)) & 1u)) a.y = -INFINITY;
-            if (!((visw >> (c + 2)) & 1u)) bq.x = -INFINITY;
-            if (!((visw >> (c + 3)) & 1u)) bq.y = -INFINITY;
-        }
-        const float2 pa = make_float2(ex2(a.x), ex2(a.y)), pb = make_float2(ex2(bq.x), ex2(bq.y));
-        sum_a = __fadd2_rn(sum_a, pa);
-        sum_b = __fadd2_rn(sum_b, pb);
-        pk[c >> 1] = pack_bf16_alu(pa.x, pa.y);
-        pk[(c >> 1) + 1] = pack_bf16_alu(pb.x, pb.y);
-    }
-}
 
 // A sequence is served only if its length is within the plan and its rows lie inside the cache.
 __device__ __forceinline__ bool sequence_ok(int L, long long row_base, int m, int max_kv_len, long long cache_rows) {
@@ -264,7 +307,7 @@ constexpr int kMaxStages = 6;  // K/V ring depth the barrier arrays allow
 struct AttnBarriers {
     unsigned long long q_full;
     unsigned long long k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
-    unsigned long long s_full[kSlots], p_full[kSlots];
+    unsigned long long s_full[kSlots], p_first[kSlots], p_full[kSlots];  // scores / first 32 keys' / all probabilities
     // Per accumulator (= score slot = item parity), two barriers used by its alternate uses: the
     // u-th P.V into accumulator e completes a phase of o_done[e][u & 1].  A waiter may skip phases (it only looks when it must rescale O, and at the
     // end); with two barriers the one it consults is never more than one phase ahead of it.
@@ -272,7 +315,9 @@ struct AttnBarriers {
     // pair mode, used in the pair's first block: the other block's query tile / K half / V half
     // has landed (and its V tail is cleared)
     unsigned long long q_peer, k_peer[kMaxStages], v_peer[kMaxStages];
-    unsigned long long v_landed, v_clean;  // the block's last V tile has landed / its rows past the sequence's last key are cleared
+    unsigned long long v_clean;  // the last V tile's rows past the sequence's last key are cleared
+    // cluster launches: every block's query tiles may be overwritten by partial rows / they have arrived here
+    unsigned long long peers_ready, inbox;
     unsigned long long drain;  // after a wait ran out: the tensor instructions issued so far have retired
 };
 
@@ -470,64 +515,81 @@ __device__ __forceinline__ void merge_rows_wide(const AttnPlan& plan, const Attn
     }
 }
 
-template <int DH, int MT, bool PAIR>
+template <int DH, int MT, bool PAIR, bool CL>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map,
                       const __grid_constant__ CUtensorMap q_map, const __nv_bfloat16* __restrict__ q, const int64_t* __restrict__ kv_off,
                       const int32_t* __restrict__ kv_len, const uint64_t* __restrict__ mask_bits, int m, int Hq,
-                      int Hkv, long long cache_rows, int max_kv_len, AttnPlan plan, float scale_log2,
+                      int Hkv, long long cache_rows, int max_kv_len, const __grid_constant__ AttnPlan plan, float scale_log2,
                       __nv_bfloat16* __restrict__ out, float* __restrict__ lse, AttnWs ws, int32_t* d_status) {
     constexpr int HALVES = DH / 64;                    // 64-column (128-byte) panels per operand tile
     constexpr uint32_t kPanel = kTK * 128;             // bytes of one panel: 128 rows x 128 bytes
     constexpr uint32_t kTile = HALVES * kPanel;
-    constexpr int kTmaWarp = kSoftmaxThreads / 32, kMmaWarp = kTmaWarp + 1;
+    constexpr int kTmaWarp = kSoftmaxThreads / 32, kMmaWarp = kTmaWarp + 1, kVWarp = kTmaWarp + 2;
     constexpr uint32_t kIdescQK = instr_desc(kTK, false, PAIR ? 256 : 128);
     constexpr uint32_t kIdescPV = instr_desc(DH, true, PAIR ? 256 : 128);
     constexpr uint32_t kOCol = kSlots * kTK;           // first accumulator column of O
+    constexpr uint32_t kRowBytes = DH * 2;
     // bytes a block holds of one K tile and of one V tile (a pair splits K by keys, V by columns)
     constexpr uint32_t kKPanel = PAIR ? kPanel / 2 : kPanel, kKTile = HALVES * kKPanel;
     constexpr uint32_t kVTile = PAIR ? kPanel : kTile;
+    static_assert(!(PAIR && CL), "a cluster's blocks compute on their own");
     static_assert(!PAIR || (MT == 1 && DH == 128), "a pair block holds one 128-row tile, head_dim 128");
 
     extern __shared__ unsigned char smem_raw[];
     __shared__ AttnBarriers bars;
     __shared__ uint32_t s_tmem_base;
     __shared__ WaitCtl s_ctl;
+    // cluster launches: (reference maximum, sum) of this block's rows, and those that arrived for its share
+    __shared__ __align__(16) float2 s_ml[CL ? MT * 128 : 1], s_ml_in[CL ? MT * 128 + 2 * kMaxCluster : 1];
 
     const int g = plan.g, M = plan.M, S = plan.splits, NST = plan.stages;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // 0: the block that issues the pair's MMAs
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (uniform over the warp, and known to be)
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sQ = smem_base;
     const uint32_t sK = sQ + MT * kTile;
     const uint32_t sV = sK + (uint32_t)NST * kKTile;
     unsigned char* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
 
-    // ---- set-up: barriers, tensor memory (reads nothing an earlier kernel could have written) ----
+    // A launch for one sequence reads the sequence's length and offset before it waits for the
+    // preceding kernel (the two loads then cost nothing after the wait; ~0.6 us per layer).  They are
+    // final by then: the one kernel of this library that writes lengths does not let its dependents
+    // start before it has completed, and a kernel that lets them start has itself waited for its
+    // predecessors to complete.
+    const bool early_len = plan.setup_first && !plan.ordered;
+    int len_early = 0;
+    long long off_early = 0;
+    if (early_len) len_early = kv_len[0], off_early = kv_off[0];
+
+    // ---- set-up: barriers, tensor memory (reads nothing an earlier kernel could have written); a lane per
+    // ring stage, one for the rest ----
     auto set_up = [&]() {
-        if (tid == 0) {
+        if (tid < NST) {
+            mbar_init(smem_u32(&bars.k_full[tid]), 1);
+            mbar_init(smem_u32(&bars.k_empty[tid]), 1);
+            mbar_init(smem_u32(&bars.v_full[tid]), 1);
+            mbar_init(smem_u32(&bars.v_empty[tid]), 1);
+            if (PAIR) mbar_init(smem_u32(&bars.k_peer[tid]), 1), mbar_init(smem_u32(&bars.v_peer[tid]), 1);
+            fence_barrier_init();
+        } else if (tid >= 32 && tid < 34) {
+            const int e = tid & 1;  // score slot = accumulator = group
+            mbar_init(smem_u32(&bars.s_full[e]), 1);
+            const uint32_t warps = (PAIR ? 2 : 1) * (kSoftmaxThreads / 64);  // one arrival per warp of the slot's group
+            mbar_init(smem_u32(&bars.p_first[e]), warps);
+            mbar_init(smem_u32(&bars.p_full[e]), warps);
+            mbar_init(smem_u32(&bars.o_done[e][0]), 1);
+            mbar_init(smem_u32(&bars.o_done[e][1]), 1);
+            fence_barrier_init();
+        } else if (tid == 64) {
             s_ctl.abort = 0;
             s_ctl.limit = plan.wait_limit;
             mbar_init(smem_u32(&bars.q_full), plan.q_tma ? 1 : kSoftmaxThreads);
-            for (int s = 0; s < kMaxStages; ++s) {
-                mbar_init(smem_u32(&bars.k_full[s]), 1);
-                mbar_init(smem_u32(&bars.k_empty[s]), 1);
-                mbar_init(smem_u32(&bars.v_full[s]), 1);
-                mbar_init(smem_u32(&bars.v_empty[s]), 1);
-            }
-            for (int s = 0; s < kSlots; ++s) {
-                mbar_init(smem_u32(&bars.s_full[s]), 1);
-                mbar_init(smem_u32(&bars.p_full[s]), (PAIR ? 2 : 1) * (kSoftmaxThreads / 64));  // one arrival per warp of the slot's group
-            }
-            mbar_init(smem_u32(&bars.q_peer), 1);
-            for (int s = 0; s < kMaxStages; ++s) {
-                mbar_init(smem_u32(&bars.k_peer[s]), 1);
-                mbar_init(smem_u32(&bars.v_peer[s]), 1);
-            }
-            for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&bars.o_done[s >> 1][s & 1]), 1);
+            if (PAIR) mbar_init(smem_u32(&bars.q_peer), 1);
             mbar_init(smem_u32(&bars.drain), 1);
             mbar_init(smem_u32(&bars.v_clean), 1);
-            mbar_init(smem_u32(&bars.v_landed), 1);
+            if (CL) mbar_init(smem_u32(&bars.peers_ready), plan.cluster), mbar_init(smem_u32(&bars.inbox), 1);
             fence_barrier_init();
         }
         if (warp == kMmaWarp) {
@@ -545,22 +607,10 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             if (plan.q_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&q_map) : "memory");
         }
         tc_fence_before();
-        if (PAIR) cluster_sync_all();  // both blocks' barriers exist before either signals the other
+        if (PAIR || CL) cluster_sync_all();  // all blocks' barriers exist before any signals another
         else __syncthreads();
         tc_fence_after();
     };
-    // A launch for one sequence reads the sequence's length and offset before it waits for the
-    // preceding kernel (the two loads then cost nothing after the wait; ~0.6 us per layer).  They are
-    // final by then: the one kernel of this library that writes lengths does not let its dependents
-    // start before it has completed, and a kernel that lets them start has itself waited for its
-    // predecessors to complete.
-    const bool early_len = plan.setup_first && !plan.ordered;
-    int len_early = 0;
-    long long off_early = 0;
-    if (early_len) {
-        const int b_early = (int)((PAIR ? blockIdx.x >> 1 : blockIdx.x) / (unsigned)(S * plan.n_rb * Hkv));
-        len_early = kv_len[b_early], off_early = kv_off[b_early];
-    }
     if (plan.setup_first) set_up();
     // (such a launch also works out which tiles and rows the block serves before it waits: below)
     if (!early_len) {
@@ -570,21 +620,22 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 
     int bid = PAIR ? blockIdx.x >> 1 : blockIdx.x;
     int split, rb, hk, b;
+    auto take = [](int& n, const FastDiv& by) {  // n -> quotient, returns the remainder
+        const int quot = by.div(n), rem = n - quot * (int)by.d;
+        n = quot;
+        return rem;
+    };
     if (plan.ordered) {  // item-major: the list says which (sequence, split) this block serves
-        rb = bid % plan.n_rb;
-        bid /= plan.n_rb;
-        hk = bid % Hkv;
-        const int item = bid / Hkv;
-        if (item >= (int)ws.order[0]) return;  // (ordered launches set up after this point)
-        const uint32_t packed = ws.order[1 + item];
-        b = (int)(packed / (uint32_t)S), split = (int)(packed % (uint32_t)S);
+        rb = take(bid, plan.by_n_rb);
+        hk = take(bid, plan.by_hkv);
+        if (bid >= (int)ws.order[0]) return;  // (ordered launches set up after this point)
+        b = (int)ws.order[1 + bid];
+        split = take(b, plan.by_splits);
     } else {
-        split = bid % S;
-        bid /= S;
-        rb = bid % plan.n_rb;
-        bid /= plan.n_rb;
-        hk = bid % Hkv;
-        b = bid / Hkv;
+        split = take(bid, plan.by_splits);
+        rb = take(bid, plan.by_n_rb);
+        hk = take(bid, plan.by_hkv);
+        b = bid;
     }
 
     const int L_raw = early_len ? len_early : kv_len[b];
@@ -593,10 +644,12 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     const int L = overflow ? 0 : L_raw;
     const int n_keys = L + m;
     const int tiles = (n_keys + kTK - 1) / kTK;
-    const int S_b = (tiles + plan.per_split - 1) / plan.per_split;  // splits this sequence uses
-    const int t_begin = min(split * plan.per_split, tiles);
-    const int nt = overflow ? 0 : min(plan.per_split, tiles - t_begin);
-    const bool direct = S_b <= 1;  // a single split writes final rows
+    // splits this sequence uses (a cluster shares a sequence's tiles out evenly; otherwise blocks have equal
+    // shares of the longest)
+    const int S_b = CL ? min(tiles, S) : plan.by_per_split.div(tiles + plan.per_split - 1);
+    const int t_begin = CL ? plan.by_splits.div(tiles * split) : min(split * plan.per_split, tiles);
+    const int nt = overflow ? 0 : CL ? plan.by_splits.div(tiles * (split + 1)) - t_begin : min(plan.per_split, tiles - t_begin);
+    const bool direct = !CL && S_b <= 1;  // a single split writes final rows
 
     // first packed row of this block and the rows that exist in it (the second block of a pair may
     // hold none: it still serves its halves of K and V)
@@ -616,19 +669,32 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         chain_release();
     }
     if (!plan.setup_first) {
-        if (!active) return;
+        if (CL ? overflow : !active) return;  // (all blocks of a cluster leave or stay together)
         set_up();
     }
     const uint32_t tmem = s_tmem_base;
     volatile WaitCtl* abort_flag = &s_ctl;
+    // Cluster launches: block j combines the rows [j * own, (j + 1) * own) of the row block; rows_of(j) of
+    // them exist (to the next even number: row pairs travel together).
+    auto rows_of = [&](int j) { return min(max(((rows_blk + 1) & ~1) - j * plan.own, 0), plan.own); };
+    if (CL && tid == 0 && !overflow) mbar_expect_tx(smem_u32(&bars.inbox), (uint32_t)(S_b * rows_of(split)) * (kRowBytes + 8));
+    bool softmax_ok = true;
     int k_issued = 0, v_issued = 0;  // TMA lane: K and V tiles requested so far
     const int n_items = nt * MT;  // item i = (tile i / MT, row tile i % MT), score slot i % 2
+    // The only tile of this block that can reach past the sequence's last key is its last one.  Its P.V covers
+    // the 16-key groups that hold a key; rows of the last such group that lie past the last key hold whatever
+    // follows the sequence in the cache and are cleared, so that a zero probability times a non-finite value
+    // cannot reach O.
+    const int jt = nt - 1;
+    const int valid_t = min(n_keys - (t_begin + jt) * kTK, kTK);  // keys that exist in the last tile
+    const int groups_t = (valid_t + 15) >> 4;                     // 16-key groups that hold one
+    const bool has_tail = (valid_t & 15) != 0;
 
     if (active) {
     if (warp == kTmaWarp) {
-        // ===== TMA producer =======================================================================
+        // ===== producer of Q and K tiles (V has its own: a K stage is free long before the V stage of the
+        // same tile, and one lane that serves both in order would leave it empty meanwhile) ==========
         if (lane == 0) {
-            bool ok = true;
             if (plan.q_tma) {
                 mbar_expect_tx(smem_u32(&bars.q_full), MT * kTile);
 #pragma unroll
@@ -636,22 +702,32 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 #pragma unroll
                     for (int h = 0; h < HALVES; ++h)
                         tma_load_4d(sQ + t * kTile + h * kPanel, &q_map, h * 64, 0,
-                                    b * m + rb * plan.per_tok + (t + (int)rank) * (kRowsPerTile / g), hk,
+                                    b * m + rb * plan.per_tok + (t + (int)rank) * (int)plan.tile_tok, hk,
                                     smem_u32(&bars.q_full));
             }
-            for (int j = 0; j < nt && ok; ++j) {
-                const int st = j % NST;
-                const uint32_t ph = (uint32_t)((j / NST) & 1);
-                const int row = (int)(row_base + (long long)(t_begin + j) * kTK);
-                if (j >= NST) ok = mbar_wait(smem_u32(&bars.k_empty[st]), ph ^ 1u, abort_flag);
-                if (!ok) break;
+            int st = 0, row = (int)(row_base + (long long)t_begin * kTK);
+            uint32_t ph = 1;
+            for (int j = 0; j < nt; ++j, row += kTK) {
+                if (j >= NST && !mbar_wait(smem_u32(&bars.k_empty[st]), ph, abort_flag)) break;
                 mbar_expect_tx(smem_u32(&bars.k_full[st]), kKTile);
 #pragma unroll
                 for (int h = 0; h < HALVES; ++h)  // a pair block takes its 64 of the tile's 128 keys
                     tma_load_3d(sK + st * kKTile + h * kKPanel, &k_map, h * 64, hk, row + (int)rank * (kTK / 2),
                                 smem_u32(&bars.k_full[st]));
                 k_issued = j + 1;
-                if (j >= NST) ok = mbar_wait(smem_u32(&bars.v_empty[st]), ph ^ 1u, abort_flag);
+                if (++st == NST) st = 0, ph ^= 1u;
+            }
+        }
+        __syncwarp();
+    } else if (warp == kVWarp) {
+        // ===== producer of V tiles ================================================================
+        bool ok = true;
+        int st = 0, last_st = 0;
+        uint32_t ph = 1, last_ph = 1;
+        if (lane == 0) {
+            int row = (int)(row_base + (long long)t_begin * kTK);
+            for (int j = 0; j < nt; ++j, row += kTK) {
+                if (j >= NST) ok = mbar_wait(smem_u32(&bars.v_empty[st]), ph, abort_flag);
                 if (!ok) break;
                 mbar_expect_tx(smem_u32(&bars.v_full[st]), kVTile);
                 if (PAIR) {  // all keys, this block's 64 of the 128 columns
@@ -662,87 +738,81 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                         tma_load_3d(sV + st * kTile + h * kPanel, &v_map, h * 64, hk, row, smem_u32(&bars.v_full[st]));
                 }
                 v_issued = j + 1;
+                last_st = st, last_ph = ph ^ 1u;
+                if (++st == NST) st = 0, ph ^= 1u;
+            }
+        }
+        ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+        if (has_tail && ok) {
+            // (every earlier use of the last V tile's stage is over: its barrier can be waited for directly)
+            last_st = __shfl_sync(0xffffffffu, last_st, 0), last_ph = __shfl_sync(0xffffffffu, last_ph, 0);
+            if (mbar_wait(smem_u32(&bars.v_full[last_st]), last_ph, abort_flag)) {
+                constexpr int PANELS = PAIR ? 1 : HALVES;
+                const int chunks = (groups_t * 16 - valid_t) * 8;
+                for (int idx = lane; idx < chunks; idx += 32)
+#pragma unroll
+                    for (int h = 0; h < PANELS; ++h)
+                        *reinterpret_cast<uint4*>(smem_gen + (sV - smem_base) + last_st * kVTile + h * kPanel +
+                                                  (valid_t + (idx >> 3)) * 128 + (idx & 7) * 16) = make_uint4(0, 0, 0, 0);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bars.v_clean));
             }
         }
     } else if (warp == kMmaWarp) {
-        // ===== MMA issuer: lane 0 alone walks the tiles, waits and issues; nothing in its loop
-        // involves the other lanes (a hand-off through the whole warp cost more than the eight
-        // instructions it guards).  The other lanes have one job: the only tile of this block that can
-        // reach past the sequence's last key is its last one, and rows past that key hold whatever
-        // follows the sequence in the cache.  Lane 0 tells them when that V tile has landed (it follows
-        // the ring's barriers phase by phase; a late joiner could not tell one use of a stage from the
-        // next), they clear those rows in this block's V tile, so that a zero probability times a
-        // non-finite value cannot reach O, and tell lane 0.
-        const int jt = nt - 1;                                  // the block's last tile
-        const int valid_t = n_keys - (t_begin + jt) * kTK;      // keys that exist in it
-        const bool has_tail = valid_t < kTK;
-        if (lane != 0) {
-            if (has_tail) {
-                const int st = jt % NST;
-                if (mbar_wait(smem_u32(&bars.v_landed), 0, abort_flag)) {
-                    constexpr int PANELS = PAIR ? 1 : HALVES;
-                    const int chunks = (kTK - valid_t) * 8;
-                    for (int idx = lane - 1; idx < chunks * PANELS; idx += 31) {
-                        const int h = idx / chunks, rem = idx % chunks;
-                        const int r = valid_t + rem / 8, c = rem % 8;
-                        *reinterpret_cast<uint4*>(smem_gen + (sV - smem_base) + st * kVTile + h * kPanel + r * 128 +
-                                                  c * 16) = make_uint4(0, 0, 0, 0);
-                    }
-                    fence_proxy_async();
-                    __syncwarp(0xfffffffeu);
-                    if (lane == 1) mbar_arrive(smem_u32(&bars.v_clean));
-                }
+        // ===== MMA issuer: the whole warp walks the tiles and waits, one elected lane issues.  The loop's
+        // values are the same in all lanes, so that descriptors and addresses stay in uniform registers,
+        // where the instruction wants them (a lane on its own moves them there one by one: ~90 cycles per
+        // instruction beside busy softmax warps, which is slower than the tensor pipe).
+        auto wait1 = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait_spin(bar, parity, abort_flag)) != 0; };
+        auto here1 = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test_wait(bar, parity)) != 0; };
+        bool ok = wait1(smem_u32(&bars.q_full), 0);
+        if (PAIR && rank != 0) {
+            // The second block of a pair issues no MMA: this warp tells the first block when this
+            // block's query tile, K half and V half are in place.
+            if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.q_peer), 0);
+            int st = 0;
+            uint32_t ph = 0;
+            for (int j = 0; j < nt && ok; ++j) {
+                ok = wait1(smem_u32(&bars.k_full[st]), ph);
+                if (!ok) break;
+                if (lane == 0) mbar_arrive_in(smem_u32(&bars.k_peer[st]), 0);
+                ok = wait1(smem_u32(&bars.v_full[st]), ph);
+                if (ok && has_tail && j == jt) ok = wait1(smem_u32(&bars.v_clean), 0);
+                if (!ok) break;
+                if (lane == 0) mbar_arrive_in(smem_u32(&bars.v_peer[st]), 0);
+                if (++st == NST) st = 0, ph ^= 1u;
             }
         } else {
-            auto wait1 = [&](uint32_t bar, uint32_t parity) { return mbar_wait_spin(bar, parity, abort_flag); };
-            bool ok = wait1(smem_u32(&bars.q_full), 0);
-            if (PAIR && rank != 0) {
-                // The second block of a pair issues no MMA: this lane tells the first block when this
-                // block's query tile, K half and V half are in place.
-                if (ok) mbar_arrive_in(smem_u32(&bars.q_peer), 0);
-                int st = 0;
-                uint32_t ph = 0;
-                for (int j = 0; j < nt && ok; ++j) {
-                    ok = wait1(smem_u32(&bars.k_full[st]), ph);
-                    if (!ok) break;
-                    mbar_arrive_in(smem_u32(&bars.k_peer[st]), 0);
-                    ok = wait1(smem_u32(&bars.v_full[st]), ph);
-                    if (ok && has_tail && j == jt) {
-                        mbar_arrive(smem_u32(&bars.v_landed));
-                        ok = wait1(smem_u32(&bars.v_clean), 0);
-                    }
-                    if (!ok) break;
-                    mbar_arrive_in(smem_u32(&bars.v_peer[st]), 0);
-                    if (++st == NST) st = 0, ph ^= 1u;
+            if (PAIR) ok = ok && wait1(smem_u32(&bars.q_peer), 0);
+            auto commit = [&](uint32_t bar) {
+                if (PAIR) tc_commit2(bar);
+                else tc_commit(bar);
+            };
+            // Descriptor words of the three operand layouts (low word: address and leading offset
+            // in 16-byte units; high word: the layout's constants).
+            constexpr int CG = PAIR ? 2 : 1;
+            const uint64_t qd_first = smem_desc(sQ, 16), kd_first = smem_desc(sK, 16), vd_first = smem_desc(sV, kPanel);
+            const uint32_t q_lo0 = (uint32_t)qd_first, k_lo0 = (uint32_t)kd_first, v_lo0 = (uint32_t)vd_first;
+            const uint32_t qk_hi = (uint32_t)(qd_first >> 32), v_hi = (uint32_t)(vd_first >> 32);
+            int k_st = 0, v_st = 0;        // ring stage of the K tile the next Q.K^T reads, of the V tile the next P.V reads
+            uint32_t k_ph = 0, v_ph = 0;   // and the phases of their barriers
+            // the K tile of item i has landed (both halves of a pair); LOOK: is it there already?
+            auto wait_qk = [&](int i) {
+                if ((i & (MT - 1)) == 0) {
+                    ok = ok && wait1(smem_u32(&bars.k_full[k_st]), k_ph);
+                    if (PAIR) ok = ok && wait1(smem_u32(&bars.k_peer[k_st]), k_ph);
                 }
-            } else {
-                if (PAIR) ok = ok && wait1(smem_u32(&bars.q_peer), 0);
-                auto commit = [&](uint32_t bar) {
-                    if (PAIR) tc_commit2(bar);
-                    else tc_commit(bar);
-                };
-                // Descriptor words of the three operand layouts (low word: address and leading offset
-                // in 16-byte units; high word: the layout's constants).
-                constexpr int CG = PAIR ? 2 : 1;
-                const uint64_t qd_first = smem_desc(sQ, 16), kd_first = smem_desc(sK, 16), vd_first = smem_desc(sV, kPanel);
-                const uint32_t q_lo0 = (uint32_t)qd_first, k_lo0 = (uint32_t)kd_first, v_lo0 = (uint32_t)vd_first;
-                const uint32_t qk_hi = (uint32_t)(qd_first >> 32), v_hi = (uint32_t)(vd_first >> 32);
-                int k_st = 0, v_st = 0;        // ring stage of the K tile the next Q.K^T reads, of the V tile the next P.V reads
-                uint32_t k_ph = 0, v_ph = 0;   // and the phases of their barriers
-                // Waits and issues are separate steps: the loop below first makes sure that everything
-                // the next sixteen instructions read is in place, then issues them back to back (the
-                // lane's own instructions between two groups of eight - waits, commits, address
-                // arithmetic - otherwise leave the tensor pipe idle for ~0.2 us each time).
-                auto wait_qk = [&](int i) {   // the K tile of item i has landed (both halves of a pair)
-                    if ((i & (MT - 1)) == 0) {
-                        ok = ok && wait1(smem_u32(&bars.k_full[k_st]), k_ph);
-                        if (PAIR) ok = ok && wait1(smem_u32(&bars.k_peer[k_st]), k_ph);
-                    }
-                };
-                auto issue_qk = [&](int i) {  // S[slot] = Q[row tile] . K[tile]^T
-                    const int t = i & (MT - 1);
-                    const uint32_t d_tmem = tmem + (uint32_t)(i & 1) * kTK;
-                    const uint32_t q_lo = q_lo0 + (uint32_t)t * (kTile >> 4), k_lo = k_lo0 + (uint32_t)k_st * (kKTile >> 4);
+            };
+            auto look_qk = [&](int i) {
+                if ((i & (MT - 1)) != 0) return true;
+                return here1(smem_u32(&bars.k_full[k_st]), k_ph) && (!PAIR || here1(smem_u32(&bars.k_peer[k_st]), k_ph));
+            };
+            auto issue_qk = [&](int i) {  // S[slot] = Q[row tile] . K[tile]^T
+                const int t = i & (MT - 1);
+                const uint32_t d_tmem = tmem + (uint32_t)(i & 1) * kTK;
+                const uint32_t q_lo = q_lo0 + (uint32_t)t * (kTile >> 4), k_lo = k_lo0 + (uint32_t)k_st * (kKTile >> 4);
+                if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < DH / 16; ++ks) {
                         const uint32_t qo = ((uint32_t)(ks / 4) * kPanel + (uint32_t)(ks % 4) * 32u) >> 4;
@@ -751,96 +821,106 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                         else umma_ss<CG, 1>(d_tmem, q_lo + qo, qk_hi, k_lo + ko, qk_hi, kIdescQK);
                     }
                     commit(smem_u32(&bars.s_full[i & 1]));
-                    if (t == MT - 1) {
-                        commit(smem_u32(&bars.k_empty[k_st]));
-                        if (++k_st == NST) k_st = 0, k_ph ^= 1u;
-                    }
-                };
-                auto wait_pv = [&](int i) {   // the V tile of item i has landed, its probabilities are written
-                    const int t = i & (MT - 1), j = MT == 1 ? i : (i >> 1);
-                    if (t == 0) {
-                        ok = ok && wait1(smem_u32(&bars.v_full[v_st]), v_ph);
-                        if (ok && has_tail && j == jt) {
-                            mbar_arrive(smem_u32(&bars.v_landed));
-                            ok = wait1(smem_u32(&bars.v_clean), 0);
-                        }
-                        if (PAIR) ok = ok && wait1(smem_u32(&bars.v_peer[v_st]), v_ph);
-                    }
-                    ok = ok && wait1(smem_u32(&bars.p_full[i & 1]), (uint32_t)((i >> 1) & 1));
-                };
-                auto issue_pv = [&](int i) {  // O[row tile] += P[slot] . V[tile]
-                    const int t = i & (MT - 1);
-                    const uint32_t d_tmem = tmem + kOCol + (uint32_t)(i & 1) * DH;  // accumulator = slot = item parity
-                    const uint32_t a_tmem = tmem + (uint32_t)(i & 1) * kTK;
-                    const uint32_t v_lo = v_lo0 + (uint32_t)v_st * (kVTile >> 4);
+                    if (t == MT - 1) commit(smem_u32(&bars.k_empty[k_st]));
+                }
+                __syncwarp();
+                if (t == MT - 1 && ++k_st == NST) k_st = 0, k_ph ^= 1u;
+            };
+            auto wait_pv = [&](int i) {   // the V tile of item i has landed, its first probabilities are written
+                const int t = i & (MT - 1), j = MT == 1 ? i : (i >> 1);
+                if (t == 0) {
+                    ok = ok && wait1(smem_u32(&bars.v_full[v_st]), v_ph);
+                    if (has_tail && j == jt) ok = ok && wait1(smem_u32(&bars.v_clean), 0);
+                    if (PAIR) ok = ok && wait1(smem_u32(&bars.v_peer[v_st]), v_ph);
+                }
+                ok = ok && wait1(smem_u32(&bars.p_first[i & 1]), (uint32_t)((i >> 1) & 1));
+            };
+            auto issue_pv = [&](int i) {  // O[row tile] += P[slot] . V[tile]
+                const int t = i & (MT - 1), j = MT == 1 ? i : (i >> 1);
+                const uint32_t d_tmem = tmem + kOCol + (uint32_t)(i & 1) * DH;  // accumulator = slot = item parity
+                const uint32_t a_tmem = tmem + (uint32_t)(i & 1) * kTK;
+                const uint32_t v_lo = v_lo0 + (uint32_t)v_st * (kVTile >> 4);
+                const int n_ks = j == jt ? groups_t : kTK / 16;
+                auto steps = [&](auto from, auto to) {
 #pragma unroll
-                    for (int ks = 0; ks < kTK / 16; ++ks) {
+                    for (int ks = decltype(from)::value; ks < decltype(to)::value; ++ks) {
                         const uint32_t vo = (uint32_t)ks * (2048u >> 4);
                         if (ks == 0) umma_ts<CG, 2>(d_tmem, a_tmem, v_lo, v_hi, kIdescPV, i >= 2 ? 1u : 0u);
-                        else umma_ts<CG, 1>(d_tmem, a_tmem + ks * 16, v_lo + vo, v_hi, kIdescPV);
-                    }
-                    commit(smem_u32(&bars.o_done[i & 1][(i >> 1) & 1]));
-                    if (t == MT - 1) {
-                        commit(smem_u32(&bars.v_empty[v_st]));
-                        if (++v_st == NST) v_st = 0, v_ph ^= 1u;
+                        else if (ks < n_ks) umma_ts<CG, 1>(d_tmem, a_tmem + ks * 8, v_lo + vo, v_hi, kIdescPV);
                     }
                 };
-                static_assert(kSlots == 2, "slot = item & 1");
-                for (int i = 0; i < kSlots && i < n_items && ok; ++i) {
-                    wait_qk(i);
+                if (elect_one()) steps(std::integral_constant<int, 0>{}, std::integral_constant<int, 2>{});
+                __syncwarp();
+                ok = wait1(smem_u32(&bars.p_full[i & 1]), (uint32_t)((i >> 1) & 1));
+                if (!ok) return;
+                tc_fence_after();
+                if (elect_one()) {
+                    steps(std::integral_constant<int, 2>{}, std::integral_constant<int, kTK / 16>{});
+                    commit(smem_u32(&bars.o_done[i & 1][(i >> 1) & 1]));
+                    if (t == MT - 1) commit(smem_u32(&bars.v_empty[v_st]));
+                }
+                __syncwarp();
+                if (t == MT - 1 && ++v_st == NST) v_st = 0, v_ph ^= 1u;
+            };
+            static_assert(kSlots == 2, "slot = item & 1");
+            for (int i = 0; i < kSlots && i < n_items && ok; ++i) {
+                wait_qk(i);
+                if (!ok) break;
+                tc_fence_after();
+                issue_qk(i);
+            }
+            for (int i = 0; i < n_items && ok; ++i) {
+                const bool more = i + kSlots < n_items;
+                // With the next K tile at hand both groups of instructions go out back to back; otherwise P.V
+                // does not wait for it.
+                const bool now = more && look_qk(i + kSlots);
+                wait_pv(i);
+                if (!ok) break;
+                tc_fence_after();
+                issue_pv(i);
+                if (!ok) break;
+                if (more && !now) {
+                    wait_qk(i + kSlots);
                     if (!ok) break;
                     tc_fence_after();
-                    issue_qk(i);
                 }
-                for (int i = 0; i < n_items && ok; ++i) {
-                    const bool more = i + kSlots < n_items;
-                    wait_pv(i);
-                    if (more) wait_qk(i + kSlots);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_pv(i);
-                    if (more) issue_qk(i + kSlots);
-                }
+                if (more) issue_qk(i + kSlots);
             }
         }
         __syncwarp();
     } else {
-        // ===== softmax warps: two groups of eight, each serving every other item ====================
-        // A pass over one item (128 rows x 128 keys) is a chain of dependent steps - scores out of
-        // tensor memory, row maximum, exchange, exponentials, probabilities back - and a group of
-        // warps running it is mostly waiting; two groups on different items keep each other's
-        // gaps filled.  Group e serves the items i with i % 2 == e: score slot e and accumulator e.
-        // With two row tiles that is row tile e; with one row tile both groups serve it, each with
-        // its own reference maximum, row sums and accumulator, and the epilogue combines the two.
-        // Inside a group, warp w reads the tensor-memory lanes of its sub-partition, 32 * (w % 4) ..
-        // + 31, and the two warps with the same w % 4 share 32 query rows, taking 64 of the tile's 128
-        // keys each; they exchange their row maxima through shared memory behind a barrier of those 64
-        // threads.  Every thread writes its probabilities over its own scores.
-        __shared__ float s_xmax[2][2][2][128];            // [use parity][group][half][row]: row maxima of the halves
-        __shared__ float s_xsum[2][2][128];               // epilogue: [group][half][row] row sums
-        __shared__ float s_xref[2][128];                  // epilogue, one row tile: [group][row] reference maxima
-        const int grp = warp >> 3, quad = warp & 3, half = (warp >> 2) & 1;
+        // ===== softmax warps: two groups of four, each serving every other item =====================
+        // A pass over one item (128 rows x 128 keys) is a chain of dependent steps - scores out of tensor
+        // memory, row maximum, exponentials, probabilities back - and two groups on different items fill
+        // each other's gaps.  Group e serves the items i with i % 2 == e: score slot e and accumulator e.
+        // With two row tiles that is row tile e; with one row tile both groups serve it, each with its own
+        // reference maximum, row sums and accumulator, and the epilogue combines the two.  A thread owns a
+        // row: its 128 scores stay in registers from the tensor-memory read to the packed probabilities, so
+        // nothing is read twice and no two threads exchange anything.
+        __shared__ float2 s_half[2][128];                 // epilogue, one row tile: [group][row] (reference, sum)
+        const int grp = warp >> 2, quad = warp & 3;
         const int r_tile = (quad << 5) | lane;            // row inside the tile = tensor-memory lane
         const uint32_t lane_sel = (uint32_t)(quad << 5) << 16;
         const int t_own = MT == 2 ? grp : 0;              // row tile this group's items belong to
-        const int W = (m + 63) >> 6;
+        const int r_blk = t_own * 128 + r_tile;           // row inside the row block
         unsigned long long mlo, mhi;
         {
-            const int r_blk = t_own * 128 + r_tile;
+            const int W = (m + 63) >> 6;
             const int pr = r_blk < rows_here ? row0 + r_blk : rb * plan.per;  // packed row = token * g + head in group
-            mlo = mask_bits[((long long)b * m + pr / g) * W];
-            mhi = W > 1 ? mask_bits[((long long)b * m + pr / g) * W + 1] : 0ull;
+            const uint64_t* bits = mask_bits + ((long long)b * m + plan.by_g.div(pr)) * W;
+            mlo = bits[0];
+            mhi = W > 1 ? bits[1] : 0ull;
         }
         if (!plan.q_tma) {
             // query rows into shared memory by hand, 128-byte swizzled (chunk c of row r at
             // c ^ (r & 7)); all copies of a thread are in flight together, absent rows zero-filled
-#pragma unroll
+#pragma unroll 4
             for (int it = 0; it < MT * 128 * (DH / 8) / kSoftmaxThreads; ++it) {
                 const int idx = tid + it * kSoftmaxThreads;
                 const int r = idx / (DH / 8), c = idx % (DH / 8);
                 const bool live = r < rows_here;
-                const int p2 = row0 + (live ? r : 0);
-                const __nv_bfloat16* src = q + (((long long)b * m + p2 / g) * Hq + hk * g + p2 % g) * DH + c * 8;
+                const int p2 = row0 + (live ? r : 0), tok = plan.by_g.div(p2);
+                const __nv_bfloat16* src = q + (((long long)b * m + tok) * Hq + hk * g + (p2 - tok * g)) * DH + c * 8;
                 const int t = r >> 7, rr = r & 127, h = c >> 3, cc = c & 7;
                 cp_async16(sQ + t * kTile + h * kPanel + rr * 128 + ((cc ^ (rr & 7)) << 4), src, live);
             }
@@ -852,97 +932,97 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 
         float m_ref = -INFINITY, l_run = 0.f;
         bool ok = true;
-        const int pair_bar = 2 + grp * 4 + quad;  // named barrier of the two warps that share this thread's rows
-        const uint32_t s_addr = tmem + lane_sel + (uint32_t)grp * kTK + (uint32_t)half * 64;  // this thread's 64 score columns
-        const uint32_t o_acc = tmem + lane_sel + kOCol + (uint32_t)grp * DH;                    // this group's accumulator
+        const uint32_t s_addr = tmem + lane_sel + (uint32_t)grp * kTK;          // this thread's scores
+        const uint32_t o_acc = tmem + lane_sel + kOCol + (uint32_t)grp * DH;    // and its row of the group's accumulator
+        auto release = [&](uint32_t bar) {  // what this warp has written to tensor memory so far may be read
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                if (PAIR) mbar_arrive_in(bar, 0);  // the pair's first block issues P.V
+                else mbar_arrive(bar);
+            }
+        };
         for (int i = grp; i < n_items; i += 2) {
             const int u = i >> 1;                          // the u-th use of this group's slot and accumulator
             const int j = MT == 2 ? u : i;                 // K/V tile of the item
-            ok = ok && mbar_wait(smem_u32(&bars.s_full[grp]), (uint32_t)(u & 1), abort_flag);
+            ok = mbar_wait(smem_u32(&bars.s_full[grp]), (uint32_t)(u & 1), abort_flag);
             ok = __all_sync(0xffffffffu, ok);  // the tensor-memory accesses below need the whole warp
+            if (!ok) break;
+            if (CL && i == n_items - 1 && quad == 0 && lane == 0) {
+                // the block's last Q.K^T has completed: its query tiles may be overwritten
+                for (int r = 0; r < S; ++r) mbar_arrive_in(smem_u32(&bars.peers_ready), (uint32_t)r);
+            }
+            uint32_t sc[4][32];
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + c * 32, sc[c]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tc_wait_ld(sc[c]);
             const int key0 = (t_begin + j) * kTK;
-            const bool tail = key0 + kTK > L;  // the tile holds tree keys or runs past the last key
-            uint32_t vis0 = ~0u, vis1 = ~0u;   // visibility of this thread's keys 0..31 and 32..63
-            if (tail) {
+            if (key0 + kTK > L) {  // the tile holds tree keys or runs past the last key: hide what the row may not see
                 uint32_t vis[4];
                 tile_visibility(mlo, mhi, key0, L, n_keys, vis);
-                vis0 = half ? vis[2] : vis[0];
-                vis1 = half ? vis[3] : vis[1];
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        if (!((vis[c] >> e) & 1u)) sc[c][e] = 0xff800000u;
             }
-            float mx = -INFINITY;
-            if (ok) {
-                // pass 1: the largest raw score of this thread's 64 keys (the scale is positive)
-                uint32_t ba[32];
-                tc_fence_after();
-                tmem_ld32(s_addr, ba);
-                tc_wait_ld(ba);
-                mx = tail ? chunk_rowmax<true>(ba, vis0, mx) : chunk_rowmax<false>(ba, 0, mx);
-                tmem_ld32(s_addr + 32, ba);
-                tc_wait_ld(ba);
-                mx = tail ? chunk_rowmax<true>(ba, vis1, mx) : chunk_rowmax<false>(ba, 0, mx);
-                s_xmax[u & 1][grp][half][r_tile] = mx;
+            // the largest raw score (the scale is positive), in four independent chains
+            float mx4[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                mx4[c] = fmaxf(__uint_as_float(sc[c][0]), __uint_as_float(sc[c][1]));
+#pragma unroll
+                for (int e = 2; e < 32; e += 2) mx4[c] = max3(mx4[c], __uint_as_float(sc[c][e]), __uint_as_float(sc[c][e + 1]));
             }
-            // the halves' maxima meet here (or both warps leave together)
-            ok = named_barrier_and(pair_bar, 64, ok);
-            if (!ok) break;
-            mx = fmaxf(mx, s_xmax[u & 1][grp][half ^ 1][r_tile]) * scale_log2;
+            const float mx = fmaxf(max3(mx4[0], mx4[1], mx4[2]), mx4[3]) * scale_log2;
 
-            // lazily rescaled reference maximum: probabilities stay below 2^8 in between.  The two
-            // threads of a row hold the same reference: they derive it from the same two maxima.
+            // lazily rescaled reference maximum: probabilities stay below 2^8 in between
             const float m_new = fmaxf(m_ref, mx);
             const bool grow = m_new > m_ref + 8.f;
             if (__any_sync(0xffffffffu, grow)) {
                 const float factor = !grow ? 1.f : (m_ref == -INFINITY ? 0.f : ex2(m_ref - m_new));
                 if (grow) m_ref = m_new, l_run *= factor;
-                // the accumulator may be rescaled once the group's previous P.V has finished; this
-                // thread owns half of the row's columns
-                bool waited = true;
-                if (u > 0)
-                    waited = mbar_wait(smem_u32(&bars.o_done[grp][(u - 1) & 1]), (uint32_t)(((u - 1) >> 1) & 1), abort_flag);
-                waited = __all_sync(0xffffffffu, waited);
-                if (!waited) ok = false;  // the other warp learns it at the next barrier
-                if (u > 0 && waited) {
+                if (u > 0) {
+                    // the accumulator may be rescaled once the group's previous P.V has finished
+                    ok = mbar_wait(smem_u32(&bars.o_done[grp][(u - 1) & 1]), (uint32_t)(((u - 1) >> 1) & 1), abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
                     tc_fence_after();
+#pragma unroll 1
+                    for (int c0 = 0; c0 < DH; c0 += 16) {
+                        uint32_t orow[16];
+                        tmem_ld16(o_acc + c0, orow);
+                        tc_wait_ld16(orow);
 #pragma unroll
-                    for (int c0 = 0; c0 < DH / 2; c0 += 32) {
-                        uint32_t orow[32];
-                        tmem_ld32(o_acc + (uint32_t)half * (DH / 2) + c0, orow);
-                        tc_wait_ld(orow);
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * factor);
-                        tmem_st32(o_acc + (uint32_t)half * (DH / 2) + c0, orow);
+                        for (int c = 0; c < 16; ++c) orow[c] = __float_as_uint(__uint_as_float(orow[c]) * factor);
+                        tmem_st16(o_acc + c0, orow);
                     }
                 }
             }
-            // pass 2: P = 2^(s * scale - reference) as bf16.  The scores are read again, 16 keys at a
-            // time, and each 16 keys become 8 packed columns written over the first half of those 16
-            // score columns: no thread ever writes a column another one reads.
+            // P = 2^(s * scale - reference) as bf16, over the first half of the scores' columns
             const float neg_ref = m_ref == -INFINITY ? 0.f : -m_ref;
             const float2 scale2 = make_float2(scale_log2, scale_log2), neg_ref2 = make_float2(neg_ref, neg_ref);
-            float2 sum_a = make_float2(0.f, 0.f), sum_b = make_float2(0.f, 0.f);
+            float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-            for (int c2 = 0; c2 < 2; ++c2) {
-                uint32_t b0[16], b1[16], pk[8];
-                tmem_ld16(s_addr + c2 * 32, b0);
-                tmem_ld16(s_addr + c2 * 32 + 16, b1);
-                tc_wait_ld16(b0);
-                tc_wait_ld16(b1);
-                const uint32_t vw = c2 ? vis1 : vis0;
-                if (tail) chunk_probs<true, 16>(b0, vw, scale2, neg_ref2, sum_a, sum_b, pk);
-                else chunk_probs<false, 16>(b0, 0, scale2, neg_ref2, sum_a, sum_b, pk);
-                tmem_st8(s_addr + c2 * 32, pk);
-                if (tail) chunk_probs<true, 16>(b1, vw >> 16, scale2, neg_ref2, sum_a, sum_b, pk);
-                else chunk_probs<false, 16>(b1, 0, scale2, neg_ref2, sum_a, sum_b, pk);
-                tmem_st8(s_addr + c2 * 32 + 16, pk);
+            for (int c = 0; c < 4; ++c) {
+                uint32_t pk[16];
+#pragma unroll
+                for (int e = 0; e < 32; e += 2) {
+                    float2 a = __ffma2_rn(make_float2(__uint_as_float(sc[c][e]), __uint_as_float(sc[c][e + 1])), scale2, neg_ref2);
+                    a.x = ex2(a.x), a.y = ex2(a.y);
+                    sum[(e >> 1) & 1] = __fadd2_rn(sum[(e >> 1) & 1], a);
+                    pk[e >> 1] = pack_bf16(a.x, a.y);
+                }
+                tmem_st16(s_addr + c * 16, pk);
+                // (P.V starts on the first 32 keys while the others' exponentials are still being taken: the
+                // pass, the products and the next scores form a chain.  2 % per layer; 64 or 96 keys: less.)
+                if (c == 0) release(smem_u32(&bars.p_first[grp]));
             }
-            l_run += (sum_a.x + sum_a.y) + (sum_b.x + sum_b.y);
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();  // every lane's P is in tensor memory: one arrival speaks for the warp
-            if (lane == 0) {
-                if (PAIR) mbar_arrive_in(smem_u32(&bars.p_full[grp]), 0);  // the pair's first block issues P.V
-                else mbar_arrive(smem_u32(&bars.p_full[grp]));
-            }
+            l_run += (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y);
+            release(smem_u32(&bars.p_full[grp]));
         }
 
         // ---- epilogue: O rows leave tensor memory through shared memory, so that the global
@@ -950,92 +1030,158 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         // Q.K^T has completed once the last P.V has.  All softmax threads first agree that none of
         // them gave up.  A group that served no item (a block with a single item) contributes nothing.
         const int n_uses = (n_items - grp + 1) / 2;  // items this group served
-        if (n_uses > 0)
-            ok = ok && mbar_wait(smem_u32(&bars.o_done[grp][(n_uses - 1) & 1]), (uint32_t)(((n_uses - 1) >> 1) & 1), abort_flag);
-        s_xsum[grp][half][r_tile] = l_run;
-        if (half == 0) s_xref[grp][r_tile] = m_ref;
+        if (ok && n_uses > 0)
+            ok = mbar_wait(smem_u32(&bars.o_done[grp][(n_uses - 1) & 1]), (uint32_t)(((n_uses - 1) >> 1) & 1), abort_flag);
+        if (MT == 1) s_half[grp][r_tile] = make_float2(m_ref, l_run);
         ok = named_barrier_and(1, kSoftmaxThreads, ok);
+        softmax_ok = ok;
         if (ok) {
             tc_fence_after();
-            constexpr int NCOL = MT == 2 ? DH / 2 : DH / 4;  // columns of an output row this thread produces
-            constexpr int row_bytes = DH * 2;
-            const int cmask = row_bytes / 16 - 1;
+            constexpr int NCOL = MT == 2 ? DH : DH / 2;  // columns of an output row this thread produces
+            constexpr int cmask = kRowBytes / 16 - 1;
             // a staged row is DH bf16; 16-byte chunk c of row r sits at chunk c ^ (r mod
             // chunks-per-row), which keeps both the row-wise writes and the chunk-wise reads free of
             // bank conflicts
-            const int r_blk = t_own * 128 + r_tile;
             // One row tile: the two groups hold partial results of the same rows under their own
-            // references; each thread combines a quarter of the row's columns.  Two row tiles: the
-            // group's accumulator is the row tile's result and each thread takes half of the columns.
-            const int col0 = MT == 2 ? half * NCOL : (2 * half + grp) * NCOL;
-            float w_own = 1.f, w_oth = 0.f, l_tot, m_tot = m_ref;
-            if (MT == 2) {
-                l_tot = s_xsum[grp][0][r_tile] + s_xsum[grp][1][r_tile];
-            } else {
-                const float m0 = s_xref[0][r_tile], m1 = s_xref[1][r_tile];
-                m_tot = fmaxf(m0, m1);
-                const float w0 = m0 == -INFINITY ? 0.f : ex2(m0 - m_tot), w1 = m1 == -INFINITY ? 0.f : ex2(m1 - m_tot);
-                l_tot = (s_xsum[0][0][r_tile] + s_xsum[0][1][r_tile]) * w0 + (s_xsum[1][0][r_tile] + s_xsum[1][1][r_tile]) * w1;
-                w_own = grp ? w1 : w0, w_oth = grp ? w0 : w1;
-                if (n_items < 2) w_own = grp ? 0.f : w0, w_oth = grp ? w0 : 0.f;  // accumulator 1 was never written
+            // references; each thread combines half of the row's columns.  Two row tiles: the
+            // group's accumulator is the row tile's result.
+            const int col0 = MT == 2 ? 0 : grp * NCOL;
+            float w0 = 1.f, w1 = 0.f, l_tot = l_run, m_tot = m_ref;
+            if (MT == 1) {
+                const float2 h0 = s_half[0][r_tile], h1 = s_half[1][r_tile];
+                m_tot = fmaxf(h0.x, h1.x);
+                w0 = h0.x == -INFINITY ? 0.f : ex2(h0.x - m_tot), w1 = h1.x == -INFINITY ? 0.f : ex2(h1.x - m_tot);
+                l_tot = h0.y * w0 + h1.y * w1;
+                if (n_items < 2) w1 = 0.f;  // accumulator 1 was never written
             }
             // final rows are normalised here; a partial stays unnormalised (the merge divides by the
             // combined sum) and is rounded to bf16 once, like a final row
             const float inv = !direct ? 1.f : (l_tot > 0.f ? 1.f / l_tot : 0.f);
-            unsigned char* srow = smem_gen + t_own * kTile + (size_t)r_tile * row_bytes;
+            w0 *= inv, w1 *= inv;
+            // (a cluster's rows are staged in the V ring, which nothing reads any more: the peers' partial
+            // rows may be arriving where the queries were)
+            unsigned char* srow = smem_gen + (CL ? sV - smem_base : 0u) + (size_t)r_blk * kRowBytes;
+            const uint32_t o_row = tmem + lane_sel + kOCol + (MT == 2 ? (uint32_t)grp * DH : 0u) + (uint32_t)col0;
 #pragma unroll
-            for (int c0 = 0; c0 < NCOL; c0 += 16) {
-                uint32_t oa[16], ob[16];
-                tmem_ld16(o_acc + (uint32_t)(col0 + c0), oa);
-                if (MT == 1) tmem_ld16(tmem + lane_sel + kOCol + (uint32_t)(grp ^ 1) * DH + (uint32_t)(col0 + c0), ob);
-                tc_wait_ld16(oa);
-                if (MT == 1) tc_wait_ld16(ob);
-                float v[16];
+            for (int c0 = 0; c0 < NCOL; c0 += 32) {
+                uint32_t oa[32], ob[32];
+                tmem_ld32(o_row + c0, oa);
+                if (MT == 1) tmem_ld32(o_row + DH + c0, ob);
+                tc_wait_ld(oa);
+                if (MT == 1) tc_wait_ld(ob);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    float x = w_own != 0.f ? __uint_as_float(oa[c]) * w_own : 0.f;
-                    if (MT == 1 && w_oth != 0.f) x += __uint_as_float(ob[c]) * w_oth;
-                    v[c] = MT == 2 ? __uint_as_float(oa[c]) * inv : x * inv;
-                }
+                for (int c = 0; c < 32; c += 8) {
+                    float v[8];
 #pragma unroll
-                for (int c = 0; c < 16; c += 8) {
-                    uint4 pkt;
-                    pkt.x = pack_bf16(v[c + 0], v[c + 1]);
-                    pkt.y = pack_bf16(v[c + 2], v[c + 3]);
-                    pkt.z = pack_bf16(v[c + 4], v[c + 5]);
-                    pkt.w = pack_bf16(v[c + 6], v[c + 7]);
+                    for (int e = 0; e < 8; ++e) {
+                        v[e] = __uint_as_float(oa[c + e]) * w0;
+                        if (MT == 1) {
+                            if (w0 == 0.f) v[e] = 0.f;
+                            if (w1 != 0.f) v[e] = fmaf(__uint_as_float(ob[c + e]), w1, v[e]);
+                        }
+                    }
                     const int chunk = (col0 + c0 + c) >> 3;
-                    *reinterpret_cast<uint4*>(srow + (((chunk ^ r_tile) & cmask) << 4)) = pkt;
+                    *reinterpret_cast<uint4*>(srow + (((chunk ^ r_tile) & cmask) << 4)) =
+                        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
                 }
             }
-            if (r_blk < rows_here && half == 0 && (MT == 2 || grp == 0)) {
-                const int pr = row0 + r_blk;
-                if (direct) {
-                    if (lse) lse[((long long)b * Hq + hk * g + pr % g) * m + pr / g] = (m_tot + log2f(l_tot)) * 0.69314718055994531f;
-                } else {
-                    ws.ml[part_row0 + r_blk] = make_float2(m_tot, l_tot);
+            if (MT == 2 || grp == 0) {
+                if (CL) {
+                    s_ml[r_blk] = make_float2(m_tot, l_tot);
+                } else if (r_blk < rows_here) {
+                    if (!direct) {
+                        ws.ml[part_row0 + r_blk] = make_float2(m_tot, l_tot);
+                    } else if (lse) {
+                        const int pr = row0 + r_blk, tok = plan.by_g.div(pr);
+                        lse[((long long)b * Hq + hk * g + (pr - tok * g)) * m + tok] = (m_tot + log2f(l_tot)) * 0.69314718055994531f;
+                    }
                 }
             }
+            if (CL) fence_proxy_async();  // the copies to the peers read what was staged
             asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");  // rows are staged
-            const int lanes_per_row = row_bytes / 16;       // 16 lanes (8 for a 64-wide bf16 row)
-            const int rows_per_pass = 32 / lanes_per_row;
-            const int sub = lane / lanes_per_row, cl = lane % lanes_per_row;
-            for (int r = warp * rows_per_pass + sub; r < rows_here; r += (kSoftmaxThreads / 32) * rows_per_pass) {
-                const int t = r >> 7, rr = r & 127;
-                const uint4 v = *reinterpret_cast<const uint4*>(smem_gen + t * kTile + (size_t)rr * row_bytes +
-                                                                (((cl ^ rr) & cmask) << 4));
-                if (direct) {
-                    const int p2 = row0 + r;
-                    __nv_bfloat16* dst = out + (((long long)b * m + p2 / g) * Hq + hk * g + p2 % g) * DH;
-                    *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(dst) + cl * 16) = v;
-                } else {
+            if (!CL) {
+                constexpr int lanes_per_row = kRowBytes / 16;       // 16 lanes (8 for a 64-wide bf16 row)
+                constexpr int rows_per_pass = 32 / lanes_per_row;
+                const int sub = lane / lanes_per_row, cl = lane % lanes_per_row;
+#pragma unroll 4
+                for (int r = warp * rows_per_pass + sub; r < rows_here; r += (kSoftmaxThreads / 32) * rows_per_pass) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(smem_gen + (size_t)r * kRowBytes + (((cl ^ r) & cmask) << 4));
                     __nv_bfloat16* dst = ws.o_part + (part_row0 + r) * DH;
+                    if (direct) {
+                        const int p2 = row0 + r, tok = plan.by_g.div(p2);
+                        dst = out + (((long long)b * m + tok) * Hq + hk * g + (p2 - tok * g)) * DH;
+                    }
                     *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(dst) + cl * 16) = v;
                 }
             }
         }
     }
     }  // active
+
+    // ---- cluster launches: every block sends each peer the partial rows that peer combines, as bulk copies from
+    // shared memory to shared memory, and combines its own share when all have arrived.  (The alternative,
+    // partial rows through L2 and a second launch that combines them, costs that launch's start and a cold
+    // pass through its code.)
+    if (CL && !overflow && warp < kTmaWarp) {
+        if (warp == 0) {
+            if (!active) {
+                if (lane < S) mbar_arrive_in(smem_u32(&bars.peers_ready), (uint32_t)lane);
+            } else if (softmax_ok && mbar_wait(smem_u32(&bars.peers_ready), 0, abort_flag)) {
+                if (lane < S) {  // a lane per peer
+                    const int j = lane, n = rows_of(j);
+                    if (n > 0) {
+                        const uint32_t bar = in_block(smem_u32(&bars.inbox), (uint32_t)j);
+                        bulk_copy_to(in_block(sQ + (uint32_t)(split * plan.own) * kRowBytes, (uint32_t)j),
+                                     sV + (uint32_t)(j * plan.own) * kRowBytes, (uint32_t)n * kRowBytes, bar);
+                        bulk_copy_to(in_block(smem_u32(s_ml_in + split * plan.own), (uint32_t)j), smem_u32(s_ml + j * plan.own),
+                                     (uint32_t)n * 8u, bar);
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        const int n_own = min(rows_of(split), rows_blk - split * plan.own);
+        if (softmax_ok && n_own > 0 && mbar_wait(smem_u32(&bars.inbox), 0, abort_flag)) {
+            constexpr int LPR = DH / 4, RPW = 32 / LPR;  // lanes per row (four columns each), rows per warp
+            const int c4 = lane % LPR;
+            // lane s of a row's lanes looks after split s: did it have tiles, the row's maximum and sum in it
+            const bool have = c4 < S && plan.by_splits.div(tiles * (c4 + 1)) > plan.by_splits.div(tiles * c4);
+            for (int i0 = warp * RPW; i0 < n_own; i0 += (kSoftmaxThreads / 32) * RPW) {
+                const int i = min(i0 + lane / LPR, n_own - 1);
+                const int r = split * plan.own + i;  // row of the row block
+                const float2 ml = have ? s_ml_in[c4 * plan.own + i] : make_float2(-INFINITY, 0.f);
+                uint2 v[kMaxCluster];
+                const unsigned char* src = smem_gen + (size_t)i * kRowBytes + ((((c4 >> 1) ^ r) & (DH / 8 - 1)) << 4) + (c4 & 1) * 8;
+#pragma unroll
+                for (int s2 = 0; s2 < kMaxCluster; ++s2)
+                    if (s2 < S) v[s2] = *reinterpret_cast<const uint2*>(src + (size_t)s2 * plan.own * kRowBytes);
+                float mmax = ml.x;
+#pragma unroll
+                for (int o = kMaxCluster / 2; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o, LPR));
+                float w = ml.x == -INFINITY ? 0.f : ex2(ml.x - mmax), l = ml.y * w;
+#pragma unroll
+                for (int o = kMaxCluster / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o, LPR);
+                l = __shfl_sync(0xffffffffu, l, 0, LPR);
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int s2 = 0; s2 < kMaxCluster; ++s2)
+                    if (s2 < S) {
+                        const float ws2 = __shfl_sync(0xffffffffu, w, s2, LPR);
+                        if (ws2 != 0.f) {
+                            acc[0] = fmaf(__uint_as_float(v[s2].x << 16), ws2, acc[0]), acc[1] = fmaf(__uint_as_float(v[s2].x & 0xffff0000u), ws2, acc[1]);
+                            acc[2] = fmaf(__uint_as_float(v[s2].y << 16), ws2, acc[2]), acc[3] = fmaf(__uint_as_float(v[s2].y & 0xffff0000u), ws2, acc[3]);
+                        }
+                    }
+                const float inv = l > 0.f ? 1.f / l : 0.f;
+                const int pr = rb * plan.per + r, tok = plan.by_g.div(pr), hq = hk * g + (pr - tok * g);
+                if (i0 + lane / LPR < n_own) {
+                    *reinterpret_cast<uint2*>(out + (((long long)b * m + tok) * Hq + hq) * DH + c4 * 4) =
+                        make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
+                    if (lse && c4 == 0) lse[((long long)b * Hq + hq) * m + tok] = (mmax + log2f(l)) * 0.69314718055994531f;
+                }
+            }
+        }
+    }
 
     // ---- merging launches: whoever finishes a (sequence, KV head, row block) last combines its splits
     // (a pair's blocks count and merge on their own, each for its 128 rows)
@@ -1066,14 +1212,14 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     // A block whose wait ran out tells its pair block (every thread that sees the flag on its way
     // here repeats the store; whoever raised it comes by after raising it), so that both take the
     // same path below.
-    if (PAIR && s_ctl.abort) {
-        uint32_t remote;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&s_ctl.abort)), "r"(rank ^ 1u));
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(1u) : "memory");
+    if ((PAIR || CL) && s_ctl.abort) {
+        for (int r = 0; r < (PAIR ? 2 : S); ++r)
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_block(smem_u32(&s_ctl.abort), (uint32_t)r)), "r"(1u) : "memory");
         asm volatile("fence.acq_rel.cluster;" ::: "memory");  // the flag is the one thing the meeting below hands over
     }
     tc_fence_before();
-    if (PAIR) cluster_sync_relaxed();  // tensor memory is released by both blocks together
+    // (a pair releases its tensor memory together; the blocks of a cluster have all received what they wait for)
+    if (PAIR || (CL && !overflow)) cluster_sync_relaxed();
     else __syncthreads();
     tc_fence_after();
     if (s_ctl.abort) {
@@ -1087,13 +1233,14 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         }
         if (warp == kTmaWarp && lane == 0) {
             if (plan.q_tma) mbar_drain(smem_u32(&bars.q_full), 0);
+            if (CL) mbar_drain(smem_u32(&bars.inbox), 0);  // what peers have sent may still be on its way
             for (int j = max(0, k_issued - NST); j < k_issued; ++j)
                 mbar_drain(smem_u32(&bars.k_full[j % NST]), (uint32_t)((j / NST) & 1));
             for (int j = max(0, v_issued - NST); j < v_issued; ++j)
                 mbar_drain(smem_u32(&bars.v_full[j % NST]), (uint32_t)((j / NST) & 1));
         }
         tc_fence_before();
-        if (PAIR) cluster_sync_all();
+        if (PAIR || CL) cluster_sync_all();
         else __syncthreads();
         tc_fence_after();
     }
@@ -1185,14 +1332,44 @@ tree_attention_merge_kernel(const int64_t* __restrict__ kv_off, const int32_t* _
     }
 }
 
-template <int DH, int MT, bool PAIR>
+static int resident_clusters(int size) {
+    constexpr int kMaxDevices = 64;
+    static std::mutex guard;
+    static int cached[kMaxDevices][kMaxCluster + 1];  // 0: not asked yet, else clusters + 1
+    int dev = 0;
+    if (size < 1 || size > kMaxCluster || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+        cudaGetLastError();
+        return 0;
+    }
+    std::lock_guard<std::mutex> lock(guard);
+    if (cached[dev][size] == 0) {
+        auto kern = tree_attention_kernel<128, 2, false, true>;
+        const size_t smem = 200 * 1024;  // any size that leaves an SM one block
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)size * 64), cfg.blockDim = dim3(kAttnThreads), cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size, attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr, cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        cached[dev][size] = n + 1;
+    }
+    return cached[dev][size] - 1;
+}
+
+template <int DH, int MT, bool PAIR, bool CL>
 static int launch_attention(const CUtensorMap& k_map, const CUtensorMap& v_map, const CUtensorMap& q_map,
                             const void* q,
                             const int64_t* kv_off, const int32_t* kv_len, const uint64_t* mask_bits, int B,
                             int m, int Hq, int Hkv, long long cache_rows, int max_kv_len, const AttnPlan& plan,
                             float scale, void* out, float* lse, const AttnWs& ws, int32_t* d_status,
                             cudaStream_t st) {
-    auto kern = tree_attention_kernel<DH, MT, PAIR>;
+    auto kern = tree_attention_kernel<DH, MT, PAIR, CL>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem) !=
         cudaSuccess) {
         cudaGetLastError();
@@ -1204,11 +1381,11 @@ static int launch_attention(const CUtensorMap& k_map, const CUtensorMap& v_map, 
         launch_chained(tree_attention_schedule_kernel, dim3(1), dim3(1024), 0, st, 1, kv_off, kv_len, B, m, cache_rows,
                        max_kv_len, plan, ws.order, ws.tickets, plan.fused_merge ? B * Hkv * plan.n_rb * (plan.pair ? 2 : 1) : 0) != EAGLE2_OK)
         return EAGLE2_ERR_CUDA;
-    if (launch_chained(kern, dim3((unsigned)blocks), dim3(kAttnThreads), plan.smem, st, PAIR ? 2u : 1u, k_map, v_map, q_map,
+    if (launch_chained(kern, dim3((unsigned)blocks), dim3(kAttnThreads), plan.smem, st, PAIR ? 2u : CL ? (unsigned)plan.cluster : 1u, k_map, v_map, q_map,
                        static_cast<const __nv_bfloat16*>(q), kv_off, kv_len, mask_bits, m, Hq, Hkv, cache_rows, max_kv_len,
                        plan, scale * 1.4426950408889634f, static_cast<__nv_bfloat16*>(out), lse, ws, d_status) != EAGLE2_OK)
         return EAGLE2_ERR_CUDA;
-    if (plan.splits > 1 && !plan.fused_merge) {
+    if (!CL && plan.splits > 1 && !plan.fused_merge) {
         const long long warps = (long long)B * Hkv * plan.M;
         long long mblocks = (warps + 7) / 8;
         if (mblocks > 8LL * sm_count()) mblocks = 8LL * sm_count();
@@ -1236,7 +1413,7 @@ extern "C" int eagle2_tree_attention_launches(int B, int m, int Hq, int Hkv, int
         return 0;
     AttnPlan plan;
     attention_plan(B, m, Hq, Hkv, d, max_kv_len, &plan);
-    return 1 + (plan.ordered ? 1 : 0) + ((plan.splits > 1 && !plan.fused_merge) ? 1 : 0);
+    return 1 + (plan.ordered ? 1 : 0) + ((plan.splits > 1 && !plan.fused_merge && plan.cluster == 1) ? 1 : 0);
 }
 
 extern "C" int eagle2_tree_attention(const void* q, const void* k_cache, const void* v_cache,
@@ -1258,7 +1435,7 @@ extern "C" int eagle2_tree_attention(const void* q, const void* k_cache, const v
     attention_plan(B, m, Hq, Hkv, d, max_kv_len, &plan);
     if (plan.per > plan.mt * kRowsPerTile || plan.per_tok * plan.n_rb < m) return EAGLE2_ERR_SHAPE;  // (cannot happen)
     AttnWs w = {nullptr, nullptr, nullptr, nullptr};
-    if (plan.splits > 1 || plan.ordered) {
+    if ((plan.splits > 1 && plan.cluster == 1) || plan.ordered) {
         if (!ws || !aligned(ws, kWsAlign)) return EAGLE2_ERR_WORKSPACE;
         if (attention_ws_layout(B, Hkv, d, plan, ws, &w) > ws_bytes) return EAGLE2_ERR_WORKSPACE;
         if ((plan.ordered && !w.order) || (plan.fused_merge && !w.tickets)) return EAGLE2_ERR_WORKSPACE;
@@ -1275,15 +1452,21 @@ extern "C" int eagle2_tree_attention(const void* q, const void* k_cache, const v
         q_map = k_map;  // unused by the kernel
     }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-#define EAGLE2_ATTN_CASE(DH_, MT_, PAIR_)                                                                       \
-    return launch_attention<DH_, MT_, PAIR_>(k_map, v_map, q_map, q, kv_off, kv_len, mask_bits, B, m, Hq, Hkv,      \
-                                             cache_rows, max_kv_len, plan, scale, out, lse, w, d_status, st)
-    if (d == 64) {
-        if (plan.mt == 1) EAGLE2_ATTN_CASE(64, 1, false);
-        EAGLE2_ATTN_CASE(64, 2, false);
+#define EAGLE2_ATTN_CASE(DH_, MT_, PAIR_, CL_)                                                                   \
+    return launch_attention<DH_, MT_, PAIR_, CL_>(k_map, v_map, q_map, q, kv_off, kv_len, mask_bits, B, m, Hq, Hkv,  \
+                                                  cache_rows, max_kv_len, plan, scale, out, lse, w, d_status, st)
+    if (plan.cluster > 1) {
+        if (d == 64 && plan.mt == 1) EAGLE2_ATTN_CASE(64, 1, false, true);
+        if (d == 64) EAGLE2_ATTN_CASE(64, 2, false, true);
+        if (plan.mt == 1) EAGLE2_ATTN_CASE(128, 1, false, true);
+        EAGLE2_ATTN_CASE(128, 2, false, true);
     }
-    if (plan.pair) EAGLE2_ATTN_CASE(128, 1, true);
-    if (plan.mt == 1) EAGLE2_ATTN_CASE(128, 1, false);
-    EAGLE2_ATTN_CASE(128, 2, false);
+    if (d == 64) {
+        if (plan.mt == 1) EAGLE2_ATTN_CASE(64, 1, false, false);
+        EAGLE2_ATTN_CASE(64, 2, false, false);
+    }
+    if (plan.pair) EAGLE2_ATTN_CASE(128, 1, true, false);
+    if (plan.mt == 1) EAGLE2_ATTN_CASE(128, 1, false, false);
+    EAGLE2_ATTN_CASE(128, 2, false, false);
 #undef EAGLE2_ATTN_CASE
 }
