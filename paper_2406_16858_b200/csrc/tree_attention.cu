@@ -137,7 +137,7 @@ static bool single_wave_plan(int B, int m, int Hkv, int d, int tiles, AttnPlan* 
     return true;
 }
 
-static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_kv_len, AttnPlan* p) {
+static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_kv_len, bool single_wave, AttnPlan* p) {
     p->g = Hq / Hkv;
     p->M = m * p->g;
     // A block holds at most 256 packed rows, i.e. at most 256/g whole tokens (g need not divide 256).
@@ -158,7 +158,7 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
     // against 19.7 us).
     const int tiles = (max_kv_len + m + kTK - 1) / kTK;
     p->cluster = 1, p->own = 0;
-    if (single_wave_plan(B, m, Hkv, d, tiles, p)) return;
+    if (single_wave && single_wave_plan(B, m, Hkv, d, tiles, p)) return;
     p->pair = (p->mt == 2 && p->q_tma && d == 128 && items * 2 <= tpcs &&
                (tiles + tpcs / items - 1) / (tpcs / items) <= 8) ? 1 : 0;
     long long s = (p->pair ? tpcs : sms) / (items > 0 ? items : 1);
@@ -206,7 +206,7 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
 }
 
 static void attention_plan(int B, int m, int Hq, int Hkv, int d, int max_kv_len, AttnPlan* p) {
-    attention_plan_sizes(B, m, Hq, Hkv, d, max_kv_len, p);
+    attention_plan_sizes(B, m, Hq, Hkv, d, max_kv_len, true, p);
     p->by_g = FastDiv(p->g), p->by_splits = FastDiv(p->splits), p->by_n_rb = FastDiv(p->n_rb), p->by_hkv = FastDiv(Hkv);
     p->by_per_split = FastDiv(p->per_split);
     p->tile_tok = kRowsPerTile / p->g;
@@ -243,9 +243,11 @@ static size_t attention_ws_layout(int B, int Hkv, int d, const AttnPlan& p, void
     return off;
 }
 
+// A call in a single wave needs no workspace, but whether a call runs that way depends on the GPU; the size asked
+// for is the one of the plans that do, so that one answer holds everywhere.
 size_t attention_workspace_bytes(int B, int m, int Hq, int Hkv, int d, int max_kv_len) {
     AttnPlan p;
-    attention_plan(B, m, Hq, Hkv, d, max_kv_len, &p);
+    attention_plan_sizes(B, m, Hq, Hkv, d, max_kv_len, false, &p);
     return attention_ws_layout(B, Hkv, d, p, nullptr, nullptr);
 }
 
@@ -1231,13 +1233,14 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             else tc_commit(smem_u32(&bars.drain));
             mbar_drain(smem_u32(&bars.drain), 0);
         }
+        if (warp == kVWarp && lane == 0)
+            for (int j = max(0, v_issued - NST); j < v_issued; ++j)
+                mbar_drain(smem_u32(&bars.v_full[j % NST]), (uint32_t)((j / NST) & 1));
         if (warp == kTmaWarp && lane == 0) {
             if (plan.q_tma) mbar_drain(smem_u32(&bars.q_full), 0);
             if (CL) mbar_drain(smem_u32(&bars.inbox), 0);  // what peers have sent may still be on its way
             for (int j = max(0, k_issued - NST); j < k_issued; ++j)
                 mbar_drain(smem_u32(&bars.k_full[j % NST]), (uint32_t)((j / NST) & 1));
-            for (int j = max(0, v_issued - NST); j < v_issued; ++j)
-                mbar_drain(smem_u32(&bars.v_full[j % NST]), (uint32_t)((j / NST) & 1));
         }
         tc_fence_before();
         if (PAIR || CL) cluster_sync_all();
@@ -1435,9 +1438,9 @@ extern "C" int eagle2_tree_attention(const void* q, const void* k_cache, const v
     attention_plan(B, m, Hq, Hkv, d, max_kv_len, &plan);
     if (plan.per > plan.mt * kRowsPerTile || plan.per_tok * plan.n_rb < m) return EAGLE2_ERR_SHAPE;  // (cannot happen)
     AttnWs w = {nullptr, nullptr, nullptr, nullptr};
-    if ((plan.splits > 1 && plan.cluster == 1) || plan.ordered) {
-        if (!ws || !aligned(ws, kWsAlign)) return EAGLE2_ERR_WORKSPACE;
-        if (attention_ws_layout(B, Hkv, d, plan, ws, &w) > ws_bytes) return EAGLE2_ERR_WORKSPACE;
+    if (const size_t need = attention_workspace_bytes(B, m, Hq, Hkv, d, max_kv_len)) {
+        if (!ws || !aligned(ws, kWsAlign) || need > ws_bytes) return EAGLE2_ERR_WORKSPACE;
+        attention_ws_layout(B, Hkv, d, plan, ws, &w);
         if ((plan.ordered && !w.order) || (plan.fused_merge && !w.tickets)) return EAGLE2_ERR_WORKSPACE;
     }
     CUtensorMap k_map, v_map, q_map;
