@@ -1,4 +1,5 @@
-"""Builds ``libeagle2.so`` in the package directory with nvcc for sm_100a.
+"""Builds ``libeagle2.so`` in the package directory with nvcc for sm_100a, and ``_native.so``, the
+Python entry points of its launching calls, with the host compiler.
 
     python -m paper_2406_16858_b200.build [--force]
 
@@ -10,6 +11,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
@@ -17,6 +19,7 @@ _ROOT = os.path.dirname(_PKG)
 _CSRC = os.path.join(_PKG, "csrc")
 _OBJ = os.path.join(_PKG, "_build")
 LIB_PATH = os.path.join(_PKG, "libeagle2.so")
+NATIVE_PATH = os.path.join(_PKG, "_native.so")
 
 SOURCES = ["api.cu", "expand.cu", "rerank_mask.cu", "tree_attention.cu", "accept.cu", "kv_compact.cu", "lm_head.cu", "lm_head_topk.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -50,7 +53,7 @@ def _compile(src: str, force: bool, newest: float) -> tuple[str, str]:
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(_OBJ, exist_ok=True)
     newest = _newest_dep()
-    if not force and os.path.exists(LIB_PATH) and os.path.getmtime(LIB_PATH) >= newest:
+    if not force and all(os.path.exists(p) and os.path.getmtime(p) >= newest for p in (LIB_PATH, NATIVE_PATH)):
         return LIB_PATH
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as pool:
         results = list(pool.map(lambda s: _compile(s, force, newest), SOURCES))
@@ -62,6 +65,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([_nvcc(), "-shared", "-o", tmp, *[o for o, _ in results],
                            "-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB_PATH)
+    tmp = NATIVE_PATH + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(_ROOT, "include"),
+                           os.path.join(_CSRC, "binding.cpp"), "-o", tmp, "-L", _PKG, "-l:libeagle2.so", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, NATIVE_PATH)
     return LIB_PATH
 
 
