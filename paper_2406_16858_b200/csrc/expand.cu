@@ -1040,6 +1040,24 @@ static int launch_expand(const float* draft_logits, long long batch_stride, int 
                                                        d_status, stream);
 }
 
+}  // namespace eagle2
+#include "expand_rows.cuh"
+namespace eagle2 {
+
+// One step: rows that a cluster's registers hold, else tiles.
+static int launch_step(const float* draft_logits, long long batch_stride, int B, int V, int k, int D, int s, int n_s,
+                       int by_confidence, const ExpandPlan& plan, int32_t* tree_token, int32_t* tree_parent, double* tree_value,
+                       int32_t* frontier, const ExpandWs& w, int32_t* d_status, cudaStream_t st) {
+    const bool vec = aligned(draft_logits, 16) && V % 4 == 0 && batch_stride % 4 == 0;
+    int nf, cs;
+    if (expand_rows_shape((long long)B * n_s, V, &nf, &cs) && (long long)B * n_s * cs <= 0x7fffffffLL)
+        return (vec ? launch_expand_rows<true> : launch_expand_rows<false>)(draft_logits, batch_stride, B, V, k, D, s, n_s, by_confidence,
+                                                                           nf, cs, tree_token, tree_parent, tree_value, frontier,
+                                                                           w.counters, w.keys, d_status, st);
+    return (vec ? launch_expand<true> : launch_expand<false>)(draft_logits, batch_stride, B, V, k, D, s, n_s, by_confidence, plan,
+                                                             tree_token, tree_parent, tree_value, frontier, w, d_status, st);
+}
+
 // Scratch of eagle2_expand_static: lives in every context that loads the library, until exit.
 static __device__ __align__(256) unsigned char g_expand_scratch[EAGLE2_EXPAND_STATIC_BYTES];
 
@@ -1090,12 +1108,8 @@ static int expand_with_workspace(const float* draft_logits, long long batch_stri
     if (!ws || !aligned(ws, kWsAlign)) return EAGLE2_ERR_WORKSPACE;
     ExpandWs w;
     if (expand_ws_layout(B, n_s, plan.chunks, k, ws, &w) > ws_bytes) return EAGLE2_ERR_WORKSPACE;
-    const bool vec = aligned(draft_logits, 16) && V % 4 == 0 && batch_stride % 4 == 0;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    return vec ? launch_expand<true>(draft_logits, batch_stride, B, V, k, D, s, n_s, by_confidence, plan, tree_token,
-                                     tree_parent, tree_value, frontier, w, d_status, st)
-               : launch_expand<false>(draft_logits, batch_stride, B, V, k, D, s, n_s, by_confidence, plan, tree_token,
-                                      tree_parent, tree_value, frontier, w, d_status, st);
+    return launch_step(draft_logits, batch_stride, B, V, k, D, s, n_s, by_confidence, plan, tree_token, tree_parent, tree_value,
+                       frontier, w, d_status, reinterpret_cast<cudaStream_t>(stream));
 }
 
 extern "C" int eagle2_expand(const float* draft_logits, long long batch_stride, int B, int V, int k,
@@ -1145,9 +1159,6 @@ extern "C" int eagle2_expand_static(const float* draft_logits, long long batch_s
         cudaGetLastError();
         return EAGLE2_ERR_CUDA;
     }
-    const bool vec = aligned(draft_logits, 16) && V % 4 == 0 && batch_stride % 4 == 0;
-    return vec ? launch_expand<true>(draft_logits, batch_stride, B, V, k, D, s, n_s, 0, plan, tree_token, tree_parent,
-                                     tree_value, frontier, w, d_status, st)
-               : launch_expand<false>(draft_logits, batch_stride, B, V, k, D, s, n_s, 0, plan, tree_token,
-                                      tree_parent, tree_value, frontier, w, d_status, st);
+    return launch_step(draft_logits, batch_stride, B, V, k, D, s, n_s, 0, plan, tree_token, tree_parent, tree_value, frontier, w,
+                       d_status, st);
 }

@@ -1,0 +1,284 @@
+// Expansion of rows whose logits a thread-block cluster can hold in registers (included by expand.cu).
+//
+// A cluster of up to eight blocks serves one row: every thread loads its 16 to 64 logits at once, the block
+// takes their softmax sum and its k best keys from registers, and the blocks' keys and sums meet in the first
+// block's shared memory, which ranks the row's children and writes the tree level.  The last row of a sequence
+// to finish ranks the next frontier.  Against a list of partials per tile in global memory, merged by the last
+// block to arrive, that leaves one global hand-over of k numbers per row where there were two of k keys per tile,
+// and the rows of a step are merged side by side.
+//
+// What bounds it: at one sequence the chain load - sums - candidates - cluster barrier - row - ticket - frontier,
+// with many rows the logits' way from memory (64 KB in flight per block, two blocks per SM).
+#pragma once
+
+#include <cooperative_groups.h>
+
+namespace eagle2 {
+
+constexpr int kRowThreads = 256;
+constexpr int kRowWarps = kRowThreads / kWarp;
+constexpr int kRowMaxCluster = 8;
+constexpr int kRowCand = 256;  // candidates a block ranks; more (ties, rows of -inf) go through exact selection
+
+// How many of n keys are above `mine`; W neighbouring lanes share the comparisons (all of them get the count).
+template <int W>
+__device__ __forceinline__ int count_above(const unsigned long long* keys, int n, unsigned long long mine) {
+    int c = 0;
+#pragma unroll 8
+    for (int j = threadIdx.x & (W - 1); j < n; j += W) c += keys[j] > mine;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    return c;
+}
+
+template <int NF, bool VEC>
+__global__ void __launch_bounds__(kRowThreads, NF == 16 ? 2 : 3)
+expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_stride, int V, int k, int D, int s, int n_s,
+                   int by_confidence, int32_t* __restrict__ tree_token, int32_t* __restrict__ tree_parent,
+                   double* __restrict__ tree_value, int32_t* __restrict__ frontier, int* __restrict__ counters,
+                   unsigned long long* __restrict__ codes, int32_t* d_status) {
+    namespace cg = cooperative_groups;
+    constexpr int NE = 4 * NF, kSlice = kRowThreads * NE;
+    constexpr float kLog2e = 1.4426950408889634f;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int cs = (int)cluster.num_blocks(), me = (int)cluster.block_rank();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __shared__ unsigned long long s_cand[kRowCand];
+    __shared__ unsigned long long s_in[kRowMaxCluster * EAGLE2_MAX_K];  // first block: every block's k best
+    __shared__ double2 s_stats[kRowMaxCluster];                         // first block: every block's (maximum, sum)
+    __shared__ unsigned long long s_best[kRowWarps], s_code[EAGLE2_MAX_K * EAGLE2_MAX_K];
+    __shared__ float s_wmax[kRowWarps], s_wsum[kRowWarps];
+    __shared__ uint32_t s_bar;   // value code that the block's k-th best is known to reach
+    __shared__ int s_n, s_flag;
+    __shared__ double s_lse;
+
+    if (cs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (waited for before the first remote store)
+    if (tid == 0) s_bar = 0u, s_n = 0;
+    const int line = blockIdx.x / cs, row = line % n_s, b = line / n_s;
+    const float* z = draft_logits + (long long)b * batch_stride + (long long)row * V;
+    const int lo = me * kSlice;
+    auto token_of = [&](int j) { return lo + (VEC ? ((j >> 2) * kRowThreads + tid) * 4 + (j & 3) : j * kRowThreads + tid); };
+    chain_wait();
+    chain_release();
+    float x[NE];
+    if (VEC) {
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            const int e = token_of(4 * i);
+            float4 v = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            if (e < V) v = __ldcs(reinterpret_cast<const float4*>(z + e));
+            x[4 * i] = v.x, x[4 * i + 1] = v.y, x[4 * i + 2] = v.z, x[4 * i + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < NE; ++j) {
+            const int e = token_of(j);
+            x[j] = e < V ? __ldcs(z + e) : -INFINITY;
+        }
+    }
+    // the row's node and its value, needed when the row is complete
+    const long long N = nodes_of(k, D);
+    const long long base = s ? (long long)k + (long long)(s - 1) * k * k : 0;
+    int parent = -1, status = 0;
+    double parent_value = 0.0;
+    if (s && me == 0) {
+        parent = frontier[(long long)b * k + row];
+        const long long prev_base = s >= 2 ? (long long)k + (long long)(s - 2) * k * k : 0;
+        const long long prev_count = s >= 2 ? (long long)k * k : k;
+        if (parent < prev_base || parent >= prev_base + prev_count) {
+            status |= EAGLE2_STATUS_BAD_TREE;
+            parent = (int)prev_base;
+        } else {
+            parent_value = tree_value[(long long)b * N + parent];
+        }
+    }
+    __syncthreads();
+
+    // ---- maxima and the bar --------------------------------------------------------------------------
+    float gm[NF];  // of four elements each
+#pragma unroll
+    for (int i = 0; i < NF; ++i) gm[i] = fmaxf(fmaxf(x[4 * i], x[4 * i + 1]), fmaxf(x[4 * i + 2], x[4 * i + 3]));
+    float tm = gm[0];
+#pragma unroll
+    for (int i = 1; i < NF; ++i) tm = fmaxf(tm, gm[i]);
+    // A value that k lanes' largest elements reach: so does the block's k-th best.
+    const float sorted = warp_sort_desc_f32(tm);
+    const float wmax = __shfl_sync(0xffffffffu, sorted, 0), reach = __shfl_sync(0xffffffffu, sorted, k - 1);
+    if (lane == 0 && reach > -INFINITY) atomicMax(&s_bar, order_code(reach));
+    __syncthreads();
+
+    // ---- the block's candidates ------------------------------------------------------------------------
+    const uint32_t bar_code = s_bar;
+    const float bar = bar_code ? order_decode(bar_code) : -INFINITY;
+    if (tm >= bar) {
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            if (!(gm[i] >= bar)) continue;
+            int c = 0;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c += x[4 * i + e] >= bar && token_of(4 * i + e) < V;
+            int at = atomicAdd(&s_n, c);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (x[4 * i + e] >= bar && token_of(4 * i + e) < V) {
+                    if (at < kRowCand) s_cand[at] = make_key(x[4 * i + e], (uint32_t)token_of(4 * i + e));
+                    ++at;
+                }
+        }
+    }
+    // ---- and its sum of exponentials -------------------------------------------------------------------
+    float part[4] = {0.f, 0.f, 0.f, 0.f};
+    if (wmax > -INFINITY) {
+        const float2 scale2 = make_float2(kLog2e, kLog2e), neg2 = make_float2(-wmax * kLog2e, -wmax * kLog2e);
+#pragma unroll
+        for (int j = 0; j < NE; j += 2) {
+            const float2 a = __ffma2_rn(make_float2(x[j], x[j + 1]), scale2, neg2);
+            part[j & 2] += fast_ex2(a.x), part[(j & 2) + 1] += fast_ex2(a.y);
+        }
+    }
+    const float wsum = warp_sum_f32((part[0] + part[1]) + (part[2] + part[3]));
+    if (lane == 0) {
+        s_wmax[warp] = wmax, s_wsum[warp] = wsum;
+        if (!(wsum == wsum) || wmax == INFINITY) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
+    }
+    __syncthreads();
+    int n = s_n;
+    if (n > kRowCand) {
+        // exact: k times the largest key below the last one taken
+        unsigned long long last = ~0ull;
+        for (int r = 0; r < k; ++r) {
+            unsigned long long best = 0ull;
+#pragma unroll
+            for (int j = 0; j < NE; ++j) {
+                const int e = token_of(j);
+                const unsigned long long key = e < V ? make_key(x[j], (uint32_t)e) : 0ull;
+                best = key < last && key > best ? key : best;
+            }
+            best = warp_max_u64(best);
+            if (lane == 0) s_best[warp] = best;
+            __syncthreads();
+            best = 0ull;
+#pragma unroll
+            for (int w = 0; w < kRowWarps; ++w) best = s_best[w] > best ? s_best[w] : best;
+            if (tid == 0) s_cand[r] = best;
+            last = best;
+            __syncthreads();
+            if (best == 0ull) break;
+        }
+        n = k;
+        __syncthreads();
+    }
+    // ranked by counting (keys differ); straight into the first block's memory
+    if (cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    unsigned long long* to = cs > 1 ? cluster.map_shared_rank(s_in, 0) : s_in;
+    for (int i = tid >> 2; i < (n + 7 & ~7); i += kRowThreads / 4) {  // four threads share a key's comparisons
+        const unsigned long long mine = i < n ? s_cand[i] : 0ull;
+        const int rank = count_above<4>(s_cand, n, mine);
+        if ((tid & 3) == 0 && rank < k && mine) to[me * k + rank] = mine;
+    }
+    if (tid >= n && tid < k) to[me * k + tid] = 0ull;
+    if (warp == kRowWarps - 1) {
+        const float pm = lane < kRowWarps ? s_wmax[lane] : -INFINITY;
+        const float cmax = warp_max_f32(pm);
+        float term = 0.f;
+        if (lane < kRowWarps && pm > -INFINITY) term = s_wsum[lane] * fast_ex2((pm - cmax) * kLog2e);
+        const float csum = warp_sum_f32(term);
+        if (lane == 0) {
+            double2* st = cs > 1 ? cluster.map_shared_rank(s_stats, 0) : s_stats;
+            st[me] = make_double2((double)cmax, (double)csum);
+        }
+    }
+    if (cs > 1) cluster.sync();
+    else __syncthreads();
+    if (me != 0) {
+        if (status) raise_status(d_status, status);
+        return;
+    }
+
+    // ---- first block: the row's children -----------------------------------------------------------------
+    const int n_in = cs * k;  // <= 256
+    if (warp == kRowWarps - 1) {  // the row's log-sum-exp, in double
+        double m = lane < cs ? s_stats[lane].x : -INFINITY;
+#pragma unroll
+        for (int o = kRowMaxCluster / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        double sum = lane < cs && s_stats[lane].x > -INFINITY ? s_stats[lane].y * exp(s_stats[lane].x - m) : 0.0;
+#pragma unroll
+        for (int o = kRowMaxCluster / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) {
+            s_lse = m + log(sum);
+            if (!(m > -INFINITY)) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
+        }
+    }
+    // (the last warp is busy with the sum; the others rank, two threads a key)
+    constexpr int kRankers = kRowThreads - kWarp;
+    unsigned long long mine[3];
+    int rank[3];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        const int i = (tid >> 1) + u * (kRankers / 2);
+        mine[u] = 0ull, rank[u] = EAGLE2_MAX_K;
+        if (tid < kRankers && u * (kRankers / 2) < n_in) {
+            if (i < n_in) mine[u] = s_in[i];
+            rank[u] = count_above<2>(s_in, n_in, mine[u]);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        if ((tid & 1) || !mine[u] || rank[u] >= k) continue;
+        const long long at = (long long)b * N + base + (long long)row * k + rank[u];
+        const double confidence = (double)key_value(mine[u]) - s_lse;  // log c_i
+        const double v = parent_value + confidence;
+        tree_token[at] = (int32_t)key_index(mine[u]);
+        tree_parent[at] = parent;
+        tree_value[at] = v;
+        // the next frontier is ranked by value, or by confidence alone in the ablation
+        const unsigned long long code = order_code_f64(by_confidence ? confidence : v);
+        if (n_s > 1) codes[((size_t)b * n_s + row) * k + rank[u]] = code;
+        else s_code[rank[u]] = code;
+    }
+    if (status) raise_status(d_status, status);
+
+    // ---- last row of the sequence: the next frontier, by (value desc, index asc) ----------------------------
+    const int n_new = n_s * k;
+    if (n_s > 1) {
+        if (!last_block_arrives(counters + b, n_s, &s_flag)) return;
+        for (int i = tid; i < n_new; i += kRowThreads) s_code[i] = __ldcg(codes + (size_t)b * n_new + i);
+    }
+    __syncthreads();
+    for (int i = tid >> 1; i < (n_new + 15 & ~15); i += kRowThreads / 2) {  // two threads a candidate
+        const unsigned long long ci = i < n_new ? s_code[i] : 0ull;
+        int place = 0;
+#pragma unroll 8
+        for (int j = tid & 1; j < n_new; j += 2) {
+            const unsigned long long cj = s_code[j];
+            place += (cj > ci) || (cj == ci && j < i);
+        }
+        place += __shfl_xor_sync(0xffffffffu, place, 1);
+        if ((tid & 1) == 0 && i < n_new && place < k) frontier[(long long)b * k + place] = (int32_t)(base + i);
+    }
+}
+
+// Slices: the shortest (most blocks) that keep the launch on the device at once; else the longest.
+// Many rows of a large vocabulary are left to the tiles, which keep more of memory's bandwidth busy (six steps at
+// V = 128256, 1 / 2 / 4 / 8 / 16 / 32 sequences of ten rows: 78 / 107 / 140 / 199 / 238 / 293 us in tiles, 72 / 80 /
+// 116 / 159 / 258 / 454 us this way; at V = 32000 69 / 73 / 77 / 109 / 145 / 224 against 56 / 57 / 64 / 78 / 115 /
+// 163 us, 64 sequences 306 against 263).
+static bool expand_rows_shape(long long rows, int V, int* nf, int* cs) {
+    if (V > kRowMaxCluster * kRowThreads * 64 || (rows > 128 && V > 2 * kRowThreads * 64)) return false;
+    for (*nf = 4;; *nf *= 2) {
+        *cs = (V + kRowThreads * 4 * *nf - 1) / (kRowThreads * 4 * *nf);
+        if (*nf == 16 || *cs == 1 || (*cs <= kRowMaxCluster && rows * *cs <= 2LL * sm_count())) return true;
+    }
+}
+
+template <bool VEC>
+static int launch_expand_rows(const float* logits, long long batch_stride, int B, int V, int k, int D, int s, int n_s,
+                              int by_confidence, int nf, int cs, int32_t* token, int32_t* parent, double* value, int32_t* frontier,
+                              int* counters, unsigned long long* codes, int32_t* d_status, cudaStream_t st) {
+    auto kern = nf == 4 ? expand_rows_kernel<4, VEC> : nf == 8 ? expand_rows_kernel<8, VEC> : expand_rows_kernel<16, VEC>;
+    return launch_chained(kern, dim3((unsigned)((long long)B * n_s * cs)), dim3(kRowThreads), 0, st, (unsigned)cs, logits, batch_stride,
+                          V, k, D, s, n_s, by_confidence, token, parent, value, frontier, counters, codes, d_status);
+}
+
+}  // namespace eagle2
