@@ -48,12 +48,12 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     __shared__ double2 s_stats[kRowMaxCluster];                         // first block: every block's (maximum, sum)
     __shared__ unsigned long long s_best[kRowWarps], s_code[EAGLE2_MAX_K * EAGLE2_MAX_K];
     __shared__ float s_wmax[kRowWarps], s_wsum[kRowWarps];
-    __shared__ uint32_t s_bar;   // value code that the block's k-th best is known to reach
+    __shared__ uint32_t s_top[kRowWarps * EAGLE2_MAX_K], s_bar;  // value codes: the warps' largest, the bar
     __shared__ int s_n, s_flag;
     __shared__ double s_lse;
 
     if (cs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (waited for before the first remote store)
-    if (tid == 0) s_bar = 0u, s_n = 0;
+    if (tid == 0) s_bar = ~0u, s_n = 0;
     const int line = blockIdx.x / cs, row = line % n_s, b = line / n_s;
     const float* z = draft_logits + (long long)b * batch_stride + (long long)row * V;
     const int lo = me * kSlice;
@@ -101,15 +101,24 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     float tm = gm[0];
 #pragma unroll
     for (int i = 1; i < NF; ++i) tm = fmaxf(tm, gm[i]);
-    // A value that k lanes' largest elements reach: so does the block's k-th best.
+    // The k-th largest of the threads' maxima is a value that k elements reach: so does the block's k-th best, and
+    // no more than k threads hold elements that do.  The warps' k largest, then the k-th of those.
     const float sorted = warp_sort_desc_f32(tm);
-    const float wmax = __shfl_sync(0xffffffffu, sorted, 0), reach = __shfl_sync(0xffffffffu, sorted, k - 1);
-    if (lane == 0 && reach > -INFINITY) atomicMax(&s_bar, order_code(reach));
+    const float wmax = __shfl_sync(0xffffffffu, sorted, 0);
+    if (lane < k) s_top[warp * k + lane] = order_code(sorted);
+    __syncthreads();
+    for (int i = tid >> 1; i < (kRowWarps * k + 15 & ~15); i += kRowThreads / 2) {  // two threads a value
+        const uint32_t mine = i < kRowWarps * k ? s_top[i] : ~0u;
+        int above = 0;
+#pragma unroll 8
+        for (int j = tid & 1; j < kRowWarps * k; j += 2) above += s_top[j] > mine;
+        above += __shfl_xor_sync(0xffffffffu, above, 1);
+        if (above < k) atomicMin(&s_bar, mine);
+    }
     __syncthreads();
 
     // ---- the block's candidates ------------------------------------------------------------------------
-    const uint32_t bar_code = s_bar;
-    const float bar = bar_code ? order_decode(bar_code) : -INFINITY;
+    const float bar = order_decode(s_bar);
     if (tm >= bar) {
 #pragma unroll
         for (int i = 0; i < NF; ++i) {
