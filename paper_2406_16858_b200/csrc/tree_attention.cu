@@ -694,19 +694,10 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 
     if (active) {
     if (warp == kTmaWarp) {
-        // ===== producer of Q and K tiles (V has its own: a K stage is free long before the V stage of the
-        // same tile, and one lane that serves both in order would leave it empty meanwhile) ==========
+        // ===== producer of K tiles.  V has its own, which asks for the queries too, so that all three set off at once: a K
+        // stage is free long before the V stage of the same tile, and one lane that serves both in order would leave it
+        // empty meanwhile ==========
         if (lane == 0) {
-            if (plan.q_tma) {
-                mbar_expect_tx(smem_u32(&bars.q_full), MT * kTile);
-#pragma unroll
-                for (int t = 0; t < MT; ++t)
-#pragma unroll
-                    for (int h = 0; h < HALVES; ++h)
-                        tma_load_4d(sQ + t * kTile + h * kPanel, &q_map, h * 64, 0,
-                                    b * m + rb * plan.per_tok + (t + (int)rank) * (int)plan.tile_tok, hk,
-                                    smem_u32(&bars.q_full));
-            }
             int st = 0, row = (int)(row_base + (long long)t_begin * kTK);
             uint32_t ph = 1;
             for (int j = 0; j < nt; ++j, row += kTK) {
@@ -722,11 +713,21 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         }
         __syncwarp();
     } else if (warp == kVWarp) {
-        // ===== producer of V tiles ================================================================
+        // ===== producer of Q and V tiles =============================================================
         bool ok = true;
         int st = 0, last_st = 0;
         uint32_t ph = 1, last_ph = 1;
         if (lane == 0) {
+            if (plan.q_tma) {
+                mbar_expect_tx(smem_u32(&bars.q_full), MT * kTile);
+#pragma unroll
+                for (int t = 0; t < MT; ++t)
+#pragma unroll
+                    for (int h = 0; h < HALVES; ++h)
+                        tma_load_4d(sQ + t * kTile + h * kPanel, &q_map, h * 64, 0,
+                                    b * m + rb * plan.per_tok + (t + (int)rank) * (int)plan.tile_tok, hk,
+                                    smem_u32(&bars.q_full));
+            }
             int row = (int)(row_base + (long long)t_begin * kTK);
             for (int j = 0; j < nt; ++j, row += kTK) {
                 if (j >= NST) ok = mbar_wait(smem_u32(&bars.v_empty[st]), ph, abort_flag);
@@ -1125,61 +1126,67 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     // partial rows through L2 and a second launch that combines them, costs that launch's start and a cold
     // pass through its code.)
     if (CL && !overflow && warp < kTmaWarp) {
-        if (warp == 0) {
-            if (!active) {
-                if (lane < S) mbar_arrive_in(smem_u32(&bars.peers_ready), (uint32_t)lane);
-            } else if (softmax_ok && mbar_wait(smem_u32(&bars.peers_ready), 0, abort_flag)) {
-                if (lane < S) {  // a lane per peer
-                    const int j = lane, n = rows_of(j);
-                    if (n > 0) {
-                        const uint32_t bar = in_block(smem_u32(&bars.inbox), (uint32_t)j);
-                        bulk_copy_to(in_block(sQ + (uint32_t)(split * plan.own) * kRowBytes, (uint32_t)j),
-                                     sV + (uint32_t)(j * plan.own) * kRowBytes, (uint32_t)n * kRowBytes, bar);
-                        bulk_copy_to(in_block(smem_u32(s_ml_in + split * plan.own), (uint32_t)j), smem_u32(s_ml + j * plan.own),
-                                     (uint32_t)n * 8u, bar);
+        if (!active) {
+            if (warp == 0 && lane < S) mbar_arrive_in(smem_u32(&bars.peers_ready), (uint32_t)lane);
+        } else if (softmax_ok && warp < S && lane == 0 && mbar_wait(smem_u32(&bars.peers_ready), 0, abort_flag)) {
+            const int j = warp, n = rows_of(j);  // a warp per peer
+            if (n > 0) {
+                const uint32_t bar = in_block(smem_u32(&bars.inbox), (uint32_t)j);
+                bulk_copy_to(in_block(sQ + (uint32_t)(split * plan.own) * kRowBytes, (uint32_t)j),
+                             sV + (uint32_t)(j * plan.own) * kRowBytes, (uint32_t)n * kRowBytes, bar);
+                bulk_copy_to(in_block(smem_u32(s_ml_in + split * plan.own), (uint32_t)j), smem_u32(s_ml + j * plan.own),
+                             (uint32_t)n * 8u, bar);
+            }
+        }
+        __syncwarp();
+        const int n_own = min(rows_of(split), rows_blk - split * plan.own);
+        // Four rows per warp side by side: lane 8 r + s weighs part s of row r, then the warp goes over the rows with
+        // DH / 4 lanes each (four columns a lane).  (One row at a time was 0.65 us a row of dependent steps.)
+        if (softmax_ok && n_own > 0 && mbar_wait(smem_u32(&bars.inbox), 0, abort_flag)) {
+            constexpr int R = 4, LPR = DH / 4, RPW = 32 / LPR, Q = R / RPW, W = kSoftmaxThreads / 32;
+            const int part = lane & 7, c4 = lane % LPR;
+            // did block `part` have tiles
+            const bool have = part < S && plan.by_splits.div(tiles * (part + 1)) > plan.by_splits.div(tiles * part);
+            const unsigned parts = __ballot_sync(0xffffffffu, have);
+            for (int i0 = warp; i0 < n_own; i0 += W * R) {  // rows i0, i0 + W, ...: few rows are a row per warp
+                const float2 ml = have ? s_ml_in[part * plan.own + min(i0 + (lane >> 3) * W, n_own - 1)] : make_float2(-INFINITY, 0.f);
+                uint2 v[Q][kMaxCluster];
+#pragma unroll
+                for (int qq = 0; qq < Q; ++qq) {
+                    const int i = min(i0 + (qq * RPW + lane / LPR) * W, n_own - 1), r = split * plan.own + i;
+                    const unsigned char* src = smem_gen + (size_t)i * kRowBytes + ((((c4 >> 1) ^ r) & (DH / 8 - 1)) << 4) + (c4 & 1) * 8;
+#pragma unroll
+                    for (int s2 = 0; s2 < kMaxCluster; ++s2) {
+                        v[qq][s2] = make_uint2(0u, 0u);
+                        if (((parts >> s2) & 1u) && i0 + qq * RPW * W < n_own) v[qq][s2] = *reinterpret_cast<const uint2*>(src + (size_t)(s2 * plan.own) * kRowBytes);
                     }
                 }
-            }
-            __syncwarp();
-        }
-        const int n_own = min(rows_of(split), rows_blk - split * plan.own);
-        if (softmax_ok && n_own > 0 && mbar_wait(smem_u32(&bars.inbox), 0, abort_flag)) {
-            constexpr int LPR = DH / 4, RPW = 32 / LPR;  // lanes per row (four columns each), rows per warp
-            const int c4 = lane % LPR;
-            // lane s of a row's lanes looks after split s: did it have tiles, the row's maximum and sum in it
-            const bool have = c4 < S && plan.by_splits.div(tiles * (c4 + 1)) > plan.by_splits.div(tiles * c4);
-            for (int i0 = warp * RPW; i0 < n_own; i0 += (kSoftmaxThreads / 32) * RPW) {
-                const int i = min(i0 + lane / LPR, n_own - 1);
-                const int r = split * plan.own + i;  // row of the row block
-                const float2 ml = have ? s_ml_in[c4 * plan.own + i] : make_float2(-INFINITY, 0.f);
-                uint2 v[kMaxCluster];
-                const unsigned char* src = smem_gen + (size_t)i * kRowBytes + ((((c4 >> 1) ^ r) & (DH / 8 - 1)) << 4) + (c4 & 1) * 8;
-#pragma unroll
-                for (int s2 = 0; s2 < kMaxCluster; ++s2)
-                    if (s2 < S) v[s2] = *reinterpret_cast<const uint2*>(src + (size_t)s2 * plan.own * kRowBytes);
                 float mmax = ml.x;
 #pragma unroll
-                for (int o = kMaxCluster / 2; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o, LPR));
+                for (int o = 4; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
                 float w = ml.x == -INFINITY ? 0.f : ex2(ml.x - mmax), l = ml.y * w;
 #pragma unroll
-                for (int o = kMaxCluster / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o, LPR);
-                l = __shfl_sync(0xffffffffu, l, 0, LPR);
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int o = 4; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+                w *= l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
-                for (int s2 = 0; s2 < kMaxCluster; ++s2)
-                    if (s2 < S) {
-                        const float ws2 = __shfl_sync(0xffffffffu, w, s2, LPR);
-                        if (ws2 != 0.f) {
-                            acc[0] = fmaf(__uint_as_float(v[s2].x << 16), ws2, acc[0]), acc[1] = fmaf(__uint_as_float(v[s2].x & 0xffff0000u), ws2, acc[1]);
-                            acc[2] = fmaf(__uint_as_float(v[s2].y << 16), ws2, acc[2]), acc[3] = fmaf(__uint_as_float(v[s2].y & 0xffff0000u), ws2, acc[3]);
-                        }
+                for (int qq = 0; qq < Q; ++qq) {
+                    if (i0 + qq * RPW * W >= n_own) break;
+                    const int rr = qq * RPW + lane / LPR, i = i0 + rr * W;
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int s2 = 0; s2 < kMaxCluster; ++s2) {
+                        if (s2 >= S) continue;
+                        const float ws2 = __shfl_sync(0xffffffffu, w, rr * 8 + s2);
+                        acc[0] = fmaf(__uint_as_float(v[qq][s2].x << 16), ws2, acc[0]), acc[1] = fmaf(__uint_as_float(v[qq][s2].x & 0xffff0000u), ws2, acc[1]);
+                        acc[2] = fmaf(__uint_as_float(v[qq][s2].y << 16), ws2, acc[2]), acc[3] = fmaf(__uint_as_float(v[qq][s2].y & 0xffff0000u), ws2, acc[3]);
                     }
-                const float inv = l > 0.f ? 1.f / l : 0.f;
-                const int pr = rb * plan.per + r, tok = plan.by_g.div(pr), hq = hk * g + (pr - tok * g);
-                if (i0 + lane / LPR < n_own) {
-                    *reinterpret_cast<uint2*>(out + (((long long)b * m + tok) * Hq + hq) * DH + c4 * 4) =
-                        make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
-                    if (lse && c4 == 0) lse[((long long)b * Hq + hq) * m + tok] = (mmax + log2f(l)) * 0.69314718055994531f;
+                    const float m_row = __shfl_sync(0xffffffffu, mmax, rr * 8), l_row = __shfl_sync(0xffffffffu, l, rr * 8);
+                    const int pr = rb * plan.per + split * plan.own + i, tok = plan.by_g.div(pr), hq = hk * g + (pr - tok * g);
+                    if (i < n_own) {
+                        *reinterpret_cast<uint2*>(out + (((long long)b * m + tok) * Hq + hq) * DH + c4 * 4) =
+                            make_uint2(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]));
+                        if (lse && c4 == 0) lse[((long long)b * Hq + hq) * m + tok] = (m_row + log2f(l_row)) * 0.69314718055994531f;
+                    }
                 }
             }
         }
@@ -1233,11 +1240,12 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             else tc_commit(smem_u32(&bars.drain));
             mbar_drain(smem_u32(&bars.drain), 0);
         }
-        if (warp == kVWarp && lane == 0)
+        if (warp == kVWarp && lane == 0) {
+            if (plan.q_tma) mbar_drain(smem_u32(&bars.q_full), 0);
             for (int j = max(0, v_issued - NST); j < v_issued; ++j)
                 mbar_drain(smem_u32(&bars.v_full[j % NST]), (uint32_t)((j / NST) & 1));
+        }
         if (warp == kTmaWarp && lane == 0) {
-            if (plan.q_tma) mbar_drain(smem_u32(&bars.q_full), 0);
             if (CL) mbar_drain(smem_u32(&bars.inbox), 0);  // what peers have sent may still be on its way
             for (int j = max(0, k_issued - NST); j < k_issued; ++j)
                 mbar_drain(smem_u32(&bars.k_full[j % NST]), (uint32_t)((j / NST) & 1));
