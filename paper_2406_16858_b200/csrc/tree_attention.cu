@@ -42,7 +42,7 @@ constexpr int kTmemCols = 512;
 constexpr int kMaxCluster = 8;
 constexpr int kSlots = 2;             // score slots in tensor memory
 constexpr int kSoftmaxThreads = 256;  // 8 softmax warps: two per SM sub-partition, one of each group
-constexpr int kAttnThreads = kSoftmaxThreads + 96;  // ... the warps that request K (and Q), issue MMAs, request V
+constexpr int kAttnThreads = kSoftmaxThreads + 96;  // ... the warps that request K, issue MMAs, request Q and V
 
 // Division of 31-bit numbers by a launch constant: a multiplication and a shift instead of the ~100 dependent
 // cycles of a run-time division (a block works out its place with half a dozen of them before its first request).
