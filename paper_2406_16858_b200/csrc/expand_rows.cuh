@@ -18,7 +18,9 @@ namespace eagle2 {
 constexpr int kRowThreads = 256;
 constexpr int kRowWarps = kRowThreads / kWarp;
 constexpr int kRowMaxCluster = 8;
-constexpr int kRowCand = 256;  // candidates a block ranks; more (ties, rows of -inf) go through exact selection
+constexpr int kRowGroups = 32;   // groups of eight threads, whose maxima give the bar
+static_assert(kRowGroups * 8 == kRowThreads && EAGLE2_MAX_K <= kRowGroups, "the bar is one of the groups' maxima");
+constexpr int kRowCand = 512;  // candidates a block ranks; more (ties, rows of -inf) go through exact selection
 
 // How many of n keys are above `mine`; W neighbouring lanes share the comparisons (all of them get the count).
 template <int W>
@@ -30,6 +32,9 @@ __device__ __forceinline__ int count_above(const unsigned long long* keys, int n
     for (int o = 1; o < W; o <<= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     return c;
 }
+
+// 2^d for a whole d <= 0 (0 below the smallest normal number; NaN stays), exactly
+__device__ __forceinline__ float pow2_whole(float d) { return d >= -126.f ? __int_as_float(((int)d + 127) << 23) : d * 0.f; }
 
 template <int NF, bool VEC>
 __global__ void __launch_bounds__(kRowThreads, NF == 16 ? 2 : 3)
@@ -45,15 +50,15 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     __shared__ unsigned long long s_cand[kRowCand];
     __shared__ unsigned long long s_in[kRowMaxCluster * EAGLE2_MAX_K];  // first block: every block's k best
-    __shared__ double2 s_stats[kRowMaxCluster];                         // first block: every block's (maximum, sum)
+    __shared__ float2 s_stats[kRowMaxCluster];                          // first block: every block's (reference, sum)
     __shared__ unsigned long long s_best[kRowWarps], s_code[EAGLE2_MAX_K * EAGLE2_MAX_K];
-    __shared__ float s_wmax[kRowWarps], s_wsum[kRowWarps];
-    __shared__ uint32_t s_top[kRowWarps * EAGLE2_MAX_K], s_bar;  // value codes: the warps' largest, the bar
+    __shared__ float s_wref[kRowWarps], s_wsum[kRowWarps];
+    __shared__ __align__(16) float s_top[kRowGroups];
     __shared__ int s_n, s_flag;
     __shared__ double s_lse;
 
     if (cs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (waited for before the first remote store)
-    if (tid == 0) s_bar = ~0u, s_n = 0;
+    if (tid == 0) s_n = 0;
     const int line = blockIdx.x / cs, row = line % n_s, b = line / n_s;
     const float* z = draft_logits + (long long)b * batch_stride + (long long)row * V;
     const int lo = me * kSlice;
@@ -92,33 +97,57 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
             parent_value = tree_value[(long long)b * N + parent];
         }
     }
-    __syncthreads();
 
-    // ---- maxima and the bar --------------------------------------------------------------------------
+    // ---- maxima --------------------------------------------------------------------------
     float gm[NF];  // of four elements each
 #pragma unroll
     for (int i = 0; i < NF; ++i) gm[i] = fmaxf(fmaxf(x[4 * i], x[4 * i + 1]), fmaxf(x[4 * i + 2], x[4 * i + 3]));
     float tm = gm[0];
 #pragma unroll
     for (int i = 1; i < NF; ++i) tm = fmaxf(tm, gm[i]);
-    // The k-th largest of the threads' maxima is a value that k elements reach: so does the block's k-th best, and
-    // no more than k threads hold elements that do.  The warps' k largest, then the k-th of those.
-    const float sorted = warp_sort_desc_f32(tm);
-    const float wmax = __shfl_sync(0xffffffffu, sorted, 0);
-    if (lane < k) s_top[warp * k + lane] = order_code(sorted);
-    __syncthreads();
-    for (int i = tid >> 1; i < (kRowWarps * k + 15 & ~15); i += kRowThreads / 2) {  // two threads a value
-        const uint32_t mine = i < kRowWarps * k ? s_top[i] : ~0u;
-        int above = 0;
-#pragma unroll 8
-        for (int j = tid & 1; j < kRowWarps * k; j += 2) above += s_top[j] > mine;
-        above += __shfl_xor_sync(0xffffffffu, above, 1);
-        if (above < k) atomicMin(&s_bar, mine);
+    float um = tm;  // of eight threads
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) um = fmaxf(um, __shfl_xor_sync(0xffffffffu, um, o));
+    if ((lane & 7) == 0) s_top[tid >> 3] = um;
+    float wmax = fmaxf(um, __shfl_xor_sync(0xffffffffu, um, 8));
+    wmax = fmaxf(wmax, __shfl_xor_sync(0xffffffffu, wmax, 16));
+
+    // ---- the sum of exponentials -----------------------------------------------------------------------
+    // Relative to the warp's maximum in base 2, rounded up to a whole number: factors between references are exact.
+    const float wref = ceilf(wmax * kLog2e);
+    float part[4] = {0.f, 0.f, 0.f, 0.f};
+    if (wmax > -INFINITY) {
+        const float2 scale2 = make_float2(kLog2e, kLog2e), neg2 = make_float2(-wref, -wref);
+#pragma unroll
+        for (int j = 0; j < NE; j += 2) {
+            const float2 a = __ffma2_rn(make_float2(x[j], x[j + 1]), scale2, neg2);
+            part[j & 2] += fast_ex2(a.x), part[(j & 2) + 1] += fast_ex2(a.y);
+        }
+    }
+    const float wsum = warp_sum_f32((part[0] + part[1]) + (part[2] + part[3]));
+    if (lane == 0) {
+        s_wref[warp] = wref, s_wsum[warp] = wsum;
+        if (!(wsum == wsum) || wmax == INFINITY) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
     }
     __syncthreads();
 
+    // ---- the bar ------------------------------------------------------------------------------------------
+    // The k-th largest of the 32 groups' maxima is a value that k elements reach: so does the block's k-th best, and
+    // about 32 ln(32 / (32 - k)) elements do (12 for k = 10).  Every warp works it out for itself.  (The k-th of the
+    // threads' maxima leaves 10, but takes a sort per warp and another meeting of the block: 0.7 us of a call's 8.)
+    float bar;
+    {
+        const float mine = s_top[lane];
+        int above = 0;
+#pragma unroll
+        for (int j = 0; j < kRowGroups; j += 4) {
+            const float4 t = *reinterpret_cast<const float4*>(s_top + j);
+            above += (t.x > mine) + (t.y > mine) + (t.z > mine) + (t.w > mine);
+        }
+        bar = order_decode(__reduce_min_sync(0xffffffffu, above < k ? order_code(mine) : ~0u));
+    }
+
     // ---- the block's candidates ------------------------------------------------------------------------
-    const float bar = order_decode(s_bar);
     if (tm >= bar) {
 #pragma unroll
         for (int i = 0; i < NF; ++i) {
@@ -134,21 +163,6 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
                     ++at;
                 }
         }
-    }
-    // ---- and its sum of exponentials -------------------------------------------------------------------
-    float part[4] = {0.f, 0.f, 0.f, 0.f};
-    if (wmax > -INFINITY) {
-        const float2 scale2 = make_float2(kLog2e, kLog2e), neg2 = make_float2(-wmax * kLog2e, -wmax * kLog2e);
-#pragma unroll
-        for (int j = 0; j < NE; j += 2) {
-            const float2 a = __ffma2_rn(make_float2(x[j], x[j + 1]), scale2, neg2);
-            part[j & 2] += fast_ex2(a.x), part[(j & 2) + 1] += fast_ex2(a.y);
-        }
-    }
-    const float wsum = warp_sum_f32((part[0] + part[1]) + (part[2] + part[3]));
-    if (lane == 0) {
-        s_wmax[warp] = wmax, s_wsum[warp] = wsum;
-        if (!(wsum == wsum) || wmax == INFINITY) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
     }
     __syncthreads();
     int n = s_n;
@@ -187,14 +201,12 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     }
     if (tid >= n && tid < k) to[me * k + tid] = 0ull;
     if (warp == kRowWarps - 1) {
-        const float pm = lane < kRowWarps ? s_wmax[lane] : -INFINITY;
-        const float cmax = warp_max_f32(pm);
-        float term = 0.f;
-        if (lane < kRowWarps && pm > -INFINITY) term = s_wsum[lane] * fast_ex2((pm - cmax) * kLog2e);
-        const float csum = warp_sum_f32(term);
+        const float ref = lane < kRowWarps ? s_wref[lane] : -INFINITY;
+        const float cref = warp_max_f32(ref);
+        const float csum = warp_sum_f32(ref > -INFINITY ? s_wsum[lane] * pow2_whole(ref - cref) : 0.f);
         if (lane == 0) {
-            double2* st = cs > 1 ? cluster.map_shared_rank(s_stats, 0) : s_stats;
-            st[me] = make_double2((double)cmax, (double)csum);
+            float2* st = cs > 1 ? cluster.map_shared_rank(s_stats, 0) : s_stats;
+            st[me] = make_float2(cref, csum);
         }
     }
     if (cs > 1) cluster.sync();
@@ -207,14 +219,15 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     // ---- first block: the row's children -----------------------------------------------------------------
     const int n_in = cs * k;  // <= 256
     if (warp == kRowWarps - 1) {  // the row's log-sum-exp, in double
-        double m = lane < cs ? s_stats[lane].x : -INFINITY;
+        const float2 st = lane < cs ? s_stats[lane] : make_float2(-INFINITY, 0.f);
+        float m = st.x;
 #pragma unroll
-        for (int o = kRowMaxCluster / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        double sum = lane < cs && s_stats[lane].x > -INFINITY ? s_stats[lane].y * exp(s_stats[lane].x - m) : 0.0;
+        for (int o = kRowMaxCluster / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        double sum = st.x > -INFINITY ? (double)(st.y * pow2_whole(st.x - m)) : 0.0;
 #pragma unroll
         for (int o = kRowMaxCluster / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (lane == 0) {
-            s_lse = m + log(sum);
+            s_lse = (double)m * 0.69314718055994530942 + log(sum);
             if (!(m > -INFINITY)) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
         }
     }
