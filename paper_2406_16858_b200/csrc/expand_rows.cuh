@@ -51,6 +51,7 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     __shared__ unsigned long long s_cand[kRowCand];
     __shared__ unsigned long long s_in[kRowMaxCluster * EAGLE2_MAX_K];  // first block: every block's k best
     __shared__ float2 s_stats[kRowMaxCluster];                          // first block: every block's (reference, sum)
+    __shared__ unsigned long long s_row[EAGLE2_MAX_K];                  // first block: the row's k best
     __shared__ unsigned long long s_best[kRowWarps], s_code[EAGLE2_MAX_K * EAGLE2_MAX_K];
     __shared__ float s_wref[kRowWarps], s_wsum[kRowWarps];
     __shared__ __align__(16) float s_top[kRowGroups];
@@ -59,6 +60,7 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
 
     if (cs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (waited for before the first remote store)
     if (tid == 0) s_n = 0;
+    if (tid < k) s_row[tid] = 0ull;
     const int line = blockIdx.x / cs, row = line % n_s, b = line / n_s;
     const float* z = draft_logits + (long long)b * batch_stride + (long long)row * V;
     const int lo = me * kSlice;
@@ -233,40 +235,43 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     }
     // (the last warp is busy with the sum; the others rank, two threads a key)
     constexpr int kRankers = kRowThreads - kWarp;
-    unsigned long long mine[3];
-    int rank[3];
-#pragma unroll
-    for (int u = 0; u < 3; ++u) {
-        const int i = (tid >> 1) + u * (kRankers / 2);
-        mine[u] = 0ull, rank[u] = EAGLE2_MAX_K;
-        if (tid < kRankers && u * (kRankers / 2) < n_in) {
-            if (i < n_in) mine[u] = s_in[i];
-            rank[u] = count_above<2>(s_in, n_in, mine[u]);
+    if (tid < kRankers)
+        for (int i = tid >> 1; i < (n_in + 15 & ~15); i += kRankers / 2) {
+            const unsigned long long mine = i < n_in ? s_in[i] : 0ull;
+            const int rank = count_above<2>(s_in, n_in, mine);
+            if ((tid & 1) == 0 && mine && rank < k) s_row[rank] = mine;
         }
-    }
     __syncthreads();
-#pragma unroll
-    for (int u = 0; u < 3; ++u) {
-        if ((tid & 1) || !mine[u] || rank[u] >= k) continue;
-        const long long at = (long long)b * N + base + (long long)row * k + rank[u];
-        const double confidence = (double)key_value(mine[u]) - s_lse;  // log c_i
+    // A lane per child: what the row hands on is written by one warp, whose first lane announces it without another
+    // meeting of the block.
+    if (tid < k && s_row[tid]) {
+        const long long at = (long long)b * N + base + (long long)row * k + tid;
+        const double confidence = (double)key_value(s_row[tid]) - s_lse;  // log c_i
         const double v = parent_value + confidence;
-        tree_token[at] = (int32_t)key_index(mine[u]);
+        tree_token[at] = (int32_t)key_index(s_row[tid]);
         tree_parent[at] = parent;
         tree_value[at] = v;
         // the next frontier is ranked by value, or by confidence alone in the ablation
-        const unsigned long long code = order_code_f64(by_confidence ? confidence : v);
-        if (n_s > 1) codes[((size_t)b * n_s + row) * k + rank[u]] = code;
-        else s_code[rank[u]] = code;
+        if (n_s > 1) codes[((size_t)b * n_s + row) * k + tid] = order_code_f64(by_confidence ? confidence : v);
     }
+    if (n_s == 1 && tid < k) frontier[(long long)b * k + tid] = (int32_t)(base + tid);  // a row's children are in order
     if (status) raise_status(d_status, status);
+    if (n_s == 1) return;
 
     // ---- last row of the sequence: the next frontier, by (value desc, index asc) ----------------------------
     const int n_new = n_s * k;
-    if (n_s > 1) {
-        if (!last_block_arrives(counters + b, n_s, &s_flag)) return;
-        for (int i = tid; i < n_new; i += kRowThreads) s_code[i] = __ldcg(codes + (size_t)b * n_new + i);
+    if (warp == 0) {
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();  // cumulative: covers the stores of the warp's other lanes
+            s_flag = atomicAdd(counters + b, 1) == n_s - 1;
+            if (s_flag) counters[b] = 0;
+        }
     }
+    __syncthreads();
+    if (!s_flag) return;
+    __threadfence();
+    for (int i = tid; i < n_new; i += kRowThreads) s_code[i] = __ldcg(codes + (size_t)b * n_new + i);
     __syncthreads();
     for (int i = tid >> 1; i < (n_new + 15 & ~15); i += kRowThreads / 2) {  // two threads a candidate
         const unsigned long long ci = i < n_new ? s_code[i] : 0ull;
