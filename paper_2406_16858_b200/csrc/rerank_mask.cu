@@ -8,6 +8,7 @@
 namespace eagle2 {
 
 constexpr int kRerankThreads = 512;
+constexpr int kRerankCand = 512;  // candidates ranked by counting; more (ties of thousands of nodes) are sorted
 
 // Monotone map double -> uint64 (larger value, larger code; -0 folded onto +0).  The caller has
 // already replaced NaN.
@@ -51,11 +52,13 @@ __device__ __forceinline__ int mask_row(const int32_t* s_par, int i, int ns, int
     return status;
 }
 
-// Values are compared as integer codes throughout (fp64 compares are slow on this part).  The
-// ranking is a bitonic sort of (code, index) pairs, padded to a power of two with code 0, which
-// sorts behind every real value.  With `frontier` given there is no ranking at all (the ablation
-// without reranking, Section 5.2): the selection is every node the expansion phase selected, i.e.
-// every node that is some node's parent plus the last step's frontier, lowest indices first.
+// Values are compared as integer codes throughout (fp64 compares are slow on this part).  Only the set of the `most`
+// best nodes is needed, not their order: the maxima of groups of two or four threads give a bar that `most` nodes
+// reach (few more do), and the nodes that reach it are ranked by counting.  What bounds it is latency, one block per
+// sequence in a chain of a dozen block-wide steps; sorting all 510 nodes of k = 10, D = 6 took another 45.
+// With `frontier` given there is no ranking at all (the ablation without reranking, Section 5.2): the selection is every
+// node the expansion phase selected, i.e. every node that is some node's parent plus the last step's frontier, lowest
+// indices first.
 __global__ void __launch_bounds__(kRerankThreads)
 rerank_kernel(const int32_t* __restrict__ tree_token, const int32_t* __restrict__ tree_parent,
               const double* __restrict__ tree_value, const int32_t* __restrict__ frontier, int k, int N,
@@ -107,7 +110,11 @@ rerank_kernel(const int32_t* __restrict__ tree_token, const int32_t* __restrict_
     } else {
     // effective value = minimum of the values on the path from the root (parents have lower
     // indices, so the walk ends)
-    for (int i = tid; i < P; i += kRerankThreads) {
+    // (a group's threads take nodes far from each other: neighbours are one node's children, good or bad together, and
+    // groups of those would leave three times the candidates)
+    const int first = (tid & 3) * (kRerankThreads / 4) + (((tid >> 2) + (tid & 3) * 8) & (kRerankThreads / 4 - 1));
+    unsigned long long best = 0ull;
+    for (int i = first; i < P; i += kRerankThreads) {
         unsigned long long c = 0;
         if (i < N) {
             c = s_code[i];
@@ -115,40 +122,60 @@ rerank_kernel(const int32_t* __restrict__ tree_token, const int32_t* __restrict_
         }
         s_key[i] = c;
         s_idx[i] = i;
+        best = c > best ? c : best;
+    }
+    // The bar, in the codes' upper halves: the `most`-th largest of the groups' maxima.  Groups of four threads up to
+    // 64 nodes wanted of 128 groups (60: about 81 nodes reach it), of two above.
+    __shared__ __align__(16) uint32_t s_top[kRerankThreads / 2];
+    __shared__ unsigned long long s_cand[kRerankCand];
+    __shared__ int s_cand_at[kRerankCand];
+    __shared__ uint32_t s_bar;
+    __shared__ int s_n;
+    const int width = most <= kRerankThreads / 8 ? 4 : 2;
+    uint32_t high = (uint32_t)(best >> 32);
+    high = max(high, __shfl_xor_sync(0xffffffffu, high, 1));
+    if (width == 4) high = max(high, __shfl_xor_sync(0xffffffffu, high, 2));
+    if (tid % width == 0) s_top[tid / width] = high;
+    if (tid == 0) s_bar = ~0u, s_n = 0;
+    __syncthreads();
+    {
+        int above = 0;
+        for (int j = (tid % width) * 4; j < kRerankThreads / width; j += 4 * width) {
+            const uint4 t = *reinterpret_cast<const uint4*>(s_top + j);
+            above += (t.x > high) + (t.y > high) + (t.z > high) + (t.w > high);
+        }
+        above += __shfl_xor_sync(0xffffffffu, above, 1);
+        if (width == 4) above += __shfl_xor_sync(0xffffffffu, above, 2);
+        const uint32_t low = __reduce_min_sync(0xffffffffu, above < most ? high : ~0u);
+        if ((tid & 31) == 0) atomicMin(&s_bar, low);
     }
     __syncthreads();
-    // order: effective value descending, index ascending
-    if (P <= kRerankThreads) {
-        // one element per thread (threads past P hold padding): exchanges closer than a warp go
-        // through shuffles, the others through a double-buffered shared-memory copy
-        __shared__ unsigned long long s_xk[2][kRerankThreads];
-        __shared__ int32_t s_xi[2][kRerankThreads];
-        unsigned long long key = tid < P ? s_key[tid] : 0ull;
-        int idx = tid;
-        int flip = 0;
-#pragma unroll 1
-        for (int size = 2; size <= kRerankThreads; size <<= 1) {
-#pragma unroll 1
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                unsigned long long ok;
-                int oi;
-                if (stride < 32) {
-                    ok = __shfl_xor_sync(0xffffffffu, key, stride);
-                    oi = __shfl_xor_sync(0xffffffffu, idx, stride);
-                } else {
-                    s_xk[flip][tid] = key;
-                    s_xi[flip][tid] = idx;
-                    __syncthreads();
-                    ok = s_xk[flip][tid ^ stride];
-                    oi = s_xi[flip][tid ^ stride];
-                    flip ^= 1;
-                }
-                const bool mine_first = key > ok || (key == ok && idx < oi);
-                const bool keep_first = ((tid & stride) == 0) == ((tid & size) == 0);
-                if (mine_first != keep_first) key = ok, idx = oi;
-            }
+    const uint32_t bar = s_bar;
+    if (high >= bar)
+        for (int i = first; i < N; i += kRerankThreads) {
+            const unsigned long long c = s_key[i];
+            if ((uint32_t)(c >> 32) < bar) continue;
+            const int at = atomicAdd(&s_n, 1);
+            if (at < kRerankCand) s_cand[at] = c, s_cand_at[at] = i;
         }
-        if (tid < most) s_flat[idx] = 0;
+    __syncthreads();
+    const int n = s_n;
+    // order: effective value descending, index ascending
+    if (n <= kRerankCand) {
+        for (int c0 = tid >> 2; c0 < (n + 7 & ~7); c0 += kRerankThreads / 4) {  // four threads a candidate
+            const unsigned long long mine = c0 < n ? s_cand[c0] : 0ull;
+            const int i = c0 < n ? s_cand_at[c0] : 0;
+            int place = 0, equal = 0;
+#pragma unroll 4
+            for (int j = tid & 3; j < n; j += 4) place += s_cand[j] > mine, equal += s_cand[j] == mine;
+            place += __shfl_xor_sync(0xffffffffu, place, 1);
+            equal += __shfl_xor_sync(0xffffffffu, equal, 1);
+            place += __shfl_xor_sync(0xffffffffu, place, 2);
+            equal += __shfl_xor_sync(0xffffffffu, equal, 2);
+            if (equal > 1 && place < most)  // ties: the lower index first
+                for (int j = 0; j < n; ++j) place += s_cand[j] == mine && s_cand_at[j] < i;
+            if ((tid & 3) == 0 && c0 < n && place < most) s_flat[i] = 0;
+        }
     } else {
         for (int size = 2; size <= P; size <<= 1) {
             for (int stride = size >> 1; stride > 0; stride >>= 1) {
@@ -285,7 +312,7 @@ static int rerank_launch(const int32_t* tree_token, const int32_t* tree_parent, 
     while (P < N) P <<= 1;
     const size_t dyn = (size_t)N * (sizeof(unsigned long long) + 2 * sizeof(int32_t)) +
                        (size_t)P * (sizeof(unsigned long long) + sizeof(int32_t));
-    if (dyn > 40 * 1024 &&
+    if (dyn > 32 * 1024 &&
         cudaFuncSetAttribute(rerank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
             cudaSuccess)
         return EAGLE2_ERR_CUDA;
