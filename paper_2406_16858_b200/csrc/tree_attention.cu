@@ -103,8 +103,12 @@ static void ring_of(AttnPlan* p, int d) {
 // blocks: which way is cheapest, by the items (128 rows x 128 keys) that one block goes through.  Combining a
 // cluster's partial rows costs about as much as two of them and, for 128 rows, one and a half more (measured: four
 // tiles of 128 rows are quicker on one block, 9.0 against 9.7 us per layer, of 40 rows on four blocks, 7.2 against
-// 8.2 us), so sequences of a few tiles stay on one block each.  Row blocks of 128 rows read the K/V tiles once more than those of 256, from L2, and give twice
-// the blocks.  Launches whose blocks would be long are left to the plans below, which put more SMs to work.
+// 8.2 us), so sequences of a few tiles stay on one block each.  Row blocks of 128 rows read the K/V tiles once more
+// than those of 256, from L2, and give twice the blocks.  Launches whose blocks would be long are left to the plans
+// below, which put more SMs to work; so are those that leave half of the SMs idle behind blocks of more than 11 tiles
+// (9000 / 12000 / 16000 keys, 8 KV heads, 40 rows: clusters 15.6 / 18.3 / 21.8 us per layer, partial rows 15.6 / 16.7 /
+// 20.8; 4 KV heads, 80 rows: 15.5 / 18.2 / 21.4 against 17.0 / 15.5 / 16.4.  With three quarters of the SMs busy the
+// clusters stay ahead: 2 x 8 KV heads, 40 rows, 12000 keys 24.3 against 24.9).
 // (Measured against partial rows and a merge launch, per layer: B = 1, 1024 keys, 8 KV heads of 4 query heads
 // 11.8 -> 10.5 us, 4096 keys 15.5 -> 14.8 us, 32 KV heads, 1024 keys 12.4 -> 12.0 us.)
 constexpr double kMaxItemsPerBlock = 24.0;
@@ -122,6 +126,7 @@ static bool single_wave_plan(int B, int m, int Hkv, int d, int tiles, AttnPlan* 
         }
     }
     if (!best_c) return false;
+    if (2 * groups * ((m + best_tok - 1) / best_tok) * best_c <= sm_count() && tiles > 11 * best_c) return false;
     p->cluster = best_c;
     p->per_tok = best_tok;
     p->per = best_tok * p->g;

@@ -27,3 +27,15 @@ def test_cluster_and_single_block_launches(m, Hq, Hkv, d, lens):
     n = 400
     samples = np.stack([rng.integers(0, B, n), rng.integers(0, Hq, n), rng.integers(0, m, n)], axis=1).astype(np.int32)
     _compare(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), samples=samples)
+
+
+@pytest.mark.parametrize("kv_len", [11254, 11255])
+def test_long_sequences_of_few_heads_are_split(kv_len):
+    """Either side of the line from which a cluster per KV head would leave too much of the device idle."""
+    m, Hq, Hkv, d = 10, 8, 2, 128
+    if kv_len > 11254:
+        assert e2.tree_attention_launches(1, m, Hq, Hkv, d, kv_len) == 2
+    q, kc, vc, off, kl, bits = _inputs(78, 1, m, Hq, Hkv, d, [kv_len])
+    rng = np.random.default_rng(6)
+    samples = np.stack([np.zeros(200, int), rng.integers(0, Hq, 200), rng.integers(0, m, 200)], axis=1).astype(np.int32)
+    _compare(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), samples=samples)
