@@ -36,6 +36,72 @@ __device__ __forceinline__ int count_above(const unsigned long long* keys, int n
 // 2^d for a whole d <= 0 (0 below the smallest normal number; NaN stays), exactly
 __device__ __forceinline__ float pow2_whole(float d) { return d >= -126.f ? __int_as_float(((int)d + 127) << 23) : d * 0.f; }
 
+// The node a row belongs to and its value; a frontier entry outside the level before is reported.
+__device__ __forceinline__ int parent_of_row(const int32_t* frontier, const double* tree_value, int b, int row, int k, int s, long long N,
+                                             int* parent, double* value) {
+    const long long prev_base = s >= 2 ? (long long)k + (long long)(s - 2) * k * k : 0;
+    const long long prev_count = s >= 2 ? (long long)k * k : k;
+    *parent = frontier[(long long)b * k + row];
+    if (*parent < prev_base || *parent >= prev_base + prev_count) {
+        *parent = (int)prev_base;
+        return EAGLE2_STATUS_BAD_TREE;
+    }
+    *value = tree_value[(long long)b * N + *parent];
+    return 0;
+}
+
+// Writes the children of a row whose k best keys (0: none) and log-sum-exp are known to the block; the block of a
+// sequence that does so last ranks the next frontier.
+__device__ __forceinline__ void hand_on_row(const unsigned long long* s_row, double lse, int parent, double parent_value, int b, int row, int k,
+                                            int n_s, long long N, long long base, int by_confidence, int32_t* tree_token,
+                                            int32_t* tree_parent, double* tree_value, int32_t* frontier, int* counters,
+                                            unsigned long long* codes, unsigned long long* s_code, int* s_flag, int status,
+                                            int32_t* d_status) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // A lane per child: what the row hands on is written by one warp, whose first lane announces it without another
+    // meeting of the block.
+    if (tid < k && s_row[tid]) {
+        const long long at = (long long)b * N + base + (long long)row * k + tid;
+        const double confidence = (double)key_value(s_row[tid]) - lse;  // log c_i
+        const double v = parent_value + confidence;
+        tree_token[at] = (int32_t)key_index(s_row[tid]);
+        tree_parent[at] = parent;
+        tree_value[at] = v;
+        // the next frontier is ranked by value, or by confidence alone in the ablation
+        if (n_s > 1) codes[((size_t)b * n_s + row) * k + tid] = order_code_f64(by_confidence ? confidence : v);
+    }
+    if (n_s == 1 && tid < k) frontier[(long long)b * k + tid] = (int32_t)(base + tid);  // a row's children are in order
+    if (status) raise_status(d_status, status);
+    if (n_s == 1) return;
+
+    // ---- last row of the sequence: the next frontier, by (value desc, index asc) ----------------------------
+    const int n_new = n_s * k;
+    if (warp == 0) {
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();  // cumulative: covers the stores of the warp's other lanes
+            *s_flag = atomicAdd(counters + b, 1) == n_s - 1;
+            if (*s_flag) counters[b] = 0;
+        }
+    }
+    __syncthreads();
+    if (!*s_flag) return;
+    __threadfence();
+    for (int i = tid; i < n_new; i += kRowThreads) s_code[i] = __ldcg(codes + (size_t)b * n_new + i);
+    __syncthreads();
+    for (int i = tid >> 1; i < (n_new + 15 & ~15); i += kRowThreads / 2) {  // two threads a candidate
+        const unsigned long long ci = i < n_new ? s_code[i] : 0ull;
+        int place = 0;
+#pragma unroll 8
+        for (int j = tid & 1; j < n_new; j += 2) {
+            const unsigned long long cj = s_code[j];
+            place += (cj > ci) || (cj == ci && j < i);
+        }
+        place += __shfl_xor_sync(0xffffffffu, place, 1);
+        if ((tid & 1) == 0 && i < n_new && place < k) frontier[(long long)b * k + place] = (int32_t)(base + i);
+    }
+}
+
 template <int NF, bool VEC>
 __global__ void __launch_bounds__(kRowThreads, NF == 16 ? 2 : 3)
 expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_stride, int V, int k, int D, int s, int n_s,
@@ -88,17 +154,7 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
     const long long base = s ? (long long)k + (long long)(s - 1) * k * k : 0;
     int parent = -1, status = 0;
     double parent_value = 0.0;
-    if (s && me == 0) {
-        parent = frontier[(long long)b * k + row];
-        const long long prev_base = s >= 2 ? (long long)k + (long long)(s - 2) * k * k : 0;
-        const long long prev_count = s >= 2 ? (long long)k * k : k;
-        if (parent < prev_base || parent >= prev_base + prev_count) {
-            status |= EAGLE2_STATUS_BAD_TREE;
-            parent = (int)prev_base;
-        } else {
-            parent_value = tree_value[(long long)b * N + parent];
-        }
-    }
+    if (s && me == 0) status |= parent_of_row(frontier, tree_value, b, row, k, s, N, &parent, &parent_value);
 
     // ---- maxima --------------------------------------------------------------------------
     float gm[NF];  // of four elements each
@@ -242,48 +298,116 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
             if ((tid & 1) == 0 && mine && rank < k) s_row[rank] = mine;
         }
     __syncthreads();
-    // A lane per child: what the row hands on is written by one warp, whose first lane announces it without another
-    // meeting of the block.
-    if (tid < k && s_row[tid]) {
-        const long long at = (long long)b * N + base + (long long)row * k + tid;
-        const double confidence = (double)key_value(s_row[tid]) - s_lse;  // log c_i
-        const double v = parent_value + confidence;
-        tree_token[at] = (int32_t)key_index(s_row[tid]);
-        tree_parent[at] = parent;
-        tree_value[at] = v;
-        // the next frontier is ranked by value, or by confidence alone in the ablation
-        if (n_s > 1) codes[((size_t)b * n_s + row) * k + tid] = order_code_f64(by_confidence ? confidence : v);
-    }
-    if (n_s == 1 && tid < k) frontier[(long long)b * k + tid] = (int32_t)(base + tid);  // a row's children are in order
-    if (status) raise_status(d_status, status);
-    if (n_s == 1) return;
+    hand_on_row(s_row, s_lse, parent, parent_value, b, row, k, n_s, N, base, by_confidence, tree_token, tree_parent, tree_value, frontier,
+                counters, codes, s_code, &s_flag, status, d_status);
+}
 
-    // ---- last row of the sequence: the next frontier, by (value desc, index asc) ----------------------------
-    const int n_new = n_s * k;
-    if (warp == 0) {
-        __syncwarp();
-        if (lane == 0) {
-            __threadfence();  // cumulative: covers the stores of the warp's other lanes
-            s_flag = atomicAdd(counters + b, 1) == n_s - 1;
-            if (s_flag) counters[b] = 0;
+// Finishes a step whose rows were ranked by another kernel in parts (the LM head that ranks its own logits: a part per
+// SM with the part's k best keys and its maximum and sum of exponentials).  A block per row; a row's `slots` places are
+// filled up to chunks_lo below split_row and chunks_hi from there on.  Keys of a row differ, but for the empty ones, 0.
+// What bounds it is the chain load - bar - candidates - row - ticket - frontier.
+constexpr int kPartKeysPerThread = 16;
+__global__ void __launch_bounds__(kRowThreads)
+expand_parts_kernel(int slots, int split_row, int chunks_lo, int chunks_hi, const double2* __restrict__ stats,
+                    const unsigned long long* __restrict__ keys, int k, int D, int s, int n_s, int32_t* __restrict__ tree_token,
+                    int32_t* __restrict__ tree_parent, double* __restrict__ tree_value, int32_t* __restrict__ frontier,
+                    int* __restrict__ counters, unsigned long long* __restrict__ codes, int32_t* d_status) {
+    __shared__ unsigned long long s_cand[kRowCand], s_code[EAGLE2_MAX_K * EAGLE2_MAX_K];
+    __shared__ unsigned long long s_row[EAGLE2_MAX_K], s_best[kRowWarps];
+    __shared__ __align__(16) uint32_t s_top[kRowGroups];
+    __shared__ float s_wmax[kRowWarps];
+    __shared__ double s_wsum[kRowWarps], s_lse;
+    __shared__ int s_n, s_flag;
+    chain_wait();
+    chain_release();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int line = blockIdx.x, row = line % n_s, b = line / n_s;
+    const int chunks = line < split_row ? chunks_lo : chunks_hi, n_in = chunks * k;
+    const unsigned long long* in = keys + (size_t)line * slots * k;
+    unsigned long long mine[kPartKeysPerThread], best = 0ull;
+#pragma unroll
+    for (int t = 0; t < kPartKeysPerThread; ++t) {
+        const int i = tid + t * kRowThreads;
+        mine[t] = i < n_in ? in[i] : 0ull;
+    }
+    const double2 part = tid < chunks ? stats[(size_t)line * slots + tid] : make_double2(-INFINITY, 0.0);
+    const long long N = nodes_of(k, D), base = s ? (long long)k + (long long)(s - 1) * k * k : 0;
+    int parent = -1, status = 0;
+    double parent_value = 0.0;
+    if (s) status |= parent_of_row(frontier, tree_value, b, row, k, s, N, &parent, &parent_value);
+    if (tid == 0) s_n = 0;
+    if (tid < k) s_row[tid] = 0ull;
+#pragma unroll
+    for (int t = 0; t < kPartKeysPerThread; ++t) best = mine[t] > best ? mine[t] : best;
+    uint32_t um = (uint32_t)(best >> 32);  // of eight threads, by value
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) um = max(um, __shfl_xor_sync(0xffffffffu, um, o));
+    if ((lane & 7) == 0) s_top[tid >> 3] = um;
+    const float wmax = warp_max_f32((float)part.x);  // (the maxima are 32-bit values)
+    if (lane == 0) s_wmax[warp] = wmax;
+    __syncthreads();
+
+    // the bar, as for a row of logits
+    uint32_t bar;
+    {
+        const uint32_t v = s_top[lane];
+        int above = 0;
+#pragma unroll
+        for (int j = 0; j < kRowGroups; j += 4) {
+            const uint4 t = *reinterpret_cast<const uint4*>(s_top + j);
+            above += (t.x > v) + (t.y > v) + (t.z > v) + (t.w > v);
         }
+        bar = __reduce_min_sync(0xffffffffu, above < k ? v : ~0u);
+    }
+    if ((uint32_t)(best >> 32) >= bar) {
+#pragma unroll
+        for (int t = 0; t < kPartKeysPerThread; ++t)
+            if (mine[t] && (uint32_t)(mine[t] >> 32) >= bar) {
+                const int at = atomicAdd(&s_n, 1);
+                if (at < kRowCand) s_cand[at] = mine[t];
+            }
+    }
+    // the parts' sums, in double
+    float m = s_wmax[0];
+#pragma unroll
+    for (int w = 1; w < kRowWarps; ++w) m = fmaxf(m, s_wmax[w]);
+    const double wsum = warp_sum_f64(part.x > -INFINITY ? part.y * exp(part.x - (double)m) : 0.0);
+    if (lane == 0) s_wsum[warp] = wsum;
+    __syncthreads();
+    int n = s_n;
+    if (n > kRowCand) {  // hundreds of equal logits: k times the largest key below the last one taken
+        unsigned long long last = ~0ull;
+        for (int r = 0; r < k; ++r) {
+            unsigned long long top = 0ull;
+#pragma unroll
+            for (int t = 0; t < kPartKeysPerThread; ++t) top = mine[t] < last && mine[t] > top ? mine[t] : top;
+            top = warp_max_u64(top);
+            if (lane == 0) s_best[warp] = top;
+            __syncthreads();
+            top = 0ull;
+#pragma unroll
+            for (int w = 0; w < kRowWarps; ++w) top = s_best[w] > top ? s_best[w] : top;
+            if (tid == 0) s_cand[r] = top;
+            last = top;
+            __syncthreads();
+        }
+        n = k;
+    }
+    if (tid == kRowThreads - 1) {
+        double sum = 0.0;
+#pragma unroll
+        for (int w = 0; w < kRowWarps; ++w) sum += s_wsum[w];
+        s_lse = (double)m + log(sum);
+        if (!(m > -INFINITY)) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
+    }
+    for (int i = tid >> 2; i < (n + 7 & ~7); i += kRowThreads / 4) {  // four threads share a key's comparisons
+        const unsigned long long key = i < n ? s_cand[i] : 0ull;
+        const int rank = count_above<4>(s_cand, n, key);
+        if ((tid & 3) == 0 && rank < k && key) s_row[rank] = key;
     }
     __syncthreads();
-    if (!s_flag) return;
-    __threadfence();
-    for (int i = tid; i < n_new; i += kRowThreads) s_code[i] = __ldcg(codes + (size_t)b * n_new + i);
-    __syncthreads();
-    for (int i = tid >> 1; i < (n_new + 15 & ~15); i += kRowThreads / 2) {  // two threads a candidate
-        const unsigned long long ci = i < n_new ? s_code[i] : 0ull;
-        int place = 0;
-#pragma unroll 8
-        for (int j = tid & 1; j < n_new; j += 2) {
-            const unsigned long long cj = s_code[j];
-            place += (cj > ci) || (cj == ci && j < i);
-        }
-        place += __shfl_xor_sync(0xffffffffu, place, 1);
-        if ((tid & 1) == 0 && i < n_new && place < k) frontier[(long long)b * k + place] = (int32_t)(base + i);
-    }
+    hand_on_row(s_row, s_lse, parent, parent_value, b, row, k, n_s, N, base, 0, tree_token, tree_parent, tree_value, frontier, counters,
+                codes, s_code, &s_flag, status, d_status);
 }
 
 // Slices: the shortest (most blocks) that keep the launch on the device at once; else the longest.

@@ -7,8 +7,7 @@
 // shared memory, and scanner threads - one per feature row - fold them into the row's running
 // maximum, sum of exponentials and k best (value, token) keys while the tensor pipe already works on
 // the next tile (two accumulators).  When a block has walked its tiles it writes one partial per row,
-// in the expansion's own workspace layout; a row-merge launch folds a row's partials into one, and the
-// expansion's merge launch finishes the step from those.
+// in the expansion's own workspace layout, and a launch of a block per row finishes the step from those.
 //
 // The vocabulary is the M side of tcgen05.mma (128 entries per block) and the feature rows are its
 // N side, N = the rows of the pass rounded up to 16: the tensor work is proportional to the rows
@@ -37,10 +36,9 @@ namespace eagle2 {
 size_t expand_partials_bytes(int B, int n_s, int chunks, int k);
 bool expand_partials_layout(int B, int n_s, int chunks, int k, void* ws, size_t ws_bytes, double2** stats,
                             unsigned long long** keys);
-int launch_expand_merge(int B, int V, int k, int D, int s, int chunks, int32_t* tree_token, int32_t* tree_parent,
-                        double* tree_value, int32_t* frontier, void* ws, int32_t* d_status, cudaStream_t stream);
-int launch_expand_row_merge(int B, int n_s, int slots, long long split_row, int chunks_lo, int chunks_hi, int k, void* ws,
-                            void* ws_rows, cudaStream_t stream);
+int launch_expand_parts(int B, int k, int D, int s, int slots, long long split_row, int chunks_lo, int chunks_hi, int32_t* tree_token,
+                        int32_t* tree_parent, double* tree_value, int32_t* frontier, void* ws, void* ws_codes, int32_t* d_status,
+                        cudaStream_t stream);
 
 constexpr int kFzWriterWarps = 4, kFzScanWarps = 8;
 constexpr int kFzThreads = (2 + kFzWriterWarps + kFzScanWarps) * 32;
@@ -429,7 +427,7 @@ static int fz_units(int V, bool pair) {
     const int tile_v = pair ? 2 * kFzTileV : kFzTileV;
     const int n_tiles = (V + tile_v - 1) / tile_v;
     int units = pair ? sm_count() / 2 : sm_count();
-    if (units > (pair ? 80 : 160)) units = pair ? 80 : 160;  // never more partials than the row merge holds
+    if (units > (pair ? 80 : 160)) units = pair ? 80 : 160;  // never more partials than the finishing launch holds
     if (units < 1) units = 1;
     return n_tiles < units ? n_tiles : units;
 }
@@ -459,7 +457,7 @@ static FzPasses fz_passes(long long rows, int V) {
     return p;
 }
 
-// Two areas: the producers' partials (`slots` per row), then the rows' merged partials (one per row).
+// Two areas: the producers' partials (`slots` per row), then the codes of the rows' children.
 static size_t fz_ws_bytes(int B, int n_s, int V, int k, size_t* second) {
     const FzPasses p = fz_passes((long long)B * n_s, V);
     const size_t first = round_up(expand_partials_bytes(B, n_s, p.slots, k), kWsAlign);
@@ -547,8 +545,7 @@ extern "C" int eagle2_lm_head_expand(const void* hidden, const void* weight, int
                                             stats, keys, d_status, st);
     if (rc != EAGLE2_OK) return rc;
     const int rest_producers = p.rest_pair ? p.producers_pair : p.producers_single;
-    rc = launch_expand_row_merge(B, n_s, p.slots, (long long)p.full * kFzMaxRows, p.full ? p.producers_pair : rest_producers,
-                                 p.rest ? rest_producers : p.producers_pair, k, ws, ws_rows, st);
-    if (rc != EAGLE2_OK) return rc;
-    return launch_expand_merge(B, V, k, D, s, 1, tree_token, tree_parent, tree_value, frontier, ws_rows, d_status, st);
+    return launch_expand_parts(B, k, D, s, p.slots, (long long)p.full * kFzMaxRows, p.full ? p.producers_pair : rest_producers,
+                               p.rest ? rest_producers : p.producers_pair, tree_token, tree_parent, tree_value, frontier, ws, ws_rows,
+                               d_status, st);
 }
