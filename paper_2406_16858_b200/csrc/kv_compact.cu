@@ -4,6 +4,11 @@
 // A thread owns one 16-byte column segment of one (layer, K|V, sequence): it loads that segment of
 // every accepted row first and stores afterwards, so the in-place move is safe although sources and
 // destinations overlap (destination j never exceeds source acc_path[j]).
+//
+// Caches of one layer or so (two segments a thread): one launch, a block per sequence, which advances the length itself.
+// It is bound by its launch and two trips to memory; the second launch was 0.7 us of a small cycle's 34.  More segments:
+// the move over the whole device, then a launch that advances the lengths (a cluster of blocks per sequence that meet
+// before the update was no faster at 32 layers: 539.5 against 540.3 us per cycle).
 #include "common.cuh"
 
 namespace eagle2 {
@@ -22,6 +27,41 @@ __device__ __forceinline__ bool path_is_valid(const int32_t* path, int len, int 
     return true;
 }
 
+// One column segment of one layer's K or V rows behind `base`.
+__device__ __forceinline__ void move_segment(uint4* base, const int32_t* path, int len, int segs) {
+    uint4 held[kCompactMaxDepth];
+#pragma unroll
+    for (int j = 0; j < kCompactMaxDepth; ++j)
+        if (j < len) held[j] = base[(long long)path[j] * segs];
+#pragma unroll
+    for (int j = 0; j < kCompactMaxDepth; ++j)
+        if (j < len && path[j] != j) base[(long long)j * segs] = held[j];
+}
+
+constexpr int kCompactBlockThreads = 512;
+__global__ void __launch_bounds__(kCompactBlockThreads)
+kv_compact_block_kernel(void* const* __restrict__ k_layers, void* const* __restrict__ v_layers,
+                        const int64_t* __restrict__ kv_off, int32_t* __restrict__ kv_len,
+                        const int32_t* __restrict__ acc_path, const int32_t* __restrict__ acc_len, int m, int D, int segs,
+                        int items, int32_t* d_status) {
+    const int b = blockIdx.x;
+    chain_wait();  // (no early release of the dependents: they may read the lengths before they wait)
+    const int len = acc_len[b], before = kv_len[b];
+    const int32_t* path = acc_path + (long long)b * D;
+    const bool valid = path_is_valid(path, len, D, m);
+    if (valid && len > 0)
+        for (int i = threadIdx.x; i < items; i += kCompactBlockThreads) {
+            const int part = i / segs;
+            uint4* rows = reinterpret_cast<uint4*>(part & 1 ? v_layers[part >> 1] : k_layers[part >> 1]);
+            move_segment(rows + (kv_off[b] + before) * (long long)segs + (i - part * segs), path, len, segs);
+        }
+    __syncthreads();  // every thread has read the old length
+    if (threadIdx.x == 0) {
+        if (valid) kv_len[b] = before + len;
+        else raise_status(d_status, EAGLE2_STATUS_BAD_TREE);
+    }
+}
+
 __global__ void __launch_bounds__(kCompactThreads)
 kv_compact_kernel(void* const* __restrict__ k_layers, void* const* __restrict__ v_layers,
                   const int64_t* __restrict__ kv_off, const int32_t* __restrict__ kv_len,
@@ -37,13 +77,7 @@ kv_compact_kernel(void* const* __restrict__ k_layers, void* const* __restrict__ 
     if (seg >= segs || len == 0 || !path_is_valid(path, len, D, m)) return;
     uint4* base = reinterpret_cast<uint4*>(which ? v_layers[layer] : k_layers[layer]) +
                   (kv_off[b] + kv_len[b]) * (long long)segs + seg;
-    uint4 held[kCompactMaxDepth];
-#pragma unroll
-    for (int j = 0; j < kCompactMaxDepth; ++j)
-        if (j < len) held[j] = base[(long long)path[j] * segs];
-#pragma unroll
-    for (int j = 0; j < kCompactMaxDepth; ++j)
-        if (j < len && path[j] != j) base[(long long)j * segs] = held[j];
+    move_segment(base, path, len, segs);
 }
 
 // Runs after the move (same stream): every block of the move kernel has read the old lengths.
@@ -82,6 +116,10 @@ extern "C" int eagle2_kv_compact(void* const* k_layers, void* const* v_layers, i
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const int segs = (int)(row_bytes / 16);
     const int seg_blocks = (segs + kCompactThreads - 1) / kCompactThreads;
+    const long long items = 2LL * n_layers * segs;
+    if (items <= 2 * kCompactBlockThreads)
+        return launch_chained(kv_compact_block_kernel, dim3((unsigned)B), dim3(kCompactBlockThreads), 0, st, 1, k_layers, v_layers,
+                              kv_off, kv_len, acc_path, acc_len, m, D, segs, (int)items, d_status);
     if (n_layers > 0) {
         if ((long long)B * seg_blocks > 0x7fffffffLL) return EAGLE2_ERR_SHAPE;
         dim3 grid((unsigned)(B * seg_blocks), (unsigned)(n_layers * 2));

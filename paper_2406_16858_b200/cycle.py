@@ -105,7 +105,8 @@ class CycleBuffers:
         s = self.shape
         per_layer = e2.tree_attention_launches(s.B, s.m, s.Hq, s.Hkv, s.d, s.max_kv_len)
         accept = 2 if s.temperature > 0 and s.V > 131072 else 1  # larger vocabularies: chains, then the walk
-        return s.D + 1 + s.n_layers * per_layer + accept + 2
+        compact = 1 if s.n_layers * 2 * s.Hkv * s.d * 2 // 16 <= 1024 else 2  # few segments: one block per sequence
+        return s.D + 1 + s.n_layers * per_layer + accept + compact
 
 
 def enqueue_cycle(buf: CycleBuffers, draft_rows, target_logits, u_accept, u_bonus, q_layers, k_layers,
