@@ -261,15 +261,17 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         }
         bad |= !(sum_p > 0.0) | (with_q && !(sum_q > 0.0));
         const float c_p = (float)(1.0 / sum_p), c_q = with_q ? (float)(1.0 / sum_q) : 0.f;
-        // what this warp's exponentials have to be multiplied with to be probabilities
-        const float fp = exp2_approx(rp - gp) * c_p, fq = FULLQ ? exp2_approx(rq - gq) * c_q : 0.f;
+        // What this warp's exponentials have to be multiplied with to be probabilities.  A warp without mass (beyond
+        // the vocabulary, or all its tokens at -inf) has no reference to compare with the row's: its factor is 0.
+        const float fp = mp > -INFINITY ? exp2_approx(rp - gp) * c_p : 0.f;
+        const float fq = FULLQ && mq > -INFINITY ? exp2_approx(rq - gq) * c_q : 0.f;
         const float q_to_p = fp > 0.f ? fminf(fq / fp, 1e30f) : 0.f;  // q in units of the warp's p
         float kid_p = 0.f, kid_q = 0.f;
         if (lane < nc) {
             if (kid_tok >= 0 && kid_tok < V) {
                 const WalkChild c = s_kid[node & 1][lane];
-                kid_p = c.ep * (exp2_approx(c.mp - gp) * c_p);
-                if (FULLQ) kid_q = c.eq * (exp2_approx(c.mq - gq) * c_q);
+                kid_p = c.ep > 0.f ? c.ep * (exp2_approx(c.mp - gp) * c_p) : 0.f;
+                if (FULLQ) kid_q = c.eq > 0.f ? c.eq * (exp2_approx(c.mq - gq) * c_q) : 0.f;
             } else {
                 bad = 1;
             }
