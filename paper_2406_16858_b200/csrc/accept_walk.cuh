@@ -28,11 +28,11 @@ constexpr int kWalkWarps = kWalkThreads / kWarp;
 constexpr int kWalkMaxCluster = 8;
 constexpr int kWalkEntries = kWalkWarps * kWalkMaxCluster;  // one per warp of the cluster
 
-struct WalkSums {  // a warp's contribution to the softmax sums of a node
+struct WalkSums {  // a warp's contribution to the softmax sums of a node, and its largest logits
     double sum_p, sum_q;
     float max_p, max_q;
 };
-struct WalkChild {  // a child's token as its holder has it: unnormalised, with the holder's maxima
+struct WalkChild {  // a child's token as its holder has it: unnormalised, with the largest logits of the holder's warp
     float ep, eq, mp, mq;
 };
 
@@ -44,6 +44,37 @@ __device__ __forceinline__ float exp2_approx(float x) {  // 2 ulp; -inf gives 0
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// The exponent of 2 that a warp's exponentials are taken relative to, from its largest logit; to_log2: log2(e) / T.
+// Far from zero (up to the largest numbers a float holds: masks often are its lowest) that product overflows or is
+// rounded by more than the exponents' own differences, so that there differences are taken before the product.
+constexpr float kWalkFar = 4194304.f;  // 2^22: the product's rounding is below 1/4
+__device__ __forceinline__ bool walk_near(float max_logit, float to_log2) { return fabsf(max_logit * to_log2) < kWalkFar; }
+__device__ __forceinline__ float walk_reference(float max_logit, float to_log2) { return max_logit * to_log2; }
+// Factor from one warp's reference to that of the warp with the row's largest logit (0 for a warp without mass).
+__device__ __forceinline__ float walk_factor(float max_logit, float row_max, float to_log2) {
+    const bool near_w = walk_near(max_logit, to_log2), near_r = walk_near(row_max, to_log2);
+    float d;
+    if (near_w && near_r) d = walk_reference(max_logit, to_log2) - walk_reference(row_max, to_log2);
+    else if (near_w) d = fmaf(-row_max, to_log2, walk_reference(max_logit, to_log2));
+    else if (near_r) d = fmaf(max_logit, to_log2, -walk_reference(row_max, to_log2));
+    else d = max_logit == row_max ? 0.f : (max_logit - row_max) * to_log2;
+    return exp2_approx(d);
+}
+// A thread's N logits, in place, to exponentials relative to its warp's reference; their sum (in two chains).
+template <int N>
+__device__ __forceinline__ float walk_exponentials(float (&x)[N], float max_logit, float to_log2) {
+    float t[2] = {0.f, 0.f};
+    if (walk_near(max_logit, to_log2)) {
+        const float ref = walk_reference(max_logit, to_log2);
+#pragma unroll
+        for (int j = 0; j < N; ++j) x[j] = exp2_approx(fmaf(x[j], to_log2, -ref)), t[j & 1] += x[j];
+    } else {
+        const float at = max_logit > -INFINITY ? max_logit : 0.f;  // (-inf less -inf is not a number)
+#pragma unroll
+        for (int j = 0; j < N; ++j) x[j] = exp2_approx((x[j] - at) * to_log2), t[j & 1] += x[j];
+    }
+    return t[0] + t[1];
 }
 // Probability mass in units of 2^-54: integer sums do not depend on their order, and two additions over the
 // warp's lanes (27 bits each) take a quarter of the time of five shuffled steps in 64-bit floating point.
@@ -205,24 +236,18 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         }
         mp = warp_max_f32(mp);
         if (FULLQ) mq = warp_max_f32(mq);
-        const float rp = mp > -INFINITY ? mp * to_log2 : 0.f, rq = mq > -INFINITY ? mq * to_log2 : 0.f;
-        float tp[2] = {0.f, 0.f}, tq[2] = {0.f, 0.f};
-#pragma unroll
-        for (int j = 0; j < NE; ++j) {
-            p[j] = exp2_approx(fmaf(p[j], to_log2, -rp));
-            tp[j & 1] += p[j];
-            if (FULLQ) q[j] = exp2_approx(fmaf(q[j], to_log2, -rq)), tq[j & 1] += q[j];
-        }
-        const double wp = warp_sum_f64((double)(tp[0] + tp[1])), wq = with_q ? warp_sum_f64((double)(tq[0] + tq[1])) : 0.0;
+        const double wp = warp_sum_f64((double)walk_exponentials<NE>(p, mp, to_log2));
+        double wq = 0.0;
+        if (FULLQ && with_q) wq = warp_sum_f64((double)walk_exponentials<FULLQ ? NE : 1>(q, mq, to_log2));
         if (lane < cs) {
             WalkSums* dst = cluster.map_shared_rank(&s_sums[node & 1][me * kWalkWarps + warp], lane);
-            dst->sum_p = wp, dst->sum_q = wq, dst->max_p = rp, dst->max_q = rq;
+            dst->sum_p = wp, dst->sum_q = wq, dst->max_p = mp, dst->max_q = mq;
         }
         for (int i = 0; i < nc; ++i) {  // the holder of a child's token tells every block
             const int t = __shfl_sync(0xffffffffu, kid_tok, i);
             const int j = element_of(t);
             if (j >= 0 && t < V) {
-                WalkChild c = {0.f, 0.f, rp, rq};
+                WalkChild c = {0.f, 0.f, mp, mq};
 #pragma unroll
                 for (int u = 0; u < NE; ++u)
                     if (u == j) {
@@ -233,7 +258,7 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
             }
         }
         meet();
-        // (a warp without mass has sum 0: its reference does not count; a NaN or +inf logit makes its sum NaN)
+        // (a warp without mass has sum 0: its largest logit does not count; a NaN or +inf logit makes its sum NaN)
         constexpr int kPerLane = kWalkEntries / 32;
         double gs_p[kPerLane], gs_q[kPerLane];
         float gm_p[kPerLane], gm_q[kPerLane], gp = -INFINITY, gq = -INFINITY;
@@ -251,27 +276,29 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         double sum_p = 0.0, sum_q = 0.0;
 #pragma unroll
         for (int u = 0; u < kPerLane; ++u) {
-            if (gs_p[u] != 0.0) sum_p += gs_p[u] * (double)exp2_approx(gm_p[u] - gp);
-            if (FULLQ && gs_q[u] != 0.0) sum_q += gs_q[u] * (double)exp2_approx(gm_q[u] - gq);
+            if (gs_p[u] != 0.0) sum_p += gs_p[u] * (double)walk_factor(gm_p[u], gp, to_log2);
+            if (FULLQ && gs_q[u] != 0.0) sum_q += gs_q[u] * (double)walk_factor(gm_q[u], gq, to_log2);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             sum_p += __shfl_xor_sync(0xffffffffu, sum_p, o);
             if (FULLQ) sum_q += __shfl_xor_sync(0xffffffffu, sum_q, o);
         }
-        bad |= !(sum_p > 0.0) | (with_q && !(sum_q > 0.0));
+        // (a row whose largest logit overflows when divided by the temperature counts as one that was not finite)
+        bad |= !(sum_p > 0.0) | !(fabsf(gp * inv_t) < INFINITY);
+        if (FULLQ && with_q) bad |= !(sum_q > 0.0) | !(fabsf(gq * inv_t) < INFINITY);
         const float c_p = (float)(1.0 / sum_p), c_q = with_q ? (float)(1.0 / sum_q) : 0.f;
         // What this warp's exponentials have to be multiplied with to be probabilities.  A warp without mass (beyond
         // the vocabulary, or all its tokens at -inf) has no reference to compare with the row's: its factor is 0.
-        const float fp = mp > -INFINITY ? exp2_approx(rp - gp) * c_p : 0.f;
-        const float fq = FULLQ && mq > -INFINITY ? exp2_approx(rq - gq) * c_q : 0.f;
+        const float fp = mp > -INFINITY ? walk_factor(mp, gp, to_log2) * c_p : 0.f;
+        const float fq = FULLQ && mq > -INFINITY ? walk_factor(mq, gq, to_log2) * c_q : 0.f;
         const float q_to_p = fp > 0.f ? fminf(fq / fp, 1e30f) : 0.f;  // q in units of the warp's p
         float kid_p = 0.f, kid_q = 0.f;
         if (lane < nc) {
             if (kid_tok >= 0 && kid_tok < V) {
                 const WalkChild c = s_kid[node & 1][lane];
-                kid_p = c.ep > 0.f ? c.ep * (exp2_approx(c.mp - gp) * c_p) : 0.f;
-                if (FULLQ) kid_q = c.eq > 0.f ? c.eq * (exp2_approx(c.mq - gq) * c_q) : 0.f;
+                kid_p = c.ep > 0.f ? c.ep * (walk_factor(c.mp, gp, to_log2) * c_p) : 0.f;
+                if (FULLQ) kid_q = c.eq > 0.f ? c.eq * (walk_factor(c.mq, gq, to_log2) * c_q) : 0.f;
             } else {
                 bad = 1;
             }

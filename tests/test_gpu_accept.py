@@ -32,10 +32,13 @@ def _pipeline(cfg, seed):
 
 
 def _compare(cfg, draft, sel, target, ua, ub, temperature, point_mass=False, t_stride=None,
-             d_stride=None):
+             d_stride=None, on_device=None):
+    """on_device: other logits of the same softmax, for the device alone."""
     d_arg = None if (temperature == 0 or point_mass) else draft
     want = ref.accept(target, d_arg, sel, cfg.V, cfg.k, cfg.D, cfg.m, temperature, ua, ub,
                       t_stride=t_stride, d_stride=d_stride, debug=temperature > 0)
+    if on_device is not None:
+        target, d_arg = on_device(target), None if d_arg is None else on_device(d_arg)
     alen, apath, bonus, st = gpu_accept(target, d_arg, sel.index, sel.parent, sel.token, sel.n_sel,
                                         cfg.V, cfg.k, cfg.D, cfg.m, temperature, ua, ub,
                                         t_stride=t_stride, d_stride=d_stride)

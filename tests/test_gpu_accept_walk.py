@@ -2,7 +2,9 @@
 import numpy as np
 import pytest
 
+from oracle import ref
 from test_gpu_accept import _compare, _pipeline
+from workloads import generators as gen
 from workloads import get_config
 
 pytestmark = pytest.mark.gpu
@@ -34,3 +36,40 @@ def test_logits_far_below_zero(V, B, temperature, shift):
     target, draft = target + np.float32(shift), draft + np.float32(shift)
     _compare(cfg, draft, sel, target, ua, ub, temperature)
     _compare(cfg, draft, sel, target, ua, ub, temperature, point_mass=True)
+
+
+@pytest.mark.parametrize("V,B", [(33, 8), (2052, 8), (32000, 4), (131071, 2)])
+@pytest.mark.parametrize("kind", ["masked", "mostly_masked", "flat", "one_huge", "far_below", "far_above"])
+def test_logits_of_any_size(V, B, kind):
+    """Rows whose tokens are excluded by the lowest number a float holds, whole warps of them, and rows far from zero."""
+    cfg = get_config("tiny", V=V, B=B, k=4, D=3, m=16)
+    rng = np.random.default_rng(V)
+    lowest, highest = np.finfo(np.float32).min, np.finfo(np.float32).max
+    at = int(rng.integers(0, V - 8))
+    out = rng.random(V) < 0.9  # tokens excluded in every row
+    out[at:at + 8] = False
+    if kind == "masked":  # a run of tokens and a few others stay
+        out[:] = True
+        out[at:at + 8 + V // 50] = False
+        out[rng.integers(0, V, 8)] = False
+
+    def change(rows):
+        if kind == "one_huge":
+            rows[..., at] = highest
+        elif kind.startswith("far"):  # steps of 1 to 4 between neighbouring numbers
+            rows[:] = np.round(rows) * 4 + np.float32((-1 if kind == "far_below" else 1) * 2.0 ** 24)
+        elif kind == "flat":  # nothing but the mask: every token is as likely as any other (to the oracle, of logits 0)
+            rows[:] = 0.0
+        else:
+            rows[..., out] = lowest
+        return rows
+
+    draft = change(gen.draft_rows(cfg, 14))
+    tree = ref.build_tree(draft, V, cfg.k, cfg.D)
+    sel = ref.rerank(tree.token, tree.parent, tree.value, cfg.k, cfg.D, cfg.m)
+    target = change(gen.target_rows(cfg, 14, draft, tree.parent, sel.index))
+    ua, ub = gen.uniforms(cfg, 14)
+    on_device = (lambda rows: np.full_like(rows, lowest)) if kind == "flat" else None
+    for temperature in (1.0, 1.5):
+        for point_mass in (False, True):
+            _compare(cfg, draft, sel, target, ua, ub, temperature, point_mass=point_mass, on_device=on_device)
