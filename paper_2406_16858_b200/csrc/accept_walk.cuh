@@ -19,6 +19,8 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace eagle2 {
@@ -46,34 +48,40 @@ __device__ __forceinline__ float exp2_approx(float x) {  // 2 ulp; -inf gives 0
     return y;
 }
 // The exponent of 2 that a warp's exponentials are taken relative to, from its largest logit; to_log2: log2(e) / T.
+// (Rounded on its own: the tokens' exponents and the factors between warps have to mean the same number.)
 // Far from zero (up to the largest numbers a float holds: masks often are its lowest) that product overflows or is
 // rounded by more than the exponents' own differences, so that there differences are taken before the product.
-constexpr float kWalkFar = 4194304.f;  // 2^22: the product's rounding is below 1/4
-__device__ __forceinline__ bool walk_near(float max_logit, float to_log2) { return fabsf(max_logit * to_log2) < kWalkFar; }
-__device__ __forceinline__ float walk_reference(float max_logit, float to_log2) { return max_logit * to_log2; }
-// Factor from one warp's reference to that of the warp with the row's largest logit (0 for a warp without mass).
+constexpr float kWalkFar = 4194304.f;  // 2^22: the product's rounding is at most 1/4
+__device__ __forceinline__ float walk_reference(float max_logit, float to_log2) {
+    return max_logit > -INFINITY ? __fmul_rn(max_logit, to_log2) : 0.f;  // (a warp without mass: any number does)
+}
+__device__ __forceinline__ bool walk_near(float max_logit, float to_log2) { return fabsf(walk_reference(max_logit, to_log2)) < kWalkFar; }
+// Factor from one warp's reference to that of the warp with the row's largest logit; FAR: one of the row's is far (rare:
+// kept out of the way of the code that a launch runs through once and cold).
+static __device__ __noinline__ float walk_factor_far(float max_logit, float row_max, float to_log2) {
+    const float ref_w = walk_reference(max_logit, to_log2), ref_r = walk_reference(row_max, to_log2);
+    const bool near_w = fabsf(ref_w) < kWalkFar, near_r = fabsf(ref_r) < kWalkFar;
+    if (near_w && near_r) return exp2_approx(ref_w - ref_r);
+    if (near_w) return exp2_approx(fmaf(-row_max, to_log2, ref_w));
+    if (near_r) return exp2_approx(fmaf(max_logit, to_log2, -ref_r));
+    return max_logit == row_max ? 1.f : exp2_approx((max_logit - row_max) * to_log2);
+}
+template <bool FAR>
 __device__ __forceinline__ float walk_factor(float max_logit, float row_max, float to_log2) {
-    const bool near_w = walk_near(max_logit, to_log2), near_r = walk_near(row_max, to_log2);
-    float d;
-    if (near_w && near_r) d = walk_reference(max_logit, to_log2) - walk_reference(row_max, to_log2);
-    else if (near_w) d = fmaf(-row_max, to_log2, walk_reference(max_logit, to_log2));
-    else if (near_r) d = fmaf(max_logit, to_log2, -walk_reference(row_max, to_log2));
-    else d = max_logit == row_max ? 0.f : (max_logit - row_max) * to_log2;
-    return exp2_approx(d);
+    if (FAR) return walk_factor_far(max_logit, row_max, to_log2);
+    return exp2_approx(walk_reference(max_logit, to_log2) - walk_reference(row_max, to_log2));
 }
 // A thread's N logits, in place, to exponentials relative to its warp's reference; their sum (in two chains).
 template <int N>
 __device__ __forceinline__ float walk_exponentials(float (&x)[N], float max_logit, float to_log2) {
-    float t[2] = {0.f, 0.f};
-    if (walk_near(max_logit, to_log2)) {
-        const float ref = walk_reference(max_logit, to_log2);
+    float t[2] = {0.f, 0.f}, ref = walk_reference(max_logit, to_log2);
+    if (__builtin_expect(!walk_near(max_logit, to_log2), 0)) {
+        ref = 0.f;
 #pragma unroll
-        for (int j = 0; j < N; ++j) x[j] = exp2_approx(fmaf(x[j], to_log2, -ref)), t[j & 1] += x[j];
-    } else {
-        const float at = max_logit > -INFINITY ? max_logit : 0.f;  // (-inf less -inf is not a number)
-#pragma unroll
-        for (int j = 0; j < N; ++j) x[j] = exp2_approx((x[j] - at) * to_log2), t[j & 1] += x[j];
+        for (int j = 0; j < N; ++j) x[j] -= max_logit;
     }
+#pragma unroll
+    for (int j = 0; j < N; ++j) x[j] = exp2_approx(fmaf(x[j], to_log2, -ref)), t[j & 1] += x[j];
     return t[0] + t[1];
 }
 // Probability mass in units of 2^-54: integer sums do not depend on their order, and two additions over the
@@ -262,6 +270,7 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         constexpr int kPerLane = kWalkEntries / 32;
         double gs_p[kPerLane], gs_q[kPerLane];
         float gm_p[kPerLane], gm_q[kPerLane], gp = -INFINITY, gq = -INFINITY;
+        bool far = false;
 #pragma unroll
         for (int u = 0; u < kPerLane; ++u) {
             const int i = lane + 32 * u;
@@ -270,15 +279,34 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
             gs_p[u] = w.sum_p, gs_q[u] = w.sum_q, gm_p[u] = w.max_p, gm_q[u] = w.max_q;
             if (w.sum_p != 0.0) gp = fmaxf(gp, w.max_p);
             if (FULLQ && w.sum_q != 0.0) gq = fmaxf(gq, w.max_q);
+            far |= !walk_near(w.max_p, to_log2) | (FULLQ && !walk_near(w.max_q, to_log2));
         }
+        far = __any_sync(0xffffffffu, far);
         gp = order_decode(__reduce_max_sync(0xffffffffu, order_code(gp)));
         if (FULLQ) gq = order_decode(__reduce_max_sync(0xffffffffu, order_code(gq)));
         double sum_p = 0.0, sum_q = 0.0;
-#pragma unroll
-        for (int u = 0; u < kPerLane; ++u) {
-            if (gs_p[u] != 0.0) sum_p += gs_p[u] * (double)walk_factor(gm_p[u], gp, to_log2);
-            if (FULLQ && gs_q[u] != 0.0) sum_q += gs_q[u] * (double)walk_factor(gm_q[u], gq, to_log2);
+        // Factors: of this warp's exponentials, of the child's in this lane (0 for a warp without mass, which has no
+        // largest logit, and for a token without any).
+        float fp = 0.f, fq = 0.f, kid_p = 0.f, kid_q = 0.f;
+        WalkChild child = {0.f, 0.f, 0.f, 0.f};
+        if (lane < nc) {
+            if (kid_tok >= 0 && kid_tok < V) child = s_kid[node & 1][lane];
+            else bad = 1;
         }
+        auto weigh = [&](auto far_tag) {
+            constexpr bool FAR = decltype(far_tag)::value;
+#pragma unroll
+            for (int u = 0; u < kPerLane; ++u) {
+                if (gs_p[u] != 0.0) sum_p += gs_p[u] * (double)walk_factor<FAR>(gm_p[u], gp, to_log2);
+                if (FULLQ && gs_q[u] != 0.0) sum_q += gs_q[u] * (double)walk_factor<FAR>(gm_q[u], gq, to_log2);
+            }
+            if (mp > -INFINITY) fp = walk_factor<FAR>(mp, gp, to_log2);
+            if (FULLQ && mq > -INFINITY) fq = walk_factor<FAR>(mq, gq, to_log2);
+            if (child.ep > 0.f) kid_p = walk_factor<FAR>(child.mp, gp, to_log2);
+            if (FULLQ && child.eq > 0.f) kid_q = walk_factor<FAR>(child.mq, gq, to_log2);
+        };
+        if (__builtin_expect(far, 0)) weigh(std::true_type{});
+        else weigh(std::false_type{});
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             sum_p += __shfl_xor_sync(0xffffffffu, sum_p, o);
@@ -288,21 +316,11 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         bad |= !(sum_p > 0.0) | !(fabsf(gp * inv_t) < INFINITY);
         if (FULLQ && with_q) bad |= !(sum_q > 0.0) | !(fabsf(gq * inv_t) < INFINITY);
         const float c_p = (float)(1.0 / sum_p), c_q = with_q ? (float)(1.0 / sum_q) : 0.f;
-        // What this warp's exponentials have to be multiplied with to be probabilities.  A warp without mass (beyond
-        // the vocabulary, or all its tokens at -inf) has no reference to compare with the row's: its factor is 0.
-        const float fp = mp > -INFINITY ? walk_factor(mp, gp, to_log2) * c_p : 0.f;
-        const float fq = FULLQ && mq > -INFINITY ? walk_factor(mq, gq, to_log2) * c_q : 0.f;
+        // what this warp's exponentials have to be multiplied with to be probabilities, and the children's
+        fp = fp > 0.f ? fp * c_p : 0.f, fq = fq > 0.f ? fq * c_q : 0.f;
         const float q_to_p = fp > 0.f ? fminf(fq / fp, 1e30f) : 0.f;  // q in units of the warp's p
-        float kid_p = 0.f, kid_q = 0.f;
-        if (lane < nc) {
-            if (kid_tok >= 0 && kid_tok < V) {
-                const WalkChild c = s_kid[node & 1][lane];
-                kid_p = c.ep > 0.f ? c.ep * (walk_factor(c.mp, gp, to_log2) * c_p) : 0.f;
-                if (FULLQ) kid_q = c.eq > 0.f ? c.eq * (walk_factor(c.mq, gq, to_log2) * c_q) : 0.f;
-            } else {
-                bad = 1;
-            }
-        }
+        kid_p = child.ep > 0.f ? child.ep * (kid_p * c_p) : 0.f;
+        if (FULLQ) kid_q = child.eq > 0.f ? child.eq * (kid_q * c_q) : 0.f;
 
         // ---- the rejection chain over the node's children ----------------------------------------------
         int taken = -1;
