@@ -304,6 +304,8 @@ int eagle2_tree_attention(const void* q, const void* k_cache, const void* v_cach
  *   draft_logits_all  fp32 [B][R][V], stride d_stride; may be NULL (see above).
  *   u_accept fp32 [B][m] indexed by flat node, u_bonus fp32 [B], both in [0,1); unused at T == 0.
  *   Only rows that the walk reaches are sure to be read (and to raise EAGLE2_STATUS_NONFINITE_LOGIT).
+ *   At temperature > 0 a selected node whose sel_index is no node of the tree raises
+ *   EAGLE2_STATUS_BAD_TREE (where draft rows are given), and its sequence's result is arbitrary.
  *   acc_len [B] accepted draft tokens, acc_path [B][D] their flat positions (-1 padded),
  *   bonus_token [B].
  */

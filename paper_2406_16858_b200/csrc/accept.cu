@@ -286,13 +286,16 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
         float ux = 0.f;
         bool match = false;
         if (x < ns) {
+            // (a node outside the tree, or whose parent does not precede it, belongs to no row)
             const int idx = sel_index[(long long)b * m + x];
-            match = idx >= 0 && draft_row_of_child(idx, k) == r;
+            parx = sel_parent[(long long)b * m + x];
+            const bool ok = idx >= 0 && draft_row_of_child(idx, k) < R && parx >= -1 && parx < x;
+            match = ok && draft_row_of_child(idx, k) == r;
             if (match) {
                 tokx = sel_token[(long long)b * m + x];
-                parx = sel_parent[(long long)b * m + x];
                 ux = u_accept[(long long)b * m + x];
             }
+            if (!ok && r == 0 && me == 0) raise_status(d_status, EAGLE2_STATUS_BAD_TREE);
         }
         const unsigned bal = __ballot_sync(0xffffffffu, match);
         if ((tid & 31) == 0) s_ballot[tid >> 5] = bal;
@@ -609,8 +612,11 @@ accept_bonus_kernel(const float* __restrict__ target_logits, long long t_stride,
     const int32_t* idx_b = sel_index + (long long)b * m;
 
     for (int x = tid; x < m; x += kScanThreads) {
-        s_par[x] = sel_parent[(long long)b * m + x];
-        s_thr[x] = ws.thr[(size_t)b * m + x];
+        // (a node that the chain kernel gave to no row has no threshold: it hangs nowhere)
+        const int par = sel_parent[(long long)b * m + x];
+        const bool ok = x < ns && idx_b[x] >= 0 && draft_row_of_child(idx_b[x], k) < R && par >= -1 && par < x;
+        s_par[x] = ok ? par : -2;
+        s_thr[x] = ok ? ws.thr[(size_t)b * m + x] : 0.0;
         s_u[x] = u_accept[(long long)b * m + x];
     }
     __syncthreads();

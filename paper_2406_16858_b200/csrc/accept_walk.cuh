@@ -128,11 +128,16 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
     chain_wait();
     chain_release();
     const int ns = min(n_sel[b], m);
+    int status = 0;
     if (tid < m) {
         s_par[tid] = sel_parent[(long long)b * m + tid];
         s_tok[tid] = sel_token[(long long)b * m + tid];
-        s_idx[tid] = sel_index[(long long)b * m + tid];
         s_u[tid] = u_accept[(long long)b * m + tid];
+        if (FULLQ) {  // which draft row a node's children come from: one that is there, whatever the index says
+            int idx = sel_index[(long long)b * m + tid];
+            if (tid < ns && (idx < 0 || idx >= nodes_of(k, D))) idx = 0, status = EAGLE2_STATUS_BAD_TREE;
+            s_idx[tid] = idx;
+        }
     }
     if (tid == 0) s_found = 0x7fffffff, s_last = -1;
     if (cs > 1) cluster.sync();  // every block runs before any remote store
@@ -394,7 +399,8 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         for (int j = 0; j < NE; ++j) p[j] *= fp;
         break;
     }
-    if (bad) raise_status(d_status, EAGLE2_STATUS_NONFINITE_LOGIT);
+    if (bad) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
+    raise_status(d_status, status);
     if (me == 0 && tid == 0) {
         acc_len[b] = len;
         for (int j = len; j < D; ++j) acc_path[(long long)b * D + j] = -1;

@@ -2,6 +2,8 @@
 import numpy as np
 import pytest
 
+import paper_2406_16858_b200 as e2
+from harness import gpu_accept
 from oracle import ref
 from test_gpu_accept import _compare, _pipeline
 from workloads import generators as gen
@@ -73,3 +75,21 @@ def test_logits_of_any_size(V, B, kind):
     for temperature in (1.0, 1.5):
         for point_mass in (False, True):
             _compare(cfg, draft, sel, target, ua, ub, temperature, point_mass=point_mass, on_device=on_device)
+
+
+@pytest.mark.parametrize("V", [1004, 131076])  # the walk, and the two launches
+@pytest.mark.parametrize("index", [10 ** 6, -1, 2 ** 31 - 1])
+def test_a_selection_outside_the_tree_is_reported(V, index):
+    """A child's candidate index says which draft row proposed it; one that is no node of the tree raises the status,
+    and the other sequences are not touched by it."""
+    cfg = get_config("tiny", V=V, B=3, k=4, D=3, m=16)
+    draft, sel, target, ua, ub = _pipeline(cfg, 15)
+    want = ref.accept(target, draft, sel, V, cfg.k, cfg.D, cfg.m, 1.0, ua, ub)
+    bad = sel.index.copy()
+    bad[1, :2] = index
+    alen, apath, _, st = gpu_accept(target, draft, bad, sel.parent, sel.token, sel.n_sel, V, cfg.k, cfg.D, cfg.m, 1.0, ua, ub)
+    assert st == e2.STATUS_BAD_TREE
+    assert 0 <= alen[1] <= cfg.D and (apath[1] < cfg.m).all()
+    for b in (0, 2):
+        assert want.margins[b, 0] > 1e-6
+        assert alen[b] == want.acc_len[b] and (apath[b] == want.acc_path[b]).all()
