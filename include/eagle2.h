@@ -303,7 +303,9 @@ int eagle2_tree_attention(const void* q, const void* k_cache, const void* v_cach
  *   target_logits     fp32 [B][m+1][V], sequence stride t_stride elements (0 shares one set).
  *   draft_logits_all  fp32 [B][R][V], stride d_stride; may be NULL (see above).
  *   u_accept fp32 [B][m] indexed by flat node, u_bonus fp32 [B], both in [0,1); unused at T == 0.
- *   Only rows that the walk reaches are sure to be read (and to raise EAGLE2_STATUS_NONFINITE_LOGIT).
+ *   A bad row that the walk reaches (a target row of its nodes, or the draft row of their children)
+ *   raises EAGLE2_STATUS_NONFINITE_LOGIT.  Other rows have no part in the result and need not be read:
+ *   one that is bad may be reported (temperature == 0 and V > 131072 read more of them) or not.
  *   At temperature > 0 a selected node whose sel_index is no node of the tree raises
  *   EAGLE2_STATUS_BAD_TREE (where draft rows are given), and its sequence's result is arbitrary.
  *   acc_len [B] accepted draft tokens, acc_path [B][D] their flat positions (-1 padded),

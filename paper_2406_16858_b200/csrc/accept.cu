@@ -727,6 +727,7 @@ accept_bonus_kernel(const float* __restrict__ target_logits, long long t_stride,
     if (law.mode == 0)
         for (int c = tid; c < chunks; c += kScanThreads) gm = fmaxf(gm, (float)st[c].x);
     const double gmax = law.mode == 0 ? (double)block_max_f32(gm, s_redf) : 0.0;
+    if (tid == 0 && !(gmax > -INFINITY)) raise_status(d_status, EAGLE2_STATUS_NONFINITE_LOGIT);  // a row of only -inf
     auto chunk_weight = [&](int c) -> double {
         const double2 v = st[c];
         if (law.mode != 0) return v.y;

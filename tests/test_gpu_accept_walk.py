@@ -93,3 +93,43 @@ def test_a_selection_outside_the_tree_is_reported(V, index):
     for b in (0, 2):
         assert want.margins[b, 0] > 1e-6
         assert alen[b] == want.acc_len[b] and (apath[b] == want.acc_path[b]).all()
+
+
+@pytest.mark.parametrize("V,B", [(1004, 8), (1001, 8), (32000, 1), (131076, 2)])
+@pytest.mark.parametrize("point_mass", [False, True])
+@pytest.mark.parametrize("temperature", [0.0, 1.0])
+def test_bad_logits_on_the_walk_raise_the_status(V, B, point_mass, temperature):
+    """NaN, +inf and a row of -inf, in a row that the walk reaches (a target row or the draft row of its children): the
+    status, as the oracle has it.  A row that no walk reaches may be reported or not, and changes nothing else."""
+    cfg = get_config("tiny", V=V, B=B, k=4, D=3, m=16)
+    draft, sel, target, ua, ub = _pipeline(cfg, 16)
+    args = (sel.index, sel.parent, sel.token, sel.n_sel, V, cfg.k, cfg.D, cfg.m, temperature, ua, ub)
+    with_draft = temperature > 0 and not point_mass
+    good = gpu_accept(target, draft if with_draft else None, *args)
+    assert good[3] == 0
+    b = B - 1
+    stop = int(good[1][b, good[0][b] - 1]) if good[0][b] else -1  # the node where the walk ends
+    off = next(x for x in range(cfg.m) if (sel.parent[b] == x).any() and x not in good[1][b])  # expanded, not on the walk
+
+    def status(rows, b, row, bad):
+        kept = rows[b, row].copy()
+        if bad == "row":
+            rows[b, row] = -np.inf
+        else:
+            rows[b, row, V - 3] = bad
+        got = gpu_accept(target, draft if with_draft else None, *args)
+        want = ref.accept(target, draft if with_draft else None, sel, V, cfg.k, cfg.D, cfg.m, temperature, ua, ub)
+        rows[b, row] = kept
+        return got, want
+
+    kinds = [np.nan] if temperature == 0 else [np.nan, np.inf, "row"]  # (an arg-max needs no finite values)
+    for bad in kinds:
+        for rows, row in [(target, 0), (target, stop + 1)] + ([(draft, 0)] if with_draft else []):
+            got, want = status(rows, b, row, bad)
+            assert want.status == ref.ST_NONFINITE_LOGIT and got[3] == e2.STATUS_NONFINITE_LOGIT, (bad, row)
+        got, want = status(target, b, off + 1, bad)
+        assert want.status == 0 and got[3] in (0, e2.STATUS_NONFINITE_LOGIT)
+        if temperature > 0 and V <= 131072:
+            assert got[3] == 0
+        for mine, was in zip(got[:3], good[:3]):
+            assert (mine == was).all()
