@@ -90,6 +90,10 @@ __device__ __forceinline__ unsigned long long order_code_f64(double x) {
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
+// Logits beyond it (masks often are the lowest float; times log2(e) that overflows) are not summed: below it they weigh
+// nothing beside any other, above it the largest one stands for the row, since neighbouring floats are e^64 apart.
+constexpr float kFarLogit = 536870912.f;  // 2^29
+
 constexpr int kWarpList = 64;  // candidate keys a warp holds between two tightenings of its threshold
 
 __device__ __forceinline__ float fast_ex2(float x) {
@@ -219,7 +223,7 @@ __device__ __forceinline__ void expand_finish(int b, int V, int k, int D, int s,
                     }
                 sum = warp_sum_f64(sum);
                 if (valid[q] && !(m > -INFINITY)) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
-                lse[q] = m + log(sum);
+                lse[q] = sum == 0.0 ? m : m + log(sum);
             }
             // top-k of the chunk winners, 32*BATCH at a time together with the best so far; lane c ends
             // up holding the c-th.  The k-th largest lane maximum is a threshold no winner can be below;
@@ -367,7 +371,7 @@ __device__ __forceinline__ void expand_finish(int b, int V, int k, int D, int s,
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
             if (valid && !(mx > -INFINITY)) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
-            const double lse = mx + log(sum);
+            const double lse = sum == 0.0 ? mx : mx + log(sum);
             int parent = (s && valid) ? s_parent[r] : -1;
             const double parent_value = (s && valid) ? s_pvalue[r] : 0.0;
             if (parent < -1) {
@@ -580,7 +584,7 @@ expand_kernel(const float* __restrict__ draft_logits, long long batch_stride, in
             s_t *= fast_ex2((m_t - tm) * kLog2e);  // 0 when nothing was summed yet
             m_t = tm;
         }
-        if (m_t > -INFINITY) {
+        if (fabsf(m_t) < kFarLogit) {
             // packed pairs: two elements per multiply-add and per addition, four chains of additions
             const float2 scale2 = make_float2(kLog2e, kLog2e), neg2 = make_float2(-m_t * kLog2e, -m_t * kLog2e);
             float2 acc_a = make_float2(0.f, 0.f), acc_b = make_float2(0.f, 0.f);
@@ -593,6 +597,10 @@ expand_kernel(const float* __restrict__ draft_logits, long long batch_stride, in
                 acc_b = __fadd2_rn(acc_b, c2);
             }
             s_t += (acc_a.x + acc_a.y) + (acc_b.x + acc_b.y);
+        } else {
+#pragma unroll
+            for (int j = 0; j < NE; ++j)
+                if (cur[j] != cur[j]) s_t = cur[j];  // a NaN is seen all the same
         }
         const uint32_t block_code = *reinterpret_cast<volatile uint32_t*>(&s_bar_code);
         float thr = block_code ? order_decode(block_code) : -INFINITY;
@@ -712,7 +720,7 @@ expand_kernel(const float* __restrict__ draft_logits, long long batch_stride, in
 
     // ---- the warp's share of the segment's partial ---------------------------------------------------
     const float wmax = warp_max_f32(m_t);
-    float scaled = m_t > -INFINITY ? s_t * fast_ex2((m_t - wmax) * kLog2e) : 0.f;
+    float scaled = m_t > -INFINITY ? s_t * fast_ex2((m_t - wmax) * kLog2e) : s_t;
     scaled = warp_sum_f32(scaled);
     if (lane == 0) s_wmax[warp] = wmax, s_wsum[warp] = scaled;
     const int bad = !(scaled == scaled) || wmax == INFINITY;  // a NaN or +Inf logit poisons the sum / the max

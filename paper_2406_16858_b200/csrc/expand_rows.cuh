@@ -172,15 +172,20 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
 
     // ---- the sum of exponentials -----------------------------------------------------------------------
     // Relative to the warp's maximum in base 2, rounded up to a whole number: factors between references are exact.
-    const float wref = ceilf(wmax * kLog2e);
+    float wref = ceilf(wmax * kLog2e);
     float part[4] = {0.f, 0.f, 0.f, 0.f};
-    if (wmax > -INFINITY) {
+    if (fabsf(wmax) < kFarLogit) {
         const float2 scale2 = make_float2(kLog2e, kLog2e), neg2 = make_float2(-wref, -wref);
 #pragma unroll
         for (int j = 0; j < NE; j += 2) {
             const float2 a = __ffma2_rn(make_float2(x[j], x[j + 1]), scale2, neg2);
             part[j & 2] += fast_ex2(a.x), part[(j & 2) + 1] += fast_ex2(a.y);
         }
+    } else {
+        wref = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < NE; ++j)
+            if (x[j] != x[j]) part[0] = x[j];  // a NaN is seen all the same
     }
     const float wsum = warp_sum_f32((part[0] + part[1]) + (part[2] + part[3]));
     if (lane == 0) {
@@ -284,9 +289,11 @@ expand_rows_kernel(const float* __restrict__ draft_logits, long long batch_strid
         double sum = st.x > -INFINITY ? (double)(st.y * pow2_whole(st.x - m)) : 0.0;
 #pragma unroll
         for (int o = kRowMaxCluster / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const uint32_t best = __reduce_max_sync(0xffffffffu, lane < cs ? (uint32_t)(s_in[lane * k] >> 32) : 0u);
         if (lane == 0) {
-            s_lse = (double)m * 0.69314718055994530942 + log(sum);
-            if (!(m > -INFINITY)) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
+            const float top = best ? order_decode(best) : -INFINITY;
+            s_lse = fabsf(top) < kFarLogit ? (double)m * 0.69314718055994530942 + log(sum) : (double)top;
+            if (!(top > -INFINITY)) status |= EAGLE2_STATUS_NONFINITE_LOGIT;
         }
     }
     // (the last warp is busy with the sum; the others rank, two threads a key)

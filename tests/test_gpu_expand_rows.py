@@ -47,3 +47,43 @@ def test_a_nan_or_a_row_of_minus_inf_raises_the_status():
         draft[0, 0, 31000] = bad
         got = GpuTree(1, V, k, D).expand_all(dev(draft))
         assert int(got.status.item()) & e2.STATUS_NONFINITE_LOGIT
+
+
+@pytest.mark.parametrize("V,k,D,B", [
+    (33, 4, 2, 1), (4097, 10, 3, 3), (20000, 10, 2, 2), (131071, 4, 2, 1),  # rows held by a cluster
+    (131076, 4, 2, 1), (70004, 5, 2, 32),  # tiles: one per block, and streamed
+])
+@pytest.mark.parametrize("kind", ["run", "scattered", "flat", "one_huge"])
+def test_tokens_masked_with_the_lowest_float(V, k, D, B, kind):
+    """Masks often are the lowest number a float holds: whole threads, warps and blocks of such tokens weigh nothing."""
+    rng = np.random.default_rng(V + k)
+    lowest = np.finfo(np.float32).min
+    draft = (2.0 * rng.standard_normal((B, ref.n_draft_rows(k, D), V))).astype(np.float32)
+    if kind == "run":  # a run of tokens stays
+        at = int(rng.integers(0, V - 4 * k))
+        draft[..., :at] = draft[..., at + 4 * k:] = lowest
+    elif kind == "scattered":  # of the others some are at -inf
+        draft[rng.random(draft.shape) < 0.8] = lowest
+        draft[rng.random(draft.shape) < 0.3] = -np.inf
+        draft[..., :: max(1, V // (2 * k))] = rng.standard_normal(draft[..., :: max(1, V // (2 * k))].shape)
+    elif kind == "flat":  # nothing but the mask
+        draft[:] = lowest
+    else:
+        draft[..., V // 2] = -lowest
+    want = ref.build_tree(draft, V, k, D)
+    got = GpuTree(B, V, k, D).expand_all(dev(draft))
+    assert int(got.status.item()) == want.status == 0
+    assert (host(got.token) == want.token).all()
+    assert np.abs(host(got.value) - want.value).max() <= 1e-5 * np.abs(want.value).max()
+    assert (host(got.frontier) == want.frontier).all()
+
+
+def test_a_nan_among_excluded_tokens_raises_the_status():
+    """Also where every other token of the warps around it is at -inf, or masked."""
+    for V, B in ((32000, 1), (131076, 1), (70004, 32)):
+        for rest in (-np.inf, np.finfo(np.float32).min):
+            draft = np.full((B, 1, V), rest, np.float32)
+            draft[:, 0, :8] = 1.0
+            draft[B - 1, 0, V - 5000:V - 1000] = np.nan
+            got = GpuTree(B, V, 4, 1).expand_all(dev(draft))
+            assert int(got.status.item()) & e2.STATUS_NONFINITE_LOGIT
