@@ -835,15 +835,22 @@ accept_bonus_kernel(const float* __restrict__ target_logits, long long t_stride,
     }
 }
 
-// A cluster's registers hold the two rows of a node up to 8 blocks x 512 threads x 32 tokens.  The walk reads
-// the rows of two or three nodes of a sequence where the chain kernel reads those of every expanded node:
-// per call at V = 128256 and B = 1 / 4 / 8 / 16 / 32 37.8 / 74 / 138 / 257 / 483 -> 34.2 / 39 / 45 / 58 / 89 us,
-// with the candidates as proposal 31 / 63 / 115 / 218 / 408 -> 13 / 18.5 / 21 / 27 / 41 us; at V = 32000
-// 24 / 37 / 49 / 81 / 140 -> 26 / 32 / 33 / 42 / 38 us, one launch less in the batch-1 cycle.
+// A cluster's registers hold the two rows of a node up to 8 blocks x 512 threads x 32 tokens.  The walk reads the rows of
+// two or three nodes of a sequence, one after the other, where the chain kernel reads those of every expanded node side
+// by side.  Mean per call over 24 trees each (k = 10, m = 60, rows in L2; two launches -> walk): V = 32000, B = 1 / 2 / 4 / 8
+// 30.1 / 30.7 / 41.8 / 53.3 -> 29.4 / 32.2 / 32.5 / 34.5 us; V = 128256, B = 1 / 2 40.6 / 50.4 -> 36.5 / 41.2, B = 16 / 32
+// 256 / 486 -> 56 / 88; with the candidates as proposal V = 4096, B = 1 15.4 -> 9.9, V = 128256, B = 32 407 -> 40.
+// With draft rows the two launches are up to 4 us shorter where little is read either way (B * V below about 24000: V = 4000,
+// B = 1 / 4 22.2 / 26.8 against 26.2 / 30.1 us; one sequence of 65537 to about 115000 tokens, whose walk needs the longest
+// slices: 80000 30.4 against 33.4 us).  Those calls walk all the same: it is one launch less, which is worth as much to a
+// program that makes its calls one by one, and its sums are the more exact ones (of 9.4 million draws 2773 against 4228
+// named another token than fp64 does).
 static bool walk_holds(int V) { return V <= kWalkMaxCluster * kWalkThreads * 32; }
 
 // The slice of a block is the shortest that leaves every sequence a cluster at once on four fifths of the
-// SMs (clusters do not tile the rest); more sequences than that take the longest slices.
+// SMs (clusters do not tile the rest); more sequences than that take the longest slices.  Against nine tenths, with draft
+// rows: sixteen clusters of eight do not all fit (B = 16, V = 16000 / 32000 / 64000 36.0 / 40.7 / 48.5 -> 30.0 / 33.8 / 44.0 us),
+// thirty-two of four would (B = 32, V = 16000 / 32000 32.5 / 35.7 -> 35.8 / 43.1); other sizes are the same either way.
 static int launch_walk(int B, int V, bool vec, const float* target, long long t_stride, const float* draft, long long d_stride,
                        const int32_t* sel_index, const int32_t* sel_parent, const int32_t* sel_token, const int32_t* n_sel,
                        const float* u_accept, const float* u_bonus, int k, int D, int m, float inv_t, int32_t* acc_len,

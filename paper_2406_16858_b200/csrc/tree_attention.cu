@@ -46,6 +46,8 @@ constexpr int kAttnThreads = kSoftmaxThreads + 96;  // ... the warps that reques
 
 // Division of 31-bit numbers by a launch constant: a multiplication and a shift instead of the ~100 dependent
 // cycles of a run-time division (a block works out its place with half a dozen of them before its first request).
+// The method is the round-up multiplier of Granlund and Montgomery, "Division by invariant integers using
+// multiplication" (PLDI 1994), section 4: m = floor(2^32 (2^l - d) / d) + 1 with l = ceil(log2 d).
 struct FastDiv {
     uint32_t d, mul, shift;
     FastDiv() = default;
@@ -155,12 +157,12 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
     const long long items = (long long)B * Hkv * p->n_rb;
     const int sms = sm_count(), tpcs = sms / 2;  // a pair needs both SMs of a TPC
     // Pairs pay off while the launch is short of blocks and every sequence is cut into several
-    // splits (they halve the query and partial traffic); a launch that fills the device without
-    // splitting is better served by independent blocks.
-    // ... and while the pair's blocks stay short: with long blocks the relay between the two blocks
-    // costs more per tile than the halved partials save (70B-shaped layer, 17 tiles per pair block
-    // against 8 per single block: 35.6 against 34.2 us; LLaMA3-8B-shaped layer, 4 against 2: 18.5
-    // against 19.7 us).
+    // splits (they halve the query and partial traffic), and while the pair's blocks stay short: with
+    // long blocks the relay between the two blocks costs more per tile than the halved partials save.
+    // What gets here beside the clusters are long sequences of one to four KV heads.  Per layer, one
+    // sequence of 60 tokens, pairs against single blocks: 8 query / 2 KV heads, 12000 / 16000 / 36000 keys
+    // 15.1 / 16.3 / 23.0 against 17.7 / 20.4 / 26.7 us; 16 / 4 heads, 12000 / 16000 / 18000 keys 16.9 / 20.2 /
+    // 20.8 against 18.5 / 20.2 / 22.8; 4 / 1 heads, 16000 keys 17.6 against 25.0.
     const int tiles = (max_kv_len + m + kTK - 1) / kTK;
     p->cluster = 1, p->own = 0;
     if (single_wave && single_wave_plan(B, m, Hkv, d, tiles, p)) return;
@@ -1406,10 +1408,11 @@ static int launch_attention(const CUtensorMap& k_map, const CUtensorMap& v_map, 
         long long mblocks = (warps + 7) / 8;
         if (mblocks > 8LL * sm_count()) mblocks = 8LL * sm_count();
         // Two of the merge kernel's blocks fit on an SM, four of its packed variant's.  A launch that two
-        // per SM can hold runs the first (LLaMA3-8B-shaped layer, 240 blocks: 16.7 us per layer against
-        // 17.1 packed and kept to two per SM, 17.8 four per SM: the blocks then sit four deep on the SMs
-        // the attention blocks left first); a larger one runs the packed variant so that it is resident
-        // at once (70B-shaped layer, 480 blocks: 32.7 -> 31.4 us per layer).
+        // per SM can hold runs the first (one sequence, 60 tokens, 16 query / 4 KV heads, 120 blocks, 12000 /
+        // 24000 keys: 16.9 / 23.7 us per layer against 17.9 / 26.1 packed: the blocks then sit four deep on the
+        // SMs the attention blocks left first); a larger one runs the packed variant so that it is resident at
+        // once (64 / 8 heads, 16384 keys, 60 tokens, 480 blocks 37.4-38.9 against 39.2-40.2 us, 100 tokens, 800
+        // blocks, 11500 keys 50.7-51.3 against 53.1-54.6; two sequences of 8000 keys 40.5 against 44).
         const bool packed = mblocks > 2LL * sm_count();
         auto merge = packed ? tree_attention_merge_kernel<DH, true> : tree_attention_merge_kernel<DH, false>;
         if (launch_chained(merge, dim3((unsigned)mblocks), dim3(256), 0, st, 1, kv_off, kv_len, B, m,
