@@ -956,9 +956,12 @@ extern "C" int eagle2_accept(const float* target_logits, long long t_stride,
                   const int32_t*, const int32_t*, const float*, int, int, int, int, int, float, AcceptWs, int32_t*) =
         resident ? (vec ? accept_chain_kernel<true, true> : accept_chain_kernel<true, false>)
                  : (vec ? accept_chain_kernel<false, true> : accept_chain_kernel<false, false>);
-    if (dyn > 40 * 1024 &&
-        cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+    // (always what the longest slice needs: concurrent callers with different vocabularies then set the same value)
+    if (resident && cudaFuncSetAttribute(chain, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(sizeof(float) * 2 * kResidentSliceMax)) != cudaSuccess) {
+        cudaGetLastError();
         return EAGLE2_ERR_CUDA;
+    }
     if (launch_chained(chain, dim3((unsigned)(B * cs), (unsigned)R, 1), dim3(kChainThreads), dyn, st, (unsigned)cs,
                        target_logits, t_stride, draft_logits_all, d_stride, sel_index, sel_parent, sel_token, n_sel,
                        u_accept, V, k, m, R, slice, inv_t, w, d_status) != EAGLE2_OK)

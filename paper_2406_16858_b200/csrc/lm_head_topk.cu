@@ -498,7 +498,8 @@ static int fz_launch(const CUtensorMap& w_map, const void* hidden, long long row
     }
     if (stages > kFzMaxStages) stages = kFzMaxStages;
     const size_t dyn = 1024 + (size_t)stages * stage_bytes + (size_t)n_chunks * t_slots * kFzTBytes;
-    if (cudaFuncSetAttribute(lm_head_topk_kernel<PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+    // (always the most a block may hold: concurrent callers with different row counts then set the same value)
+    if (cudaFuncSetAttribute(lm_head_topk_kernel<PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynMax) != cudaSuccess) {
         cudaGetLastError();
         return EAGLE2_ERR_CUDA;
     }

@@ -312,10 +312,14 @@ static int rerank_launch(const int32_t* tree_token, const int32_t* tree_parent, 
     while (P < N) P <<= 1;
     const size_t dyn = (size_t)N * (sizeof(unsigned long long) + 2 * sizeof(int32_t)) +
                        (size_t)P * (sizeof(unsigned long long) + sizeof(int32_t));
+    // (always what the largest tree needs: concurrent callers with different trees then set the same value)
+    constexpr size_t kMost = EAGLE2_MAX_NODES * (2 * sizeof(unsigned long long) + 3 * sizeof(int32_t));
+    static_assert((EAGLE2_MAX_NODES & (EAGLE2_MAX_NODES - 1)) == 0, "P <= EAGLE2_MAX_NODES");
     if (dyn > 32 * 1024 &&
-        cudaFuncSetAttribute(rerank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
-            cudaSuccess)
+        cudaFuncSetAttribute(rerank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost) != cudaSuccess) {
+        cudaGetLastError();
         return EAGLE2_ERR_CUDA;
+    }
     return launch_chained(rerank_kernel, dim3(B), dim3(kRerankThreads), dyn, reinterpret_cast<cudaStream_t>(stream), 1,
                           tree_token, tree_parent, tree_value, frontier, k, N, P, m, most, sel_index, sel_parent,
                           sel_token, sel_depth, n_sel, kv_len, mask_bits, mask_dense, pos_ids, d_status);

@@ -26,7 +26,7 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
-#include <mutex>
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -94,12 +94,15 @@ struct AttnPlan {
 // many SMs each of a GPU's processing clusters has, which differs from one GPU to the next.
 static int resident_clusters(int size);
 
-static void ring_of(AttnPlan* p, int d) {
-    const size_t unit = (size_t)(d / 64) * kTK * 128;  // one 128-row operand tile
+static size_t operand_tile_bytes(int d) { return (size_t)(d / 64) * kTK * 128; }  // 128 rows
+static void ring_of(AttnPlan* p, int d) {  // (the same for every plan with as many row tiles and the same head size)
+    const size_t unit = operand_tile_bytes(d);
     int stages = (int)((220 * 1024 - p->mt * unit) / (2 * unit));
     p->stages = stages > 4 ? 4 : (stages < 2 ? 2 : stages);
     p->smem = (p->mt + 2 * (size_t)p->stages) * unit + 1024;
 }
+constexpr int kPairStages = 4, kPairStagesOrdered = 5;
+static size_t pair_smem(int stages, int d) { return (1 + (size_t)stages) * operand_tile_bytes(d) + 1024; }
 
 // Launches that the device holds at once with every (sequence, KV head, row block) on one block or one cluster of
 // blocks: which way is cheapest, by the items (128 rows x 128 keys) that one block goes through.  Combining a
@@ -206,9 +209,8 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
     p->wait_limit = wait_limit_cycles();
     p->setup_first = B == 1;  // ragged batches leave many splits without tiles: those leave at once
     if (p->pair) {  // per block: one 128-row query tile, half-size K and V stages
-        const size_t unit = (size_t)(d / 64) * kTK * 128;
-        p->stages = p->ordered ? 5 : 4;
-        p->smem = unit + (size_t)p->stages * unit + 1024;
+        p->stages = p->ordered ? kPairStagesOrdered : kPairStages;
+        p->smem = pair_smem(p->stages, d);
     }
 }
 
@@ -1352,32 +1354,33 @@ tree_attention_merge_kernel(const int64_t* __restrict__ kv_off, const int32_t* _
 
 static int resident_clusters(int size) {
     constexpr int kMaxDevices = 64;
-    static std::mutex guard;
-    static int cached[kMaxDevices][kMaxCluster + 1];  // 0: not asked yet, else clusters + 1
+    // 0: not asked yet, else clusters + 1.  (Threads that ask at the same time get and store the same answer.)
+    static std::atomic<int> cached[kMaxDevices][kMaxCluster + 1];
     int dev = 0;
     if (size < 1 || size > kMaxCluster || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
         cudaGetLastError();
         return 0;
     }
-    std::lock_guard<std::mutex> lock(guard);
-    if (cached[dev][size] == 0) {
-        auto kern = tree_attention_kernel<128, 2, false, true>;
-        const size_t smem = 200 * 1024;  // any size that leaves an SM one block
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)size * 64), cfg.blockDim = dim3(kAttnThreads), cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)size, attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr, cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            n = 0;
-        }
-        cached[dev][size] = n + 1;
+    const int known = cached[dev][size].load(std::memory_order_relaxed);
+    if (known) return known - 1;
+    auto kern = tree_attention_kernel<128, 2, false, true>;
+    AttnPlan plan;
+    plan.mt = 2;
+    ring_of(&plan, 128);  // what the kernel's launches take: one block per SM
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size * 64), cfg.blockDim = dim3(kAttnThreads), cfg.dynamicSmemBytes = plan.smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size, attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr, cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;  // (asked again by the next call: what failed now need not fail then)
     }
-    return cached[dev][size] - 1;
+    cached[dev][size].store(n + 1, std::memory_order_relaxed);
+    return n;
 }
 
 template <int DH, int MT, bool PAIR, bool CL>
@@ -1388,8 +1391,9 @@ static int launch_attention(const CUtensorMap& k_map, const CUtensorMap& v_map, 
                             float scale, void* out, float* lse, const AttnWs& ws, int32_t* d_status,
                             cudaStream_t st) {
     auto kern = tree_attention_kernel<DH, MT, PAIR, CL>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem) !=
-        cudaSuccess) {
+    // (always the same value for a kernel, whatever the plan: concurrent callers with other plans set it too)
+    const size_t most = PAIR ? pair_smem(kPairStagesOrdered, DH) : plan.smem;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) {
         cudaGetLastError();
         return EAGLE2_ERR_CUDA;
     }
