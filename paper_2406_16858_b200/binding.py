@@ -99,15 +99,27 @@ def strerror(code: int) -> str:
 _native_module = None
 
 
+def _stream_source():
+    """How native code asks torch for the current device and for its current stream's address."""
+    device, raw_stream = (getattr(torch._C, name, None) for name in ("_cuda_getDevice", "_cuda_getCurrentRawStream"))
+    if device and raw_stream:  # torch's own short cuts: no Python objects for device and stream
+        return device, raw_stream
+    return torch.cuda.current_device, lambda dev: torch.cuda.current_stream(dev).cuda_stream
+
+
 def _native():
     """The native entry points of the launching calls (loaded on first use)."""
     global _native_module
     if _native_module is None:
         lib()  # says what to do if nothing has been built
-        from . import _native as module
+        try:
+            from . import _native as module
+        except ImportError as e:
+            raise ImportError("the native entry points have not been built for this interpreter: run "
+                              "`python -m paper_2406_16858_b200.build`") from e
         if torch.cuda.is_available():
             torch.cuda.current_stream()  # brings CUDA up
-            module.set_stream_source(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+            module.set_stream_source(*_stream_source())
         _native_module = module
     return _native_module
 

@@ -1,5 +1,6 @@
-"""Builds ``libeagle2.so`` in the package directory with nvcc for sm_100a, and ``_native.so``, the
-Python entry points of its launching calls, with the host compiler.
+"""Builds ``libeagle2.so`` in the package directory with nvcc for sm_100a, and the module ``_native``,
+the Python entry points of its launching calls, with the host compiler.  The module's file name carries
+the interpreter's ABI tag: another interpreter does not find it and builds its own.
 
     python -m paper_2406_16858_b200.build [--force]
 
@@ -19,7 +20,7 @@ _ROOT = os.path.dirname(_PKG)
 _CSRC = os.path.join(_PKG, "csrc")
 _OBJ = os.path.join(_PKG, "_build")
 LIB_PATH = os.path.join(_PKG, "libeagle2.so")
-NATIVE_PATH = os.path.join(_PKG, "_native.so")
+NATIVE_PATH = os.path.join(_PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 SOURCES = ["api.cu", "expand.cu", "rerank_mask.cu", "tree_attention.cu", "accept.cu", "kv_compact.cu", "lm_head.cu", "lm_head_topk.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -70,6 +71,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
                            "-I", sysconfig.get_paths()["include"], "-I", os.path.join(_ROOT, "include"),
                            os.path.join(_CSRC, "binding.cpp"), "-o", tmp, "-L", _PKG, "-l:libeagle2.so", "-Wl,-rpath,$ORIGIN"])
     os.replace(tmp, NATIVE_PATH)
+    untagged = os.path.join(_PKG, "_native.so")  # of an earlier build: any interpreter would load it
+    if os.path.exists(untagged):
+        os.remove(untagged)
     return LIB_PATH
 
 

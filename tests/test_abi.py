@@ -3,8 +3,11 @@ declares, sizes workspaces, and rejects bad arguments before launching anything.
 import ctypes as C
 import os
 import re
+import sys
+import sysconfig
 
 import pytest
+import torch
 
 import paper_2406_16858_b200 as e2
 from paper_2406_16858_b200 import binding
@@ -108,3 +111,27 @@ def test_ordered_attention_launch_reports_its_list():
     with_list = e2.workspace_bytes(e2.OP_TREE_ATTENTION, B=8, m=60, Hq=16, Hkv=16, d=128, max_kv_len=2100)
     without = e2.workspace_bytes(e2.OP_TREE_ATTENTION, B=8, m=60, Hq=16, Hkv=16, d=128, max_kv_len=1900)
     assert with_list >= 256 + 4 * 9 and without == 0
+
+
+def test_native_module_belongs_to_this_interpreter(monkeypatch):
+    """Its file name carries the ABI tag, and without it the calls say what to do instead of falling back."""
+    from paper_2406_16858_b200 import build
+    assert build.NATIVE_PATH.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and os.path.exists(build.NATIVE_PATH)
+    assert not os.path.exists(os.path.join(os.path.dirname(build.NATIVE_PATH), "_native.so"))
+    assert binding._native().__file__ == build.NATIVE_PATH
+    monkeypatch.setattr(binding, "_native_module", None)
+    monkeypatch.setitem(sys.modules, "paper_2406_16858_b200._native", None)
+    monkeypatch.delattr(e2, "_native", raising=False)
+    with pytest.raises(ImportError, match="paper_2406_16858_b200.build"):
+        e2.tree_mask(FAKE, FAKE, FAKE, FAKE, 0, 16, FAKE, None, FAKE, FAKE)
+
+
+def test_stream_source_without_torch_internals(monkeypatch):
+    for name in ("_cuda_getDevice", "_cuda_getCurrentRawStream"):
+        monkeypatch.setattr(torch._C, name, len, raising=False)
+    assert binding._stream_source() == (len, len)
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    device, raw_stream = binding._stream_source()
+    assert device is torch.cuda.current_device
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda dev: type("S", (), {"cuda_stream": 100 + dev}))
+    assert raw_stream(3) == 103
