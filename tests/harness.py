@@ -88,6 +88,32 @@ class GpuSelection:
         torch.cuda.synchronize()
 
 
+def attention_mode(B, m, Hq, Hkv, d, max_kv_len) -> str:
+    """How a tree_attention call of these sizes is launched, from what the library says about it: how many kernels, and
+    the workspace of the plan with partial rows, which tells that plan's splits.  Block pairs cut a sequence for the
+    device's 74 pairs of SMs, single blocks for its 148 SMs."""
+    launches = e2.tree_attention_launches(B, m, Hq, Hkv, d, max_kv_len)
+    if launches == 1:
+        return "no partial rows in memory"
+    g = Hq // Hkv
+    n_rb = -(-m // (256 // g))
+    tiles_of_rows = 2 if -(-m // n_rb) * g > 128 else 1
+    rows = B * Hkv * n_rb * tiles_of_rows * 128
+    up = lambda n: -(-n // 256) * 256  # noqa: E731
+    need = e2.workspace_bytes(e2.OP_TREE_ATTENTION, B=B, m=m, Hq=Hq, Hkv=Hkv, d=d, max_kv_len=max_kv_len)
+    if B > 1:
+        return "ordered"
+    splits = next(s for s in range(1, 10000) if up(4 * B) + up(rows * s * d * 2) + up(rows * s * 8) == need)
+    tiles = -(-(max_kv_len + m) // 128)
+    per_split = -(-tiles // splits)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    of = lambda units: min(32, -(-tiles // max(1, min(tiles, units // (Hkv * n_rb)))))  # noqa: E731
+    assert of(sms) != of(sms // 2), "these sizes do not tell pairs from single blocks"
+    blocks = {of(sms): "single blocks", of(sms // 2): "block pairs"}[per_split]
+    packed = -(-Hkv * m * g // 8) > 2 * sms
+    return f"{blocks}, {'two row tiles' if tiles_of_rows == 2 else 'one row tile'}, {'packed ' if packed else ''}merge launch"
+
+
 def gpu_attention(q, kc, vc, kv_off, kv_len, mask_bits, scale, want_lse=False):
     """All arguments numpy (bf16 as uint16 bits); returns (out bf16 bits [B,m,Hq,d], lse or None, status)."""
     B, m, Hq, d = q.shape

@@ -9,7 +9,7 @@ from oracle import ref
 from workloads import get_config
 from workloads import generators as gen
 
-from harness import DEV, dev, gpu_attention, host, make_ws, new_status
+from harness import DEV, attention_mode, dev, gpu_attention, host, make_ws, new_status
 
 pytestmark = pytest.mark.gpu
 TOL = 2e-2
@@ -288,10 +288,13 @@ def test_full_size_one_layer_sampled(name):
 
 
 @pytest.mark.parametrize("mode,B,Hq,Hkv,lens", [
-    ("block pairs, several splits", 1, 32, 8, [4096]),
-    ("block pairs, two row blocks", 1, 64, 8, [8192]),
-    ("one row tile per block", 1, 32, 32, [1024]),
-    ("two row tiles per block", 8, 32, 8, [2000] * 8),
+    ("clusters, two row tiles per block", 1, 32, 8, [4096]),
+    ("clusters, two row blocks", 1, 64, 8, [8192]),
+    ("clusters, one row tile per block", 1, 32, 32, [1024]),
+    ("clusters of a batch", 8, 32, 8, [2000] * 8),
+    ("a block per sequence and KV head", 10, 32, 8, [300] * 10),
+    ("block pairs, two row tiles, merge launch", 1, 8, 2, [12000]),
+    ("single blocks, two row tiles, packed merge launch", 1, 64, 8, [16384]),
     ("ordered launch, splits merged in the kernel", 24, 32, 8,
      [9000, 300, 4500, 20, 70, 5200, 1300, 0, 4037, 4036, 8100, 64, 2500, 1, 700, 3100, 128, 4097, 0, 950, 6000,
       33, 2047, 410]),
@@ -303,6 +306,8 @@ def test_full_size_tree_keys_dominate(mode, B, Hq, Hkv, lens):
     let in, a row's word shifted) then moves the output by O(1), far above the bar.  The tree is a
     random forest; the oracle computes sampled rows one by one."""
     m, d = 60, 128
+    assert attention_mode(B, m, Hq, Hkv, d, max(lens)) == (
+        mode if "launch" in mode and "ordered" not in mode else "ordered" if "ordered" in mode else "no partial rows in memory")
     rng = np.random.default_rng(len(mode))
     kv_len = np.array(lens, np.int32)
     kv_off = gen.kv_offsets(kv_len, m)
