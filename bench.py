@@ -285,10 +285,23 @@ def batched_expand_extra(e2, dev, stream, hbm_peak, B=128, n_sets=None, reps=20)
             "algorithmic_bytes_per_call": nbytes, "achieved_gbs": gbs, "frac_of_measured_hbm": gbs / hbm_peak}
 
 
+def accept_rows_read(buf):
+    """Rows of logits that the last acceptance at temperature > 0 needed: per sequence the target row of every node on
+    the walk (the root first) and the draft row of those with selected children."""
+    path, length = buf.acc_path.cpu().numpy(), buf.acc_len.cpu().numpy()
+    parent, index = buf.sel_parent.cpu().numpy(), buf.sel_index.cpu().numpy()
+    rows = 0
+    for b in range(len(length)):
+        inner = set(int(q) for q, i in zip(parent[b], index[b]) if i >= 0)
+        walk = [-1] + [int(x) for x in path[b, :length[b]]]
+        rows += len(walk) + sum(x in inner for x in walk)
+    return rows
+
+
 def batched_accept_extra(e2, dev, stream, hbm_peak, B=16, reps=10):
     """Acceptance at temperature 1 alone for B sequences of the LLaMA3-8B-shaped tree: per sequence the
-    target and draft rows of every node that has selected children are read (once each), plus the
-    two rows of the stopping node for the extra token.  One input set (0.9 GB) is larger than L2."""
+    target rows of the nodes on its walk are read, and the draft rows of those that have selected
+    children.  One input set (0.9 GB) is larger than L2; the rows read (a few MB a sequence) may be in it."""
     import torch
     from paper_2406_16858_b200.cycle import CycleBuffers, CycleShape
     cfg = get_config("llama3_8b").with_(B=B, temperature=1.0)
@@ -328,7 +341,7 @@ def batched_accept_extra(e2, dev, stream, hbm_peak, B=16, reps=10):
     torch.cuda.synchronize()
     assert int(buf.status.item()) == 0
     us = ev0.elapsed_time(ev1) * 1e3 / reps
-    nbytes = float(parents + B) * 2 * cfg.V * 4
+    nbytes = float(accept_rows_read(buf)) * cfg.V * 4
     gbs = nbytes / (us * 1e-6) / 1e9
     return {"workload": f"llama3_8b acceptance at temperature 1, B={B} ({parents} nodes with selected children)",
             "us_per_call": us, "algorithmic_bytes_per_call": nbytes, "achieved_gbs": gbs,
@@ -861,18 +874,17 @@ def run_ours(args):
         parents += sum(len(set(int(q) for q, i in zip(sp[b], si[b]) if i >= 0)) for b in range(cfg.B))
     parents /= len(sets)
     if cfg.temperature > 0:
-        accept_bytes_def = float(cfg.B * (cfg.m + 1) + parents) * cfg.V * 4   # every target row + the parents' draft rows
-        accept_bytes_read = float(parents + cfg.B) * 2 * cfg.V * 4           # rows the kernels actually read
+        accept_bytes = float(np.mean([accept_rows_read(z["buf"]) for z in sets])) * cfg.V * 4  # the rows on the walks
     else:
-        accept_bytes_def = accept_bytes_read = float(cfg.B * (cfg.m + 1)) * cfg.V * 4
+        accept_bytes = float(cfg.B * (cfg.m + 1)) * cfg.V * 4  # every target row
+    attn_launches = e2.tree_attention_launches(cfg.B, cfg.m, cfg.Hq, cfg.Hkv, cfg.d, shape.max_kv_len)
     step_rooflines = {
         "expand": {"us": us_expand, "calls": cfg.D, "algorithmic_bytes": expand_bytes,
                    "achieved_gbs": expand_bytes / (us_expand * 1e-6) / 1e9,
                    "frac_of_measured_hbm": expand_bytes / (us_expand * 1e-6) / 1e9 / hbm_peak},
         "accept": {"us": us_accept, "temperature": cfg.temperature, "parents_with_selected_children": parents,
-                   "algorithmic_bytes": accept_bytes_def, "bytes_read": accept_bytes_read,
-                   "frac_of_measured_hbm": accept_bytes_def / (us_accept * 1e-6) / 1e9 / hbm_peak,
-                   "frac_of_measured_hbm_on_bytes_read": accept_bytes_read / (us_accept * 1e-6) / 1e9 / hbm_peak},
+                   "algorithmic_bytes": accept_bytes,
+                   "frac_of_measured_hbm": accept_bytes / (us_accept * 1e-6) / 1e9 / hbm_peak},
     }
 
     line = {
@@ -891,7 +903,8 @@ def run_ours(args):
                 "d2h_bytes_per_step": d2h,
                 "overlap": "the next step's inputs go up (copy stream, alternate input set) under this step's cycle, the results go down (third stream) under the next step's uploads"},
         "gpu_launches": buf.launches_per_cycle() * K,
-        "roofline": {"kernel": "tree_attention_kernel + tree_attention_merge_kernel, one call per layer", "bound": "hbm",
+        "roofline": {"kernel": "tree_attention_kernel, one call per layer (%d launch%s)" % (attn_launches, "es" if attn_launches > 1 else ""),
+                     "bound": "hbm",
                      "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                      "peak_kind": f"of {peak_kind}", "traffic": None, "us_per_launch": us_attn,
                      "algorithmic_bytes_per_launch": attn_bytes},
