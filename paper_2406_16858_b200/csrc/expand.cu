@@ -1,12 +1,13 @@
 // Step 1 of the hot path: draft-tree expansion (paper Section 4.1).
 //
-// One launch per expansion step.  Block (segment, row, sequence) streams its segment of one logit
-// row in tiles of 4096 tokens (two tiles of asynchronous copies in flight ahead of the one being processed); each
-// warp keeps per-thread running (max, sum exp) and its own short list of top-k candidates, and the
-// block writes one partial per segment to the workspace.  The
-// last block of a sequence to arrive merges the partials, a warp per row (fp64 log-sum-exp, top-k of
-// the segment winners), writes the new tree level (token, parent, value = parent value + log-prob)
-// and ranks the new candidates by value to produce the next frontier.
+// One launch per expansion step.  Rows whose logits a cluster's registers hold, up to 128 of them (any number
+// up to 32768 tokens), go through expand_rows.cuh; the others through the tiled form in this file.
+// There block (segment, row, sequence) streams its segment of one logit row in tiles of 4096 tokens (two tiles
+// of asynchronous copies in flight ahead of the one being processed); each warp keeps per-thread running
+// (max, sum exp) and its own short list of top-k candidates, and the block writes one partial per segment to
+// the workspace.  The last block of a sequence to arrive merges the partials, a warp per row (fp64
+// log-sum-exp, top-k of the segment winners), writes the new tree level (token, parent, value = parent value +
+// log-prob) and ranks the new candidates by value to produce the next frontier.
 #include <math.h>
 
 #include <mutex>
@@ -151,8 +152,7 @@ __device__ __forceinline__ unsigned long long warp_bitonic_merge_desc(unsigned l
 
 // What the block that arrives last for a sequence does, a warp per row: the rows' log-sum-exp from
 // the segments' statistics (fp64), the k best of the segments' winners, the new tree level (token,
-// parent, value = parent value + log-probability) and the next frontier, ranked by value.  Also the
-// whole of a merge-only launch, whose partials another kernel wrote in the same layout.
+// parent, value = parent value + log-probability) and the next frontier, ranked by value.
 // my_parent / my_parent_value: thread r < n_s holds frontier slot r's node and its value.
 __device__ __forceinline__ void expand_finish(int b, int V, int k, int D, int s, int n_s, int chunks, int by_confidence,
                                               int my_parent, double my_parent_value, int32_t* __restrict__ tree_token,

@@ -20,8 +20,8 @@
 //   MMA warp         one lane (of the pair's first block) issues four K = 16 instructions per stage;
 //                    the second block's lane tells it when that block's boxes have landed;
 //   4 writer warps   one per tensor-memory lane quadrant: 32 feature rows (columns) of the finished
-//                    accumulator at a time into one of two shared-memory buffers, transposed
-//                    ([row][vocabulary entry], rows 129 words apart: no bank conflicts either way);
+//                    accumulator at a time into one of two shared-memory units of 32 x 32, transposed
+//                    ([row][vocabulary entry], rows 33 words apart: no bank conflicts either way);
 //   8 scanner warps  warp c owns feature rows 32c .. 32c+31 of the pass, a thread one row.
 // Every wait on an mbarrier is bounded (EAGLE2_STATUS_TIMEOUT, copies drained, tensor memory freed).
 #include <cuda.h>
