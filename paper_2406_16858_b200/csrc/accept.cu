@@ -273,6 +273,7 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
     __shared__ float s_redf[2 * kChainWarps];
     __shared__ int s_child[EAGLE2_MAX_K], s_ctok[EAGLE2_MAX_K];
     __shared__ float s_pf[EAGLE2_MAX_K], s_qf[EAGLE2_MAX_K], s_uc[EAGLE2_MAX_K];  // children's p, q, uniform
+    __shared__ float s_qe[EAGLE2_MAX_K];                                           // and exponentials of q
     __shared__ double s_frozen[EAGLE2_MAX_K];
     __shared__ int s_nchild, s_parent;
 
@@ -386,6 +387,23 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
     if (!(gmax_p > -INFINITY) || (full_q && !(gmax_q > -INFINITY))) bad = 1;
 
     // ---- pass 2: exponentials (kept in place, unnormalised), sums -----------------------------------
+    // q's sum leaves the children out: what is left of q after rejections is then a sum of what is left, where one
+    // minus the rejected children's share would be nothing but rounding behind a child that holds nearly all of it.
+    // The children's own exponentials are computed exactly like the resident values.
+    if (tid < nc) {
+        const int t = s_ctok[tid];
+        s_qe[tid] = full_q && t >= 0 && t < V ? exp_scaled(scale_logit(zq[t], inv_t), gmax_q) : 0.f;
+    }
+    uint32_t mine = 0u;  // children whose token this thread sums (its tokens are four consecutive ones, or single ones)
+    for (int j = 0; j < nc; ++j) {
+        const int t = s_ctok[j] - lo;
+        if (t >= 0 && t < n_local && (VEC && RESIDENT ? t / 4 : t) % kChainThreads == tid) mine |= 1u << j;
+    }
+    auto is_child = [&](int e) {
+        bool c = false;
+        for (uint32_t left = mine; left; left &= left - 1u) c |= s_ctok[__ffs(left) - 1] - lo == e;
+        return c;
+    };
     float tp = 0.f, tq = 0.f;
     if (RESIDENT && VEC) {
         for (int e = tid * 4; e < n_local; e += kChainThreads * 4) {
@@ -398,8 +416,12 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
                 float4 c = *reinterpret_cast<const float4*>(sq + e);
                 c.x = exp_scaled(c.x, gmax_q), c.y = exp_scaled(c.y, gmax_q);
                 c.z = exp_scaled(c.z, gmax_q), c.w = exp_scaled(c.w, gmax_q);
-                tq += (c.x + c.y) + (c.z + c.w);
                 *reinterpret_cast<float4*>(sq + e) = c;
+                if (mine) {
+                    c.x = is_child(e) ? 0.f : c.x, c.y = is_child(e + 1) ? 0.f : c.y;
+                    c.z = is_child(e + 2) ? 0.f : c.z, c.w = is_child(e + 3) ? 0.f : c.w;
+                }
+                tq += (c.x + c.y) + (c.z + c.w);
             }
         }
     } else {
@@ -409,7 +431,7 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
             if (RESIDENT) sp[e] = a;
             if (full_q) {
                 const float c = exp_scaled(RESIDENT ? sq[e] : scale_logit(zq[lo + e], inv_t), gmax_q);
-                tq += c;
+                if (!mine || !is_child(e)) tq += c;
                 if (RESIDENT) sq[e] = c;
             }
         }
@@ -417,6 +439,15 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
     double sum_p = (double)tp, sum_q = (double)tq;
     chain_block_sum2(sum_p, sum_q, s_redd);
     cluster_allreduce2<false>(cluster, sum_p, sum_q, s_xchg, parity);
+    // (a token counts where it first is a child)
+    auto counts = [&](int j) {
+        for (int i = 0; i < j; ++i)
+            if (s_ctok[i] == s_ctok[j]) return false;
+        return true;
+    };
+    const double without_children = sum_q;
+    for (int j = 0; j < nc; ++j)
+        if (full_q && counts(j)) sum_q += (double)s_qe[j];
     const float c_p = (float)(1.0 / sum_p), c_q = full_q ? (float)(1.0 / sum_q) : 0.f;
     // Residual mass sum_v max(p_0(v) - alpha q_0(v), 0) over this block's slice.  The resident copies
     // hold the unnormalised exponentials; p and q are formed on the fly with the same two roundings
@@ -481,7 +512,7 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
     // ---- the rejection chain over this node's children ------------------------------------------
     // (alpha, beta): the target in force is max(p_0 - alpha q_0, 0) / beta.  Every thread of every
     // block of the cluster carries the same scalars.
-    double alpha = 0.0, beta = 1.0, removed_q = 0.0, s = 1.0;
+    double alpha = 0.0, beta = 1.0, s = 1.0;
     for (int j = 0; j < nc; ++j) {
         const double pf = (double)s_pf[j], qf = (double)s_qf[j];
         const double pj = fmax(pf - alpha * qf, 0.0) / beta;
@@ -520,9 +551,10 @@ accept_chain_kernel(const float* __restrict__ target_logits, long long t_stride,
             beta = f_new;
         }
         if (tid == 0) s_frozen[j] = alpha;
-        removed_q += qf;
-        const double rest = 1.0 - removed_q;
-        s = rest > 0.0 ? 1.0 / rest : 0.0;
+        double left = without_children;
+        for (int i = nc - 1; i > j; --i)
+            if (counts(i)) left += (double)s_qe[i];
+        s = left > 0.0 ? sum_q / left : 0.0;
     }
     __syncthreads();
     if (writer) {
@@ -838,13 +870,12 @@ accept_bonus_kernel(const float* __restrict__ target_logits, long long t_stride,
 // A cluster's registers hold the two rows of a node up to 8 blocks x 512 threads x 32 tokens.  The walk reads the rows of
 // two or three nodes of a sequence, one after the other, where the chain kernel reads those of every expanded node side
 // by side.  Mean per call over 24 trees each (k = 10, m = 60, rows in L2; two launches -> walk): V = 32000, B = 1 / 2 / 4 / 8
-// 30.1 / 30.7 / 41.8 / 53.3 -> 29.4 / 32.2 / 32.5 / 34.5 us; V = 128256, B = 1 / 2 40.6 / 50.4 -> 36.5 / 41.2, B = 16 / 32
-// 256 / 486 -> 56 / 88; with the candidates as proposal V = 4096, B = 1 15.4 -> 9.9, V = 128256, B = 32 407 -> 40.
-// With draft rows the two launches are up to 4 us shorter where little is read either way (B * V below about 24000: V = 4000,
-// B = 1 / 4 22.2 / 26.8 against 26.2 / 30.1 us; one sequence of 65537 to about 115000 tokens, whose walk needs the longest
-// slices: 80000 30.4 against 33.4 us).  Those calls walk all the same: it is one launch less, which is worth as much to a
-// program that makes its calls one by one, and its sums are the more exact ones (of 9.4 million draws 2773 against 4228
-// named another token than fp64 does).
+// 30.7 / 31.0 / 41.6 / 53.5 -> 29.6 / 33.2 / 34.2 / 36.7 us; V = 128256, B = 1 / 2 40.1 / 50.8 -> 37.5 / 42.3, B = 16 / 32
+// 256 / 486 -> 58 / 92; with the candidates as proposal V = 4096, B = 1 15.4 -> 10.1, V = 128256, B = 32 407 -> 40.
+// With draft rows the two launches are up to 4 us shorter where little is read either way (B * V below about 32000: V = 4000,
+// B = 1 / 4 22.5 / 26.7 against 26.1 / 30.5 us; V = 16000, B = 2 28.4 against 31.3; one sequence of 65537 to about 115000
+// tokens, whose walk needs the longest slices: 80000 30.5 against 33.8 us).  Those calls walk all the same: it is one launch
+// less, which is worth as much to a program that makes its calls one by one, and its sums are the more exact ones.
 static bool walk_holds(int V) { return V <= kWalkMaxCluster * kWalkThreads * 32; }
 
 // The slice of a block is the shortest that leaves every sequence a cluster at once on four fifths of the

@@ -30,7 +30,8 @@ constexpr int kWalkWarps = kWalkThreads / kWarp;
 constexpr int kWalkMaxCluster = 8;
 constexpr int kWalkEntries = kWalkWarps * kWalkMaxCluster;  // one per warp of the cluster
 
-struct WalkSums {  // a warp's contribution to the softmax sums of a node, and its largest logits
+struct WalkSums {  // a warp's contribution to the softmax sums of a node (sum_q: without the node's children), and its
+                   // largest logits
     double sum_p, sum_q;
     float max_p, max_q;
 };
@@ -250,16 +251,14 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         mp = warp_max_f32(mp);
         if (FULLQ) mq = warp_max_f32(mq);
         const double wp = warp_sum_f64((double)walk_exponentials<NE>(p, mp, to_log2));
-        double wq = 0.0;
-        if (FULLQ && with_q) wq = warp_sum_f64((double)walk_exponentials<FULLQ ? NE : 1>(q, mq, to_log2));
-        if (lane < cs) {
-            WalkSums* dst = cluster.map_shared_rank(&s_sums[node & 1][me * kWalkWarps + warp], lane);
-            dst->sum_p = wp, dst->sum_q = wq, dst->max_p = mp, dst->max_q = mq;
-        }
+        float tq = 0.f;
+        if (FULLQ && with_q) tq = walk_exponentials<FULLQ ? NE : 1>(q, mq, to_log2);
+        uint32_t mine = 0u;  // the elements of this thread that are children's tokens
         for (int i = 0; i < nc; ++i) {  // the holder of a child's token tells every block
             const int t = __shfl_sync(0xffffffffu, kid_tok, i);
             const int j = element_of(t);
             if (j >= 0 && t < V) {
+                mine |= 1u << j;
                 WalkChild c = {0.f, 0.f, mp, mq};
 #pragma unroll
                 for (int u = 0; u < NE; ++u)
@@ -270,8 +269,21 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
                 for (int r = 0; r < cs; ++r) *cluster.map_shared_rank(&s_kid[node & 1][i], r) = c;
             }
         }
+        // q's sum leaves the children out: what is left of q after rejections is then a sum of what is left, where one
+        // minus the rejected children's share would be nothing but rounding behind a child that holds nearly all of it.
+        if (FULLQ && mine) {
+            float t[2] = {0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < NE; ++j) t[j & 1] += (mine >> j) & 1u ? 0.f : q[j];
+            tq = t[0] + t[1];
+        }
+        const double wq = FULLQ ? warp_sum_f64((double)tq) : 0.0;
+        if (lane < cs) {
+            WalkSums* dst = cluster.map_shared_rank(&s_sums[node & 1][me * kWalkWarps + warp], lane);
+            dst->sum_p = wp, dst->sum_q = wq, dst->max_p = mp, dst->max_q = mq;
+        }
         meet();
-        // (a warp without mass has sum 0: its largest logit does not count; a NaN or +inf logit makes its sum NaN)
+        // (a warp without mass has sum 0 and no largest logit; a NaN or +inf logit makes its sum NaN)
         constexpr int kPerLane = kWalkEntries / 32;
         double gs_p[kPerLane], gs_q[kPerLane];
         float gm_p[kPerLane], gm_q[kPerLane], gp = -INFINITY, gq = -INFINITY;
@@ -279,17 +291,17 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
 #pragma unroll
         for (int u = 0; u < kPerLane; ++u) {
             const int i = lane + 32 * u;
-            WalkSums w = {0.0, 0.0, 0.f, 0.f};
+            WalkSums w = {0.0, 0.0, -INFINITY, -INFINITY};
             if (i < cs * kWalkWarps) w = s_sums[node & 1][i];
             gs_p[u] = w.sum_p, gs_q[u] = w.sum_q, gm_p[u] = w.max_p, gm_q[u] = w.max_q;
-            if (w.sum_p != 0.0) gp = fmaxf(gp, w.max_p);
-            if (FULLQ && w.sum_q != 0.0) gq = fmaxf(gq, w.max_q);
+            gp = fmaxf(gp, w.max_p);
+            if (FULLQ) gq = fmaxf(gq, w.max_q);
             far |= !walk_near(w.max_p, to_log2) | (FULLQ && !walk_near(w.max_q, to_log2));
         }
         far = __any_sync(0xffffffffu, far);
         gp = order_decode(__reduce_max_sync(0xffffffffu, order_code(gp)));
         if (FULLQ) gq = order_decode(__reduce_max_sync(0xffffffffu, order_code(gq)));
-        double sum_p = 0.0, sum_q = 0.0;
+        double sum_p = 0.0, sum_q = 0.0;  // (sum_q: without the children, which are added below)
         // Factors: of this warp's exponentials, of the child's in this lane (0 for a warp without mass, which has no
         // largest logit, and for a token without any).
         float fp = 0.f, fq = 0.f, kid_p = 0.f, kid_q = 0.f;
@@ -312,15 +324,33 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
         };
         if (__builtin_expect(far, 0)) weigh(std::true_type{});
         else weigh(std::false_type{});
+        // What is left of q behind child i, lane i: the sum without children and the children after it (a token counts
+        // where it first is).  Sums and scan go side by side.
+        double behind = 0.0;  // of this lane's child and those after it
+        if (FULLQ) {
+            const unsigned same = __match_any_sync(0xffffffffu, kid_tok);
+            if (lane < nc && __ffs(same) - 1 == lane) behind = (double)child.eq * (double)kid_q;
+        }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sum_p += __shfl_xor_sync(0xffffffffu, sum_p, o);
-            if (FULLQ) sum_q += __shfl_xor_sync(0xffffffffu, sum_q, o);
+        for (int s = 0; s < 5; ++s) {
+            sum_p += __shfl_xor_sync(0xffffffffu, sum_p, 16 >> s);
+            if (FULLQ) {
+                sum_q += __shfl_xor_sync(0xffffffffu, sum_q, 16 >> s);
+                const double add = __shfl_down_sync(0xffffffffu, behind, 1 << s);
+                if (lane + (1 << s) < 32) behind += add;
+            }
+        }
+        double left = 0.0;
+        if (FULLQ) {
+            const double after = __shfl_down_sync(0xffffffffu, behind, 1);
+            left = sum_q + (lane < 31 ? after : 0.0);
+            sum_q += __shfl_sync(0xffffffffu, behind, 0);
         }
         // (a row whose largest logit overflows when divided by the temperature counts as one that was not finite)
         bad |= !(sum_p > 0.0) | !(fabsf(gp * inv_t) < INFINITY);
         if (FULLQ && with_q) bad |= !(sum_q > 0.0) | !(fabsf(gq * inv_t) < INFINITY);
         const float c_p = (float)(1.0 / sum_p), c_q = with_q ? (float)(1.0 / sum_q) : 0.f;
+        if (FULLQ) left *= with_q ? 1.0 / sum_q : 0.0;
         // what this warp's exponentials have to be multiplied with to be probabilities, and the children's
         fp = fp > 0.f ? fp * c_p : 0.f, fq = fq > 0.f ? fq * c_q : 0.f;
         const float q_to_p = fp > 0.f ? fminf(fq / fp, 1e30f) : 0.f;  // q in units of the warp's p
@@ -352,7 +382,7 @@ accept_walk_kernel(const float* __restrict__ target_logits, long long t_stride,
                     mass = mass_of_all(((part[0] + part[1]) + (part[2] + part[3])) * fp);
                 }
                 if (mass > 0.0) alpha = alpha_new, beta = mass;  // zero residual mass: the target stays
-                rest -= qf;
+                rest = __shfl_sync(0xffffffffu, left, i);
                 const int e = element_of(__shfl_sync(0xffffffffu, kid_tok, i));
                 if (e >= 0) {
                     const float ai = (float)alpha * q_to_p;

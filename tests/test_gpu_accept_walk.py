@@ -133,3 +133,23 @@ def test_bad_logits_on_the_walk_raise_the_status(V, B, point_mass, temperature):
             assert got[3] == 0
         for mine, was in zip(got[:3], good[:3]):
             assert (mine == was).all()
+
+
+@pytest.mark.parametrize("V,B", [(1004, 40), (1001, 40), (32000, 8), (131076, 3)])
+@pytest.mark.parametrize("lead", [14.0, 18.0, 40.0])
+def test_a_proposal_that_one_child_nearly_fills(V, B, lead):
+    """Behind a first child with all but a little of the draft's mass the second is tested against its share of what is
+    left, which one minus the first child's probability does not say in 32 bits."""
+    cfg = get_config("tiny", V=V, B=B, k=4, D=3, m=16)
+    rng = np.random.default_rng(V)
+    base = (2.0 * rng.standard_normal((B, ref.n_draft_rows(cfg.k, cfg.D), V))).astype(np.float32)
+    base[..., :4] += 9.0  # four likely tokens
+    draft = base.copy()
+    np.put_along_axis(draft, draft.argmax(-1)[..., None], draft.max(-1, keepdims=True) + np.float32(lead), -1)
+    tree = ref.build_tree(draft, V, cfg.k, cfg.D)
+    sel = ref.rerank(tree.token, tree.parent, tree.value, cfg.k, cfg.D, cfg.m)
+    target = gen.target_rows(cfg, 3, base, tree.parent, sel.index)
+    ua, ub = gen.uniforms(cfg, 3)
+    _, want = _compare(cfg, draft, sel, target, ua, ub, 1.0)
+    tested = np.isfinite(want.accept_prob).sum(axis=1)
+    assert (tested > want.acc_len + 1).any()  # a second child was tested at some node
