@@ -7,15 +7,17 @@
 // to 256 packed rows (two 128-row UMMA tiles) and is warp specialised:
 //   softmax warps  one thread per query row.  S = Q.K^T arrives in tensor memory; the thread takes
 //                  its row into registers, applies scale, tree mask and a lazily rescaled running
-//                  maximum, and writes P as bf16 back into tensor memory over the scores.
+//                  maximum, and writes P as bf16 back into tensor memory.
 //   K, V warps     stream 128-key tiles (TMA, 128-byte swizzled) through a ring of stages each.
-//   MMA warp       issues tcgen05.mma: S = Q.K^T (operands in shared memory) and O += P.V (P from
-//                  tensor memory, V in shared memory, MN-major), two score slots in flight so that
-//                  the tensor pipe and the softmax warps overlap.
-// What bounds a block: the chain scores -> probabilities -> P.V -> next scores of a slot (0.9 us for 128 x 128
-// with both slots busy: 1.75 us per tile of 128 keys x 256 rows, where the tensor pipe alone needs 1.06 us, the
-// exponentials 1.04 us and the K/V tile's 64 KB 1.5 us).  It was 2.3 us with sixteen softmax warps that read the
-// scores twice and exchanged half rows' maxima, and MMAs issued by a diverged lane (92 instead of 55 cycles each).
+//   MMA warps      issue tcgen05.mma, one S = Q.K^T (operands in shared memory), the other O += P.V (P from
+//                  tensor memory, V in shared memory, MN-major).
+// What bounds a block: 1.65 us per tile of 128 keys x 256 rows, where the tensor pipe alone needs 1.06 us, the
+// exponentials 1.04 us and the K/V tile's 64 KB 1.5 us.  The scores have one set of tensor-memory columns, which a
+// group leaves as soon as it has them in registers (0.15 us), and the probabilities have their own: the next scores
+// come while the exponentials are taken and P.V waits its turn.  What remains is the ring scores -> registers -> next
+// scores (0.8 us per group, the tensor pipe being shared with P.V) and the pass of a group (1.45 us beside the other
+// group's, 1.0 us alone).  While the probabilities lay over the scores, a slot's scores, probabilities and P.V were
+// one chain: 1.75 us per tile; one warp that issued both kinds of MMA, polling for either, made it 1.85.
 // The block writes final rows when it serves its sequence alone; otherwise the blocks of a cluster combine
 // their rows among themselves, or partial rows go to L2 and are combined by a merge kernel or by the last
 // block to finish.
@@ -40,9 +42,8 @@ constexpr int kMaxTilesPerSplit = 16; // sequences that would need longer blocks
 constexpr int kMaxTilesPerSplitOrdered = 64;  // a block never streams more than 8192 keys
 constexpr int kTmemCols = 512;
 constexpr int kMaxCluster = 8;
-constexpr int kSlots = 2;             // score slots in tensor memory
 constexpr int kSoftmaxThreads = 256;  // 8 softmax warps: two per SM sub-partition, one of each group
-constexpr int kAttnThreads = kSoftmaxThreads + 96;  // ... the warps that request K, issue MMAs, request Q and V
+constexpr int kAttnThreads = kSoftmaxThreads + 128;  // ... the warps that request K, issue Q.K^T, request Q and V, issue P.V
 
 // Division of 31-bit numbers by a launch constant: a multiplication and a shift instead of the ~100 dependent
 // cycles of a run-time division (a block works out its place with half a dozen of them before its first request).
@@ -318,11 +319,9 @@ constexpr int kMaxStages = 6;  // K/V ring depth the barrier arrays allow
 struct AttnBarriers {
     unsigned long long q_full;
     unsigned long long k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
-    unsigned long long s_full[kSlots], p_first[kSlots], p_full[kSlots];  // scores / first 32 keys' / all probabilities
-    // Per accumulator (= score slot = item parity), two barriers used by its alternate uses: the
-    // u-th P.V into accumulator e completes a phase of o_done[e][u & 1].  A waiter may skip phases (it only looks when it must rescale O, and at the
-    // end); with two barriers the one it consults is never more than one phase ahead of it.
-    unsigned long long o_done[2][2];
+    unsigned long long s_full[2], s_free;         // a group's scores are there / the scores' columns may be overwritten
+    unsigned long long p_first[2], p_full[2];     // first 32 keys' / all probabilities of a group
+    unsigned long long o_done[2];                 // the group's P.V has completed
     // pair mode, used in the pair's first block: the other block's query tile / K half / V half
     // has landed (and its V tail is cleared)
     unsigned long long q_peer, k_peer[kMaxStages], v_peer[kMaxStages];
@@ -536,10 +535,13 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     constexpr int HALVES = DH / 64;                    // 64-column (128-byte) panels per operand tile
     constexpr uint32_t kPanel = kTK * 128;             // bytes of one panel: 128 rows x 128 bytes
     constexpr uint32_t kTile = HALVES * kPanel;
-    constexpr int kTmaWarp = kSoftmaxThreads / 32, kMmaWarp = kTmaWarp + 1, kVWarp = kTmaWarp + 2;
+    constexpr int kTmaWarp = kSoftmaxThreads / 32, kMmaWarp = kTmaWarp + 1, kVWarp = kTmaWarp + 2, kPvWarp = kTmaWarp + 3;
     constexpr uint32_t kIdescQK = instr_desc(kTK, false, PAIR ? 256 : 128);
     constexpr uint32_t kIdescPV = instr_desc(DH, true, PAIR ? 256 : 128);
-    constexpr uint32_t kOCol = kSlots * kTK;           // first accumulator column of O
+    // Tensor memory, 512 columns: one set of score columns that the groups use in turn, each group's probabilities, two
+    // accumulators.  The second group's first scores, which would have to wait for the first group, take the last 128
+    // columns: its accumulator (head_dim 128), which nothing has written yet, or columns that nothing else uses.
+    constexpr uint32_t kPCol = kTK, kPCols = kTK / 2, kOCol = kPCol + 2 * kPCols, kSCol1 = kTmemCols - kTK;
     constexpr uint32_t kRowBytes = DH * 2;
     // bytes a block holds of one K tile and of one V tile (a pair splits K by keys, V by columns)
     constexpr uint32_t kKPanel = PAIR ? kPanel / 2 : kPanel, kKTile = HALVES * kKPanel;
@@ -585,20 +587,20 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             if (PAIR) mbar_init(smem_u32(&bars.k_peer[tid]), 1), mbar_init(smem_u32(&bars.v_peer[tid]), 1);
             fence_barrier_init();
         } else if (tid >= 32 && tid < 34) {
-            const int e = tid & 1;  // score slot = accumulator = group
+            const int e = tid & 1;  // accumulator = group
             mbar_init(smem_u32(&bars.s_full[e]), 1);
-            const uint32_t warps = (PAIR ? 2 : 1) * (kSoftmaxThreads / 64);  // one arrival per warp of the slot's group
+            const uint32_t warps = (PAIR ? 2 : 1) * (kSoftmaxThreads / 64);  // one arrival per warp of a group
             mbar_init(smem_u32(&bars.p_first[e]), warps);
             mbar_init(smem_u32(&bars.p_full[e]), warps);
-            mbar_init(smem_u32(&bars.o_done[e][0]), 1);
-            mbar_init(smem_u32(&bars.o_done[e][1]), 1);
+            mbar_init(smem_u32(&bars.o_done[e]), 1);
+            if (e == 0) mbar_init(smem_u32(&bars.s_free), warps);
             fence_barrier_init();
         } else if (tid == 64) {
             s_ctl.abort = 0;
             s_ctl.limit = plan.wait_limit;
             mbar_init(smem_u32(&bars.q_full), plan.q_tma ? 1 : kSoftmaxThreads);
             if (PAIR) mbar_init(smem_u32(&bars.q_peer), 1);
-            mbar_init(smem_u32(&bars.drain), 1);
+            mbar_init(smem_u32(&bars.drain), 2);  // (each issuing warp's commit covers its own instructions)
             mbar_init(smem_u32(&bars.v_clean), 1);
             if (CL) mbar_init(smem_u32(&bars.peers_ready), plan.cluster), mbar_init(smem_u32(&bars.inbox), 1);
             fence_barrier_init();
@@ -691,7 +693,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     if (CL && tid == 0 && !overflow) mbar_expect_tx(smem_u32(&bars.inbox), (uint32_t)(S_b * rows_of(split)) * (kRowBytes + 8));
     bool softmax_ok = true;
     int k_issued = 0, v_issued = 0;  // TMA lane: K and V tiles requested so far
-    const int n_items = nt * MT;  // item i = (tile i / MT, row tile i % MT), score slot i % 2
+    const int n_items = nt * MT;  // item i = (tile i / MT, row tile i % MT), group i % 2
     // The only tile of this block that can reach past the sequence's last key is its last one.  Its P.V covers
     // the 16-key groups that hold a key; rows of the last such group that lie past the last key hold whatever
     // follows the sequence in the cache and are cleared, so that a zero probability times a non-finite value
@@ -771,87 +773,80 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 if (lane == 0) mbar_arrive(smem_u32(&bars.v_clean));
             }
         }
-    } else if (warp == kMmaWarp) {
-        // ===== MMA issuer: the whole warp walks the tiles and waits, one elected lane issues.  The loop's
-        // values are the same in all lanes, so that descriptors and addresses stay in uniform registers,
-        // where the instruction wants them (a lane on its own moves them there one by one: ~90 cycles per
-        // instruction beside busy softmax warps, which is slower than the tensor pipe).
+    } else if (warp == kMmaWarp || warp == kPvWarp) {
+        // ===== MMA issuers, a warp for Q.K^T and one for P.V: each walks its items in order and waits for nothing that
+        // concerns the other.  The whole warp waits, one elected lane issues.  The loop's values are the same in all
+        // lanes, so that descriptors and addresses stay in uniform registers, where the instruction wants them (a lane
+        // on its own moves them there one by one: ~90 cycles per instruction beside busy softmax warps, which is slower
+        // than the tensor pipe).
         auto wait1 = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait_spin(bar, parity, abort_flag)) != 0; };
-        auto here1 = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test_wait(bar, parity)) != 0; };
-        bool ok = wait1(smem_u32(&bars.q_full), 0);
-        if (PAIR && rank != 0) {
-            // The second block of a pair issues no MMA: this warp tells the first block when this
-            // block's query tile, K half and V half are in place.
-            if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.q_peer), 0);
-            int st = 0;
-            uint32_t ph = 0;
+        auto commit = [&](uint32_t bar) {
+            if (PAIR) tc_commit2(bar);
+            else tc_commit(bar);
+        };
+        // Descriptor words of the three operand layouts (low word: address and leading offset
+        // in 16-byte units; high word: the layout's constants).
+        constexpr int CG = PAIR ? 2 : 1;
+        bool ok = true;
+        int st = 0;        // ring stage of the tile
+        uint32_t ph = 0;   // and the phase of its barrier
+        if (warp == kMmaWarp) {
+            ok = wait1(smem_u32(&bars.q_full), 0);
+            if (PAIR && rank != 0) {
+                // The second block of a pair issues no MMA: these warps tell the first block when this
+                // block's query tile, K half and V half are in place.
+                if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.q_peer), 0);
+                for (int j = 0; j < nt && ok; ++j) {
+                    ok = wait1(smem_u32(&bars.k_full[st]), ph);
+                    if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.k_peer[st]), 0);
+                    if (++st == NST) st = 0, ph ^= 1u;
+                }
+            } else {
+                if (PAIR) ok = ok && wait1(smem_u32(&bars.q_peer), 0);
+                const uint64_t qd_first = smem_desc(sQ, 16), kd_first = smem_desc(sK, 16);
+                const uint32_t q_lo0 = (uint32_t)qd_first, k_lo0 = (uint32_t)kd_first, qk_hi = (uint32_t)(qd_first >> 32);
+                for (int i = 0; i < n_items; ++i) {  // S = Q[row tile] . K[tile]^T
+                    const int t = i & (MT - 1);
+                    if (t == 0) {
+                        ok = ok && wait1(smem_u32(&bars.k_full[st]), ph);
+                        if (PAIR) ok = ok && wait1(smem_u32(&bars.k_peer[st]), ph);
+                    }
+                    // (item 0 has been read before item 2 overwrites it, item i - 1 before item i; item 1 has columns of its own)
+                    if (i >= 2) ok = ok && wait1(smem_u32(&bars.s_free), (uint32_t)(i & 1));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d_tmem = tmem + (i == 1 ? kSCol1 : 0u);
+                    const uint32_t q_lo = q_lo0 + (uint32_t)t * (kTile >> 4), k_lo = k_lo0 + (uint32_t)st * (kKTile >> 4);
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 0; ks < DH / 16; ++ks) {
+                            const uint32_t qo = ((uint32_t)(ks / 4) * kPanel + (uint32_t)(ks % 4) * 32u) >> 4;
+                            const uint32_t ko = ((uint32_t)(ks / 4) * kKPanel + (uint32_t)(ks % 4) * 32u) >> 4;
+                            if (ks == 0) umma_ss<CG, 0>(d_tmem, q_lo + qo, qk_hi, k_lo + ko, qk_hi, kIdescQK);
+                            else umma_ss<CG, 1>(d_tmem, q_lo + qo, qk_hi, k_lo + ko, qk_hi, kIdescQK);
+                        }
+                        commit(smem_u32(&bars.s_full[i & 1]));
+                        if (t == MT - 1) commit(smem_u32(&bars.k_empty[st]));
+                    }
+                    __syncwarp();
+                    if (t == MT - 1 && ++st == NST) st = 0, ph ^= 1u;
+                }
+            }
+        } else if (PAIR && rank != 0) {
             for (int j = 0; j < nt && ok; ++j) {
-                ok = wait1(smem_u32(&bars.k_full[st]), ph);
-                if (!ok) break;
-                if (lane == 0) mbar_arrive_in(smem_u32(&bars.k_peer[st]), 0);
                 ok = wait1(smem_u32(&bars.v_full[st]), ph);
                 if (ok && has_tail && j == jt) ok = wait1(smem_u32(&bars.v_clean), 0);
-                if (!ok) break;
-                if (lane == 0) mbar_arrive_in(smem_u32(&bars.v_peer[st]), 0);
+                if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.v_peer[st]), 0);
                 if (++st == NST) st = 0, ph ^= 1u;
             }
         } else {
-            if (PAIR) ok = ok && wait1(smem_u32(&bars.q_peer), 0);
-            auto commit = [&](uint32_t bar) {
-                if (PAIR) tc_commit2(bar);
-                else tc_commit(bar);
-            };
-            // Descriptor words of the three operand layouts (low word: address and leading offset
-            // in 16-byte units; high word: the layout's constants).
-            constexpr int CG = PAIR ? 2 : 1;
-            const uint64_t qd_first = smem_desc(sQ, 16), kd_first = smem_desc(sK, 16), vd_first = smem_desc(sV, kPanel);
-            const uint32_t q_lo0 = (uint32_t)qd_first, k_lo0 = (uint32_t)kd_first, v_lo0 = (uint32_t)vd_first;
-            const uint32_t qk_hi = (uint32_t)(qd_first >> 32), v_hi = (uint32_t)(vd_first >> 32);
-            int k_st = 0, v_st = 0;        // ring stage of the K tile the next Q.K^T reads, of the V tile the next P.V reads
-            uint32_t k_ph = 0, v_ph = 0;   // and the phases of their barriers
-            // the K tile of item i has landed (both halves of a pair); LOOK: is it there already?
-            auto wait_qk = [&](int i) {
-                if ((i & (MT - 1)) == 0) {
-                    ok = ok && wait1(smem_u32(&bars.k_full[k_st]), k_ph);
-                    if (PAIR) ok = ok && wait1(smem_u32(&bars.k_peer[k_st]), k_ph);
-                }
-            };
-            auto look_qk = [&](int i) {
-                if ((i & (MT - 1)) != 0) return true;
-                return here1(smem_u32(&bars.k_full[k_st]), k_ph) && (!PAIR || here1(smem_u32(&bars.k_peer[k_st]), k_ph));
-            };
-            auto issue_qk = [&](int i) {  // S[slot] = Q[row tile] . K[tile]^T
-                const int t = i & (MT - 1);
-                const uint32_t d_tmem = tmem + (uint32_t)(i & 1) * kTK;
-                const uint32_t q_lo = q_lo0 + (uint32_t)t * (kTile >> 4), k_lo = k_lo0 + (uint32_t)k_st * (kKTile >> 4);
-                if (elect_one()) {
-#pragma unroll
-                    for (int ks = 0; ks < DH / 16; ++ks) {
-                        const uint32_t qo = ((uint32_t)(ks / 4) * kPanel + (uint32_t)(ks % 4) * 32u) >> 4;
-                        const uint32_t ko = ((uint32_t)(ks / 4) * kKPanel + (uint32_t)(ks % 4) * 32u) >> 4;
-                        if (ks == 0) umma_ss<CG, 0>(d_tmem, q_lo + qo, qk_hi, k_lo + ko, qk_hi, kIdescQK);
-                        else umma_ss<CG, 1>(d_tmem, q_lo + qo, qk_hi, k_lo + ko, qk_hi, kIdescQK);
-                    }
-                    commit(smem_u32(&bars.s_full[i & 1]));
-                    if (t == MT - 1) commit(smem_u32(&bars.k_empty[k_st]));
-                }
-                __syncwarp();
-                if (t == MT - 1 && ++k_st == NST) k_st = 0, k_ph ^= 1u;
-            };
-            auto wait_pv = [&](int i) {   // the V tile of item i has landed, its first probabilities are written
+            const uint64_t vd_first = smem_desc(sV, kPanel);
+            const uint32_t v_lo0 = (uint32_t)vd_first, v_hi = (uint32_t)(vd_first >> 32);
+            for (int i = 0; i < n_items; ++i) {  // O[row tile] += P[group] . V[tile]
                 const int t = i & (MT - 1), j = MT == 1 ? i : (i >> 1);
-                if (t == 0) {
-                    ok = ok && wait1(smem_u32(&bars.v_full[v_st]), v_ph);
-                    if (has_tail && j == jt) ok = ok && wait1(smem_u32(&bars.v_clean), 0);
-                    if (PAIR) ok = ok && wait1(smem_u32(&bars.v_peer[v_st]), v_ph);
-                }
-                ok = ok && wait1(smem_u32(&bars.p_first[i & 1]), (uint32_t)((i >> 1) & 1));
-            };
-            auto issue_pv = [&](int i) {  // O[row tile] += P[slot] . V[tile]
-                const int t = i & (MT - 1), j = MT == 1 ? i : (i >> 1);
-                const uint32_t d_tmem = tmem + kOCol + (uint32_t)(i & 1) * DH;  // accumulator = slot = item parity
-                const uint32_t a_tmem = tmem + (uint32_t)(i & 1) * kTK;
-                const uint32_t v_lo = v_lo0 + (uint32_t)v_st * (kVTile >> 4);
+                const uint32_t e = (uint32_t)(i & 1), p_ph = (uint32_t)((i >> 1) & 1);
+                const uint32_t d_tmem = tmem + kOCol + e * DH, a_tmem = tmem + kPCol + e * kPCols;
+                const uint32_t v_lo = v_lo0 + (uint32_t)st * (kVTile >> 4);
                 const int n_ks = j == jt ? groups_t : kTK / 16;
                 auto steps = [&](auto from, auto to) {
 #pragma unroll
@@ -861,42 +856,26 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                         else if (ks < n_ks) umma_ts<CG, 1>(d_tmem, a_tmem + ks * 8, v_lo + vo, v_hi, kIdescPV);
                     }
                 };
+                if (t == 0) {
+                    ok = wait1(smem_u32(&bars.v_full[st]), ph);
+                    if (has_tail && j == jt) ok = ok && wait1(smem_u32(&bars.v_clean), 0);
+                    if (PAIR) ok = ok && wait1(smem_u32(&bars.v_peer[st]), ph);
+                }
+                ok = ok && wait1(smem_u32(&bars.p_first[e]), p_ph);
+                if (!ok) break;
+                tc_fence_after();
                 if (elect_one()) steps(std::integral_constant<int, 0>{}, std::integral_constant<int, 2>{});
                 __syncwarp();
-                ok = wait1(smem_u32(&bars.p_full[i & 1]), (uint32_t)((i >> 1) & 1));
-                if (!ok) return;
+                ok = wait1(smem_u32(&bars.p_full[e]), p_ph);
+                if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) {
                     steps(std::integral_constant<int, 2>{}, std::integral_constant<int, kTK / 16>{});
-                    commit(smem_u32(&bars.o_done[i & 1][(i >> 1) & 1]));
-                    if (t == MT - 1) commit(smem_u32(&bars.v_empty[v_st]));
+                    commit(smem_u32(&bars.o_done[e]));
+                    if (t == MT - 1) commit(smem_u32(&bars.v_empty[st]));
                 }
                 __syncwarp();
-                if (t == MT - 1 && ++v_st == NST) v_st = 0, v_ph ^= 1u;
-            };
-            static_assert(kSlots == 2, "slot = item & 1");
-            for (int i = 0; i < kSlots && i < n_items && ok; ++i) {
-                wait_qk(i);
-                if (!ok) break;
-                tc_fence_after();
-                issue_qk(i);
-            }
-            for (int i = 0; i < n_items && ok; ++i) {
-                const bool more = i + kSlots < n_items;
-                // With the next K tile at hand both groups of instructions go out back to back; otherwise P.V
-                // does not wait for it.
-                const bool now = more && look_qk(i + kSlots);
-                wait_pv(i);
-                if (!ok) break;
-                tc_fence_after();
-                issue_pv(i);
-                if (!ok) break;
-                if (more && !now) {
-                    wait_qk(i + kSlots);
-                    if (!ok) break;
-                    tc_fence_after();
-                }
-                if (more) issue_qk(i + kSlots);
+                if (t == MT - 1 && ++st == NST) st = 0, ph ^= 1u;
             }
         }
         __syncwarp();
@@ -944,16 +923,19 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 
         float m_ref = -INFINITY, l_run = 0.f;
         bool ok = true;
-        const uint32_t s_addr = tmem + lane_sel + (uint32_t)grp * kTK;          // this thread's scores
+        const uint32_t p_addr = tmem + lane_sel + kPCol + (uint32_t)grp * kPCols;  // this thread's probabilities
         const uint32_t o_acc = tmem + lane_sel + kOCol + (uint32_t)grp * DH;    // and its row of the group's accumulator
-        auto release = [&](uint32_t bar) {  // what this warp has written to tensor memory so far may be read
-            tc_wait_st();
+        auto tell = [&](uint32_t bar) {  // this warp's accesses to tensor memory so far are over
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
-                if (PAIR) mbar_arrive_in(bar, 0);  // the pair's first block issues P.V
+                if (PAIR) mbar_arrive_in(bar, 0);  // the pair's first block issues the MMAs
                 else mbar_arrive(bar);
             }
+        };
+        auto release = [&](uint32_t bar) {  // what this warp has written to tensor memory so far may be read
+            tc_wait_st();
+            tell(bar);
         };
         for (int i = grp; i < n_items; i += 2) {
             const int u = i >> 1;                          // the u-th use of this group's slot and accumulator
@@ -967,10 +949,12 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             }
             uint32_t sc[4][32];
             tc_fence_after();
+            const uint32_t s_addr = tmem + lane_sel + (i == 1 ? kSCol1 : 0u);
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + c * 32, sc[c]);
 #pragma unroll
             for (int c = 0; c < 4; ++c) tc_wait_ld(sc[c]);
+            if (i != 1) tell(smem_u32(&bars.s_free));  // the other group's scores may come
             const int key0 = (t_begin + j) * kTK;
             if (key0 + kTK > L) {  // the tile holds tree keys or runs past the last key: hide what the row may not see
                 uint32_t vis[4];
@@ -994,15 +978,18 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             // lazily rescaled reference maximum: probabilities stay below 2^8 in between
             const float m_new = fmaxf(m_ref, mx);
             const bool grow = m_new > m_ref + 8.f;
+            // the group's previous P.V has finished: its probabilities have been read, the accumulator is at rest
+            auto at_rest = [&]() {
+                ok = u == 0 || mbar_wait(smem_u32(&bars.o_done[grp]), (uint32_t)((u - 1) & 1), abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
+                tc_fence_after();
+                return ok;
+            };
             if (__any_sync(0xffffffffu, grow)) {
                 const float factor = !grow ? 1.f : (m_ref == -INFINITY ? 0.f : ex2(m_ref - m_new));
                 if (grow) m_ref = m_new, l_run *= factor;
                 if (u > 0) {
-                    // the accumulator may be rescaled once the group's previous P.V has finished
-                    ok = mbar_wait(smem_u32(&bars.o_done[grp][(u - 1) & 1]), (uint32_t)(((u - 1) >> 1) & 1), abort_flag);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                    tc_fence_after();
+                    if (!at_rest()) break;
 #pragma unroll 1
                     for (int c0 = 0; c0 < DH; c0 += 16) {
                         uint32_t orow[16];
@@ -1014,7 +1001,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                     }
                 }
             }
-            // P = 2^(s * scale - reference) as bf16, over the first half of the scores' columns
+            // P = 2^(s * scale - reference) as bf16
             const float neg_ref = m_ref == -INFINITY ? 0.f : -m_ref;
             const float2 scale2 = make_float2(scale_log2, scale_log2), neg_ref2 = make_float2(neg_ref, neg_ref);
             float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -1028,11 +1015,12 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                     sum[(e >> 1) & 1] = __fadd2_rn(sum[(e >> 1) & 1], a);
                     pk[e >> 1] = pack_bf16(a.x, a.y);
                 }
-                tmem_st16(s_addr + c * 16, pk);
-                // (P.V starts on the first 32 keys while the others' exponentials are still being taken: the
-                // pass, the products and the next scores form a chain.  2 % per layer; 64 or 96 keys: less.)
+                if (c == 0 && !at_rest()) break;
+                tmem_st16(p_addr + c * 16, pk);
+                // (P.V starts on the first 32 keys while the others' exponentials are still being taken)
                 if (c == 0) release(smem_u32(&bars.p_first[grp]));
             }
+            if (!ok) break;
             l_run += (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y);
             release(smem_u32(&bars.p_full[grp]));
         }
@@ -1043,7 +1031,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         // them gave up.  A group that served no item (a block with a single item) contributes nothing.
         const int n_uses = (n_items - grp + 1) / 2;  // items this group served
         if (ok && n_uses > 0)
-            ok = mbar_wait(smem_u32(&bars.o_done[grp][(n_uses - 1) & 1]), (uint32_t)(((n_uses - 1) >> 1) & 1), abort_flag);
+            ok = mbar_wait(smem_u32(&bars.o_done[grp]), (uint32_t)((n_uses - 1) & 1), abort_flag);
         if (MT == 1) s_half[grp][r_tile] = make_float2(m_ref, l_run);
         ok = named_barrier_and(1, kSoftmaxThreads, ok);
         softmax_ok = ok;
@@ -1244,9 +1232,12 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         // Whoever gave up, and whenever: the tensor instructions issued so far may still read shared
         // memory and write tensor memory, and copies may still be on their way into the rings.  Both
         // must have finished before either memory is given back (fixed bound, about a second).
-        if (warp == kMmaWarp && lane == 0 && rank == 0) {
-            if (PAIR) tc_commit2(smem_u32(&bars.drain));
-            else tc_commit(smem_u32(&bars.drain));
+        if ((warp == kMmaWarp || warp == kPvWarp) && rank == 0) {
+            if (elect_one()) {
+                if (PAIR) tc_commit2(smem_u32(&bars.drain));
+                else tc_commit(smem_u32(&bars.drain));
+            }
+            __syncwarp();
             mbar_drain(smem_u32(&bars.drain), 0);
         }
         if (warp == kVWarp && lane == 0) {

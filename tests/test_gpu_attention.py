@@ -348,3 +348,21 @@ def test_full_size_tree_keys_dominate(mode, B, Hq, Hkv, lens):
     for t, (b, h, i) in enumerate(samples):
         # outputs reach |o| ~ 3 here, where bf16 steps are 2^-6: the bar scales with rows above 1
         assert np.abs(got[b, i, h] - want[t]).max() <= TOL * max(1.0, np.abs(want[t]).max())
+
+
+@pytest.mark.parametrize("tiles", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("m,Hkv,Hq,d", [(16, 4, 4, 64), (60, 4, 16, 64), (16, 4, 4, 128), (60, 4, 16, 128)])
+def test_references_that_grow_with_every_tile(m, Hkv, Hq, d, tiles):
+    """One to five tiles on one block, of one and of two row tiles: every tile's largest scores lie far above those of
+    the tile before, so that each P.V's result is rescaled before the next is added."""
+    B, L = 30, tiles * 128 - m - 3
+    q, kc, vc, off, kl, bits = _inputs(91, B, m, Hq, Hkv, d, [L] * B)
+    assert attention_mode(B, m, Hq, Hkv, d, L) == "no partial rows in memory"
+    k = gen.bf16_bits_to_f32(kc)
+    for b in range(B):
+        n = L + m
+        k[off[b]:off[b] + n] *= (1.0 + 4.0 * (np.arange(n) // 128))[:, None, None]
+    kc = gen.f32_to_bf16_bits(k)
+    rng = np.random.default_rng(9)
+    samples = np.stack([rng.integers(0, B, 300), rng.integers(0, Hq, 300), rng.integers(0, m, 300)], axis=1).astype(np.int32)
+    _compare(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), samples=samples)
