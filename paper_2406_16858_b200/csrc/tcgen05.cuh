@@ -281,8 +281,11 @@ __device__ __forceinline__ void cluster_sync_all() {
 // The same meeting without memory ordering: for points where the blocks only have to have arrived
 // (nothing written before it is read after it by the other block).  The releasing form waits for
 // the block's earlier stores to be performed, which after an epilogue's global stores costs ~0.6 us.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_relaxed() {
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+    cluster_arrive_relaxed();
+    cluster_wait();
 }
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;

@@ -86,7 +86,7 @@ struct AttnPlan {
     int fused_merge;  // 1 (ordered launches with several splits): the last block of a (sequence, KV head, row
                       // block) to finish combines the splits' partials itself, while other blocks still run
     int tile_tok;   // query rows by TMA: tree tokens per 128-row tile
-    FastDiv by_g, by_splits, by_n_rb, by_hkv, by_per_split;
+    FastDiv by_g, by_splits, by_n_rb, by_hkv, by_per_split, by_own;
     size_t smem;
     long long wait_limit;  // bound of every device-side wait of the launch, in clock cycles
 };
@@ -218,7 +218,7 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
 static void attention_plan(int B, int m, int Hq, int Hkv, int d, int max_kv_len, AttnPlan* p) {
     attention_plan_sizes(B, m, Hq, Hkv, d, max_kv_len, true, p);
     p->by_g = FastDiv(p->g), p->by_splits = FastDiv(p->splits), p->by_n_rb = FastDiv(p->n_rb), p->by_hkv = FastDiv(Hkv);
-    p->by_per_split = FastDiv(p->per_split);
+    p->by_per_split = FastDiv(p->per_split), p->by_own = FastDiv(p->own > 0 ? p->own : 1);
     p->tile_tok = kRowsPerTile / p->g;
 }
 
@@ -325,6 +325,7 @@ struct AttnBarriers {
     // pair mode, used in the pair's first block: the other block's query tile / K half / V half
     // has landed (and its V tail is cleared)
     unsigned long long q_peer, k_peer[kMaxStages], v_peer[kMaxStages];
+    unsigned long long v_go;     // the block's part of the first K tile has landed: V tiles may be requested
     unsigned long long v_clean;  // the last V tile's rows past the sequence's last key are cleared
     // cluster launches: every block's query tiles may be overwritten by partial rows / they have arrived here
     unsigned long long peers_ready, inbox;
@@ -543,6 +544,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     // columns: its accumulator (head_dim 128), which nothing has written yet, or columns that nothing else uses.
     constexpr uint32_t kPCol = kTK, kPCols = kTK / 2, kOCol = kPCol + 2 * kPCols, kSCol1 = kTmemCols - kTK;
     constexpr uint32_t kRowBytes = DH * 2;
+    constexpr uint32_t kPanels = MT == 2 ? 1 : 2, kPanelRow = kRowBytes / kPanels;  // cluster launches: partial rows by the columns of a warp
     // bytes a block holds of one K tile and of one V tile (a pair splits K by keys, V by columns)
     constexpr uint32_t kKPanel = PAIR ? kPanel / 2 : kPanel, kKTile = HALVES * kKPanel;
     constexpr uint32_t kVTile = PAIR ? kPanel : kTile;
@@ -602,7 +604,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             if (PAIR) mbar_init(smem_u32(&bars.q_peer), 1);
             mbar_init(smem_u32(&bars.drain), 2);  // (each issuing warp's commit covers its own instructions)
             mbar_init(smem_u32(&bars.v_clean), 1);
-            if (CL) mbar_init(smem_u32(&bars.peers_ready), plan.cluster), mbar_init(smem_u32(&bars.inbox), 1);
+            if (PAIR) mbar_init(smem_u32(&bars.v_go), 1);
+            if (CL) mbar_init(smem_u32(&bars.peers_ready), plan.cluster), mbar_init(smem_u32(&bars.inbox), 1 + kSoftmaxThreads / 32);
             fence_barrier_init();
         }
         if (warp == kMmaWarp) {
@@ -619,9 +622,17 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             asm volatile("prefetch.tensormap [%0];" ::"l"(&v_map) : "memory");
             if (plan.q_tma) asm volatile("prefetch.tensormap [%0];" ::"l"(&q_map) : "memory");
         }
+    };
+    // All blocks' barriers exist before any signals another: a pair meets at once (its second block signals as soon as its
+    // first tile is there); a cluster's blocks signal one another after their last scores, so that they arrive here and
+    // wait (in the softmax warps before their first scores, in the others after their work).  The barriers were
+    // made visible by the fence behind their initialisation, so that the meeting need not order memory (the
+    // releasing form took 0.5 us of the 1.1 us before a launch's first request).
+    auto meet = [&]() {
         tc_fence_before();
-        if (PAIR || CL) cluster_sync_all();  // all blocks' barriers exist before any signals another
+        if (PAIR) cluster_sync_all();
         else __syncthreads();
+        if (CL) cluster_arrive_relaxed();
         tc_fence_after();
     };
     if (plan.setup_first) set_up();
@@ -677,6 +688,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     // a split past the sequence's last tile (never merged), or a rejected sequence: both blocks of a
     // pair take the same decision
     const bool active = nt > 0 && rows_blk > 0;
+    if (plan.setup_first) meet();
     if (early_len) {
         chain_wait();
         chain_release();
@@ -684,14 +696,15 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     if (!plan.setup_first) {
         if (CL ? overflow : !active) return;  // (all blocks of a cluster leave or stay together)
         set_up();
+        meet();
     }
     const uint32_t tmem = s_tmem_base;
     volatile WaitCtl* abort_flag = &s_ctl;
-    // Cluster launches: block j combines the rows [j * own, (j + 1) * own) of the row block; rows_of(j) of
-    // them exist (to the next even number: row pairs travel together).
+    // Cluster launches: block j combines the rows [j * own, (j + 1) * own) of the row block; rows_of(j) of them exist
+    // (to the next even number: row pairs travel together).  The inbox barrier counts what the other blocks' copies
+    // bring and this block's own softmax warps.
     auto rows_of = [&](int j) { return min(max(((rows_blk + 1) & ~1) - j * plan.own, 0), plan.own); };
-    if (CL && tid == 0 && !overflow) mbar_expect_tx(smem_u32(&bars.inbox), (uint32_t)(S_b * rows_of(split)) * (kRowBytes + 8));
-    bool softmax_ok = true;
+    if (CL && tid == 0 && !overflow) mbar_expect_tx(smem_u32(&bars.inbox), (uint32_t)((S_b - (active ? 1 : 0)) * rows_of(split)) * (kRowBytes + 8));
     int k_issued = 0, v_issued = 0;  // TMA lane: K and V tiles requested so far
     const int n_items = nt * MT;  // item i = (tile i / MT, row tile i % MT), group i % 2
     // The only tile of this block that can reach past the sequence's last key is its last one.  Its P.V covers
@@ -739,9 +752,13 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                                     b * m + rb * plan.per_tok + (t + (int)rank) * (int)plan.tile_tok, hk,
                                     smem_u32(&bars.q_full));
             }
+            // A pair's first scores need both blocks' queries and halves of a K tile, and what else is on its way delays
+            // them: 12000 keys, 8 query / 2 KV heads 15.5 -> 14.9 us per layer with V asked for behind them.  Without
+            // pairs the V tiles come late then (50 rows, 40 heads 26.9 -> 27.4 us).
+            if (PAIR) ok = mbar_wait(smem_u32(&bars.v_go), 0, abort_flag);
             int row = (int)(row_base + (long long)t_begin * kTK);
             for (int j = 0; j < nt; ++j, row += kTK) {
-                if (j >= NST) ok = mbar_wait(smem_u32(&bars.v_empty[st]), ph, abort_flag);
+                if (j >= NST) ok = ok && mbar_wait(smem_u32(&bars.v_empty[st]), ph, abort_flag);
                 if (!ok) break;
                 mbar_expect_tx(smem_u32(&bars.v_full[st]), kVTile);
                 if (PAIR) {  // all keys, this block's 64 of the 128 columns
@@ -798,6 +815,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.q_peer), 0);
                 for (int j = 0; j < nt && ok; ++j) {
                     ok = wait1(smem_u32(&bars.k_full[st]), ph);
+                    if (j == 0 && lane == 0) mbar_arrive(smem_u32(&bars.v_go));
                     if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.k_peer[st]), 0);
                     if (++st == NST) st = 0, ph ^= 1u;
                 }
@@ -809,6 +827,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                     const int t = i & (MT - 1);
                     if (t == 0) {
                         ok = ok && wait1(smem_u32(&bars.k_full[st]), ph);
+                        if (PAIR && i == 0 && lane == 0) mbar_arrive(smem_u32(&bars.v_go));
                         if (PAIR) ok = ok && wait1(smem_u32(&bars.k_peer[st]), ph);
                     }
                     // (item 0 has been read before item 2 overwrites it, item i - 1 before item i; item 1 has columns of its own)
@@ -888,6 +907,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         // reference maximum, row sums and accumulator, and the epilogue combines the two.  A thread owns a
         // row: its 128 scores stay in registers from the tensor-memory read to the packed probabilities, so
         // nothing is read twice and no two threads exchange anything.
+        if (CL) cluster_wait();  // (the meeting of the cluster's blocks, see above)
         __shared__ float2 s_half[2][128];                 // epilogue, one row tile: [group][row] (reference, sum)
         const int grp = warp >> 2, quad = warp & 3;
         const int r_tile = (quad << 5) | lane;            // row inside the tile = tensor-memory lane
@@ -1032,9 +1052,9 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         const int n_uses = (n_items - grp + 1) / 2;  // items this group served
         if (ok && n_uses > 0)
             ok = mbar_wait(smem_u32(&bars.o_done[grp]), (uint32_t)((n_uses - 1) & 1), abort_flag);
+        if (CL) ok = ok && mbar_wait(smem_u32(&bars.peers_ready), 0, abort_flag);
         if (MT == 1) s_half[grp][r_tile] = make_float2(m_ref, l_run);
         ok = named_barrier_and(1, kSoftmaxThreads, ok);
-        softmax_ok = ok;
         if (ok) {
             tc_fence_after();
             constexpr int NCOL = MT == 2 ? DH : DH / 2;  // columns of an output row this thread produces
@@ -1052,42 +1072,47 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 m_tot = fmaxf(h0.x, h1.x);
                 w0 = h0.x == -INFINITY ? 0.f : ex2(h0.x - m_tot), w1 = h1.x == -INFINITY ? 0.f : ex2(h1.x - m_tot);
                 l_tot = h0.y * w0 + h1.y * w1;
-                if (n_items < 2) w1 = 0.f;  // accumulator 1 was never written
             }
             // final rows are normalised here; a partial stays unnormalised (the merge divides by the
             // combined sum) and is rounded to bf16 once, like a final row
             const float inv = !direct ? 1.f : (l_tot > 0.f ? 1.f / l_tot : 0.f);
             w0 *= inv, w1 *= inv;
-            // (a cluster's rows are staged in the V ring, which nothing reads any more: the peers' partial
-            // rows may be arriving where the queries were)
-            unsigned char* srow = smem_gen + (CL ? sV - smem_base : 0u) + (size_t)r_blk * kRowBytes;
+            // Rows are staged in shared memory: where the queries were, or, those of a cluster, in the V ring, which nothing
+            // reads any more, as panels of the columns that one warp writes, and those that this block itself combines
+            // where the other blocks' parts of them arrive.
+            const int own_j = CL ? plan.by_own.div(r_blk) : 0, own_i = r_blk - own_j * plan.own;
+            unsigned char* srow = smem_gen + (size_t)r_blk * kRowBytes;
+            if (CL) srow = own_j == split ? smem_gen + (size_t)((split * kPanels + (MT == 2 ? 0 : grp)) * plan.own + own_i) * kPanelRow
+                                          : smem_gen + (sV - smem_base) + (size_t)((MT == 2 ? 0 : grp) * (MT * 128) + r_blk) * kPanelRow;
             const uint32_t o_row = tmem + lane_sel + kOCol + (MT == 2 ? (uint32_t)grp * DH : 0u) + (uint32_t)col0;
+            uint32_t oa[NCOL / 32][32], ob[MT == 1 ? NCOL / 32 : 1][32];
 #pragma unroll
-            for (int c0 = 0; c0 < NCOL; c0 += 32) {
-                uint32_t oa[32], ob[32];
-                tmem_ld32(o_row + c0, oa);
-                if (MT == 1) tmem_ld32(o_row + DH + c0, ob);
-                tc_wait_ld(oa);
-                if (MT == 1) tc_wait_ld(ob);
+            for (int c = 0; c < NCOL / 32; ++c) {
+                tmem_ld32(o_row + c * 32, oa[c]);
+                if (MT == 1) tmem_ld32(o_row + DH + c * 32, ob[c]);
+            }
+#pragma unroll
+            for (int c0 = 0; c0 < NCOL / 32; ++c0) {
+                tc_wait_ld(oa[c0]);
+                if (MT == 1) tc_wait_ld(ob[c0]);
 #pragma unroll
                 for (int c = 0; c < 32; c += 8) {
-                    float v[8];
+                    uint32_t x[4];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        v[e] = __uint_as_float(oa[c + e]) * w0;
-                        if (MT == 1) {
-                            if (w0 == 0.f) v[e] = 0.f;
-                            if (w1 != 0.f) v[e] = fmaf(__uint_as_float(ob[c + e]), w1, v[e]);
-                        }
+                    for (int e = 0; e < 8; e += 2) {
+                        float2 v = __fmul2_rn(make_float2(__uint_as_float(oa[c0][c + e]), __uint_as_float(oa[c0][c + e + 1])), make_float2(w0, w0));
+                        if (MT == 1 && n_items > 1)  // (a single item leaves accumulator 1 unwritten)
+                            v = __ffma2_rn(make_float2(__uint_as_float(ob[c0][c + e]), __uint_as_float(ob[c0][c + e + 1])), make_float2(w1, w1), v);
+                        x[e >> 1] = pack_bf16(v.x, v.y);
                     }
-                    const int chunk = (col0 + c0 + c) >> 3;
-                    *reinterpret_cast<uint4*>(srow + (((chunk ^ r_tile) & cmask) << 4)) =
-                        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+                    const int chunk = ((CL ? 0 : col0) + c0 * 32 + c) >> 3;
+                    *reinterpret_cast<uint4*>(srow + (((chunk ^ r_tile) & (CL ? kPanelRow / 16 - 1 : cmask)) << 4)) = make_uint4(x[0], x[1], x[2], x[3]);
                 }
             }
             if (MT == 2 || grp == 0) {
                 if (CL) {
-                    s_ml[r_blk] = make_float2(m_tot, l_tot);
+                    if (own_j == split) s_ml_in[split * plan.own + own_i] = make_float2(m_tot, l_tot);
+                    else s_ml[r_blk] = make_float2(m_tot, l_tot);
                 } else if (r_blk < rows_here) {
                     if (!direct) {
                         ws.ml[part_row0 + r_blk] = make_float2(m_tot, l_tot);
@@ -1097,8 +1122,22 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                     }
                 }
             }
-            if (CL) fence_proxy_async();  // the copies to the peers read what was staged
-            asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");  // rows are staged
+            if (CL) {  // this warp's rows set off, a lane per block that combines some of them
+                fence_proxy_async();
+                __syncwarp();
+                const int w0r = t_own * 128 + quad * 32, lo = max(w0r, lane * plan.own), hi = min(w0r + 32, lane * plan.own + rows_of(lane));
+                if (lane < S && lane != split && hi > lo) {
+                    const uint32_t bar = in_block(smem_u32(&bars.inbox), (uint32_t)lane), pan = MT == 2 ? 0u : (uint32_t)grp;
+                    bulk_copy_to(in_block(sQ + (uint32_t)((split * kPanels + pan) * plan.own + lo - lane * plan.own) * kPanelRow, (uint32_t)lane),
+                                 sV + (pan * (MT * 128) + (uint32_t)lo) * kPanelRow, (uint32_t)(hi - lo) * kPanelRow, bar);
+                    if (MT == 2 || grp == 0)
+                        bulk_copy_to(in_block(smem_u32(s_ml_in + split * plan.own + lo - lane * plan.own), (uint32_t)lane), smem_u32(s_ml + lo),
+                                     (uint32_t)(hi - lo) * 8u, bar);
+                }
+                if (lane == 0) mbar_arrive(smem_u32(&bars.inbox));
+            } else {
+                asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");  // rows are staged
+            }
             if (!CL) {
                 constexpr int lanes_per_row = kRowBytes / 16;       // 16 lanes (8 for a 64-wide bf16 row)
                 constexpr int rows_per_pass = 32 / lanes_per_row;
@@ -1117,78 +1156,30 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         }
     }
     }  // active
-
-    // ---- cluster launches: every block sends each peer the partial rows that peer combines, as bulk copies from
-    // shared memory to shared memory, and combines its own share when all have arrived.  (The alternative,
-    // partial rows through L2 and a second launch that combines them, costs that launch's start and a cold
-    // pass through its code.)
-    if (CL && !overflow && warp < kTmaWarp) {
-        if (!active) {
-            if (warp == 0 && lane < S) mbar_arrive_in(smem_u32(&bars.peers_ready), (uint32_t)lane);
-        } else if (softmax_ok && warp < S && lane == 0 && mbar_wait(smem_u32(&bars.peers_ready), 0, abort_flag)) {
-            const int j = warp, n = rows_of(j);  // a warp per peer
-            if (n > 0) {
-                const uint32_t bar = in_block(smem_u32(&bars.inbox), (uint32_t)j);
-                bulk_copy_to(in_block(sQ + (uint32_t)(split * plan.own) * kRowBytes, (uint32_t)j),
-                             sV + (uint32_t)(j * plan.own) * kRowBytes, (uint32_t)n * kRowBytes, bar);
-                bulk_copy_to(in_block(smem_u32(s_ml_in + split * plan.own), (uint32_t)j), smem_u32(s_ml + j * plan.own),
-                             (uint32_t)n * 8u, bar);
-            }
-        }
+    if (CL && !(active && warp < kTmaWarp)) {
         __syncwarp();
-        const int n_own = min(rows_of(split), rows_blk - split * plan.own);
-        // Four rows per warp side by side: lane 8 r + s weighs part s of row r, then the warp goes over the rows with
-        // DH / 4 lanes each (four columns a lane).  (One row at a time was 0.65 us a row of dependent steps.)
-        if (softmax_ok && n_own > 0 && mbar_wait(smem_u32(&bars.inbox), 0, abort_flag)) {
-            constexpr int R = 4, LPR = DH / 4, RPW = 32 / LPR, Q = R / RPW, W = kSoftmaxThreads / 32;
-            const int part = lane & 7, c4 = lane % LPR;
-            // did block `part` have tiles
-            const bool have = part < S && plan.by_splits.div(tiles * (part + 1)) > plan.by_splits.div(tiles * part);
-            const unsigned parts = __ballot_sync(0xffffffffu, have);
-            for (int i0 = warp; i0 < n_own; i0 += W * R) {  // rows i0, i0 + W, ...: few rows are a row per warp
-                const float2 ml = have ? s_ml_in[part * plan.own + min(i0 + (lane >> 3) * W, n_own - 1)] : make_float2(-INFINITY, 0.f);
-                uint2 v[Q][kMaxCluster];
-#pragma unroll
-                for (int qq = 0; qq < Q; ++qq) {
-                    const int i = min(i0 + (qq * RPW + lane / LPR) * W, n_own - 1), r = split * plan.own + i;
-                    const unsigned char* src = smem_gen + (size_t)i * kRowBytes + ((((c4 >> 1) ^ r) & (DH / 8 - 1)) << 4) + (c4 & 1) * 8;
-#pragma unroll
-                    for (int s2 = 0; s2 < kMaxCluster; ++s2) {
-                        v[qq][s2] = make_uint2(0u, 0u);
-                        if (((parts >> s2) & 1u) && i0 + qq * RPW * W < n_own) v[qq][s2] = *reinterpret_cast<const uint2*>(src + (size_t)(s2 * plan.own) * kRowBytes);
-                    }
-                }
-                float mmax = ml.x;
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
-                float w = ml.x == -INFINITY ? 0.f : ex2(ml.x - mmax), l = ml.y * w;
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-                w *= l > 0.f ? 1.f / l : 0.f;
-#pragma unroll
-                for (int qq = 0; qq < Q; ++qq) {
-                    if (i0 + qq * RPW * W >= n_own) break;
-                    const int rr = qq * RPW + lane / LPR, i = i0 + rr * W;
-                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int s2 = 0; s2 < kMaxCluster; ++s2) {
-                        if (s2 >= S) continue;
-                        const float ws2 = __shfl_sync(0xffffffffu, w, rr * 8 + s2);
-                        acc[0] = fmaf(__uint_as_float(v[qq][s2].x << 16), ws2, acc[0]), acc[1] = fmaf(__uint_as_float(v[qq][s2].x & 0xffff0000u), ws2, acc[1]);
-                        acc[2] = fmaf(__uint_as_float(v[qq][s2].y << 16), ws2, acc[2]), acc[3] = fmaf(__uint_as_float(v[qq][s2].y & 0xffff0000u), ws2, acc[3]);
-                    }
-                    const float m_row = __shfl_sync(0xffffffffu, mmax, rr * 8), l_row = __shfl_sync(0xffffffffu, l, rr * 8);
-                    const int pr = rb * plan.per + split * plan.own + i, tok = plan.by_g.div(pr), hq = hk * g + (pr - tok * g);
-                    if (i < n_own) {
-                        *reinterpret_cast<uint2*>(out + (((long long)b * m + tok) * Hq + hq) * DH + c4 * 4) =
-                            make_uint2(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]));
-                        if (lse && c4 == 0) lse[((long long)b * Hq + hq) * m + tok] = (m_row + log2f(l_row)) * 0.69314718055994531f;
-                    }
-                }
-            }
-        }
+        cluster_wait();
     }
 
+    // ---- cluster launches: every block combines its share of the rows when all blocks' parts of them have arrived.
+    // What bounds it: the copies between the blocks, at ~30 bytes per ns and block (120 rows of 128 columns 1.2 us from the
+    // last block's last row, 60 rows 0.5 us), and the block-wide steps around them.  From the last P.V to the last store, 120
+    // rows on six blocks: 3.4 us, of which 0.8 us waiting for a block with one tile more; it was 4.5 us while all rows were
+    // staged before the first copy set off, the block's own among them, and the cluster met behind the last store.  Rows
+    // stored by the softmax warps straight to the blocks that combine them leave at half that rate (2.2 us); partial
+    // rows through L2 and a second launch that combines them cost that launch's start and a cold pass through its code.
+    int n_own = 0;         // rows that this block combines
+    unsigned parts = 0;    // blocks that had tiles
+    if (CL && !overflow) {
+        if (!active) {
+            if (warp == 0 && lane < S) mbar_arrive_in(smem_u32(&bars.peers_ready), (uint32_t)lane);
+            if (warp < kTmaWarp && lane == 0) mbar_arrive(smem_u32(&bars.inbox));
+        }
+        n_own = max(0, min(plan.own, rows_blk - split * plan.own));
+        const int part = lane & (kMaxCluster - 1);
+        parts = __ballot_sync(0xffffffffu, part < S && plan.by_splits.div(tiles * (part + 1)) > plan.by_splits.div(tiles * part));
+        if (n_own > 0 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.inbox), 0, abort_flag))) n_own = 0;
+    }
     // ---- merging launches: whoever finishes a (sequence, KV head, row block) last combines its splits
     // (a pair's blocks count and merge on their own, each for its 128 rows)
     if (plan.fused_merge && !direct) {  // uniform over the block; blocks without tiles left long ago
@@ -1224,9 +1215,58 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         asm volatile("fence.acq_rel.cluster;" ::: "memory");  // the flag is the one thing the meeting below hands over
     }
     tc_fence_before();
-    // (a pair releases its tensor memory together; the blocks of a cluster have all received what they wait for)
-    if (PAIR || (CL && !overflow)) cluster_sync_relaxed();
-    else __syncthreads();
+    // (a pair releases its tensor memory together; a cluster's blocks stay until all have received what they wait for,
+    // and combine meanwhile)
+    if (CL && !overflow) {
+        cluster_arrive_relaxed();
+        if (n_own > 0) {
+            // A thread per 16 bytes of an output row; every part's (maximum, sum) and bytes are fetched before any is used.
+            // (0.8 us, by its instructions: a loop over the parts, short as it is, takes 1.5 us of dependent steps, a warp
+            // per four rows that shares out the weights by shuffles 1.5 us.)
+            constexpr int CPR = DH / 8, CPP = kPanelRow / 16;  // 16-byte chunks of a row, of its part in one panel
+            for (int it = tid; it < n_own * CPR; it += kAttnThreads) {
+                const int i = it / CPR, c = it % CPR, r = split * plan.own + i;
+                const unsigned char* src = smem_gen + (size_t)(c / CPP * plan.own + i) * kPanelRow + (((c ^ r) & (CPP - 1)) << 4);
+                uint4 v[kMaxCluster];
+                float2 ml[kMaxCluster];
+#pragma unroll
+                for (int s2 = 0; s2 < kMaxCluster; ++s2) {
+                    ml[s2] = make_float2(-INFINITY, 0.f), v[s2] = make_uint4(0u, 0u, 0u, 0u);
+                    if ((parts >> s2) & 1u) {
+                        ml[s2] = s_ml_in[s2 * plan.own + i];
+                        v[s2] = *reinterpret_cast<const uint4*>(src + (size_t)(s2 * plan.own) * kRowBytes);
+                    }
+                }
+                float mmax = ml[0].x, l = 0.f;
+#pragma unroll
+                for (int s2 = 1; s2 < kMaxCluster; ++s2) mmax = fmaxf(mmax, ml[s2].x);
+                float2 acc[4] = {};
+#pragma unroll
+                for (int s2 = 0; s2 < kMaxCluster; ++s2) {
+                    if (!((parts >> s2) & 1u)) continue;  // (uniform)
+                    const float w = ml[s2].x == -INFINITY ? 0.f : ex2(ml[s2].x - mmax);
+                    l = fmaf(ml[s2].y, w, l);
+                    const float2 w2 = make_float2(w, w);
+                    const uint32_t x[4] = {v[s2].x, v[s2].y, v[s2].z, v[s2].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        acc[e] = __ffma2_rn(make_float2(__uint_as_float(x[e] << 16), __uint_as_float(x[e] & 0xffff0000u)), w2, acc[e]);
+                }
+                const float inv = l > 0.f ? 1.f / l : 0.f;
+                const int pr = rb * plan.per + r, tok = plan.by_g.div(pr), hq = hk * g + (pr - tok * g);
+                *reinterpret_cast<uint4*>(out + (((long long)b * m + tok) * Hq + hq) * DH + c * 8) =
+                    make_uint4(pack_bf16(acc[0].x * inv, acc[0].y * inv), pack_bf16(acc[1].x * inv, acc[1].y * inv),
+                               pack_bf16(acc[2].x * inv, acc[2].y * inv), pack_bf16(acc[3].x * inv, acc[3].y * inv));
+                if (lse && c == 0) lse[((long long)b * Hq + hq) * m + tok] = (mmax + log2f(l)) * 0.69314718055994531f;
+            }
+        }
+        __syncwarp();
+        cluster_wait();
+    } else if (PAIR) {
+        cluster_sync_relaxed();
+    } else {
+        __syncthreads();
+    }
     tc_fence_after();
     if (s_ctl.abort) {
         // Whoever gave up, and whenever: the tensor instructions issued so far may still read shared
@@ -1246,7 +1286,6 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 mbar_drain(smem_u32(&bars.v_full[j % NST]), (uint32_t)((j / NST) & 1));
         }
         if (warp == kTmaWarp && lane == 0) {
-            if (CL) mbar_drain(smem_u32(&bars.inbox), 0);  // what peers have sent may still be on its way
             for (int j = max(0, k_issued - NST); j < k_issued; ++j)
                 mbar_drain(smem_u32(&bars.k_full[j % NST]), (uint32_t)((j / NST) & 1));
         }
