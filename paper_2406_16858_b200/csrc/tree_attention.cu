@@ -455,74 +455,66 @@ __device__ __forceinline__ void merge_row(const AttnPlan& plan, const AttnWs& ws
         lse[((long long)b * Hq + hq) * m + tok] = (mmax + log2f(l)) * 0.69314718055994531f;
 }
 
-// The same combination for R consecutive packed rows of one row block at once, when the sequence has
-// at most SB splits (R * SB <= 16): a block that merges its 128 or 256 rows by itself has few warps and
-// many rows, and one row at a time is one memory round trip per row.  Lane rr * SB + s fetches the
-// (maximum, sum) pair of row rr in split s; every lane fetches its DH/32 columns of all R * SB partial
-// rows before it uses any; the splits are added in the same order as in merge_row.
-template <int DH, int R, int SB>
-__device__ __forceinline__ void merge_rows_wide(const AttnPlan& plan, const AttnWs& ws, int b, int hk, int pr0, int n,
-                                                int S_b, int m, int Hq, int Hkv, __nv_bfloat16* __restrict__ out,
-                                                float* __restrict__ lse) {
-    static_assert(R * SB <= 16 && (SB & (SB - 1)) == 0, "sixteen partial rows in flight per lane");
-    const int lane = threadIdx.x & 31;
-    const int g = plan.g, S = plan.splits;
-    const int rb = pr0 / plan.per, r0 = pr0 % plan.per;
-    const size_t rows_per_block = (size_t)plan.mt * kRowsPerTile;
-    const size_t stride = (size_t)plan.n_rb * rows_per_block;  // rows between consecutive splits
-    const size_t first = (((size_t)b * Hkv + hk) * S) * stride + rb * rows_per_block + r0;
-    constexpr int PER = DH / 32;  // 4 or 2 consecutive columns per lane
-    const int rr_l = lane / SB, s_l = lane % SB;
-    const bool have = lane < R * SB && rr_l < n && s_l < S_b;
-    const float2 ml = have ? __ldcg(ws.ml + first + rr_l + (size_t)s_l * stride) : make_float2(-INFINITY, 0.f);
-    uint2 v[R][SB];
+// Eight columns of an output row from its parts: (reference maximum in log2 units, sum) and bf16 columns of each part
+// whose bit in `parts` is set (uniform over the warp).
+template <int W>
+__device__ __forceinline__ uint4 combine_parts(const float2 (&ml)[W], const uint4 (&v)[W], unsigned parts, float& mmax, float& l) {
+    mmax = -INFINITY, l = 0.f;
 #pragma unroll
-    for (int rr = 0; rr < R; ++rr)
+    for (int s = 0; s < W; ++s)
+        if ((parts >> s) & 1u) mmax = fmaxf(mmax, ml[s].x);
+    float2 acc[4] = {};
 #pragma unroll
-        for (int sp = 0; sp < SB; ++sp) {
-            v[rr][sp] = make_uint2(0u, 0u);
-            if (rr < n && sp < S_b) {
-                const __nv_bfloat16* src = ws.o_part + (first + rr + (size_t)sp * stride) * DH + lane * PER;
-                if (PER == 4) v[rr][sp] = __ldcg(reinterpret_cast<const uint2*>(src));
-                else v[rr][sp].x = __ldcg(reinterpret_cast<const uint32_t*>(src));
-            }
-        }
-    float mx = ml.x;
+    for (int s = 0; s < W; ++s) {
+        if (!((parts >> s) & 1u)) continue;
+        const float w = ml[s].x == -INFINITY ? 0.f : ex2(ml[s].x - mmax);
+        l = fmaf(ml[s].y, w, l);
+        const float2 w2 = make_float2(w, w);
+        const uint32_t x[4] = {v[s].x, v[s].y, v[s].z, v[s].w};
 #pragma unroll
-    for (int o = SB / 2; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    // a split without visible keys leaves its partial row unwritten: weight 0, never multiplied
-    const float w = (have && ml.x != -INFINITY) ? exp2f(ml.x - mx) : 0.f;
-    float lw = w != 0.f ? ml.y * w : 0.f;
+        for (int e = 0; e < 4; ++e)
+            acc[e] = __ffma2_rn(make_float2(__uint_as_float(x[e] << 16), __uint_as_float(x[e] & 0xffff0000u)), w2, acc[e]);
+    }
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    return make_uint4(pack_bf16(acc[0].x * inv, acc[0].y * inv), pack_bf16(acc[1].x * inv, acc[1].y * inv),
+                      pack_bf16(acc[2].x * inv, acc[2].y * inv), pack_bf16(acc[3].x * inv, acc[3].y * inv));
+}
+
+// A block combines its n rows (packed rows row0, row0 + 1, ...; partial rows part0, part0 + 1, ... of the first split)
+// from S_b <= W splits: a thread per 16 bytes of an output row, R of them at a time, everything fetched before any of it
+// is used.  Bound by the trips to L2, with up to 18 fetches of 16 bytes in flight per thread: 128 rows of five splits 1.7 us
+// (a warp per two rows, 8 bytes a lane, took 10 us, at the end of the launch).
+template <int DH, int W, int R>
+__device__ __forceinline__ void merge_block(const AttnPlan& plan, const AttnWs& ws, size_t part0, int b, int hk, int row0, int n,
+                                            int S_b, int m, int Hq, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
+    constexpr int CPR = DH / 8;
+    const size_t stride = (size_t)plan.n_rb * plan.mt * kRowsPerTile;  // rows between consecutive splits
+    const int total = n * CPR;
+#pragma unroll 1
+    for (int it0 = threadIdx.x; it0 < total; it0 += R * kAttnThreads) {
+        uint4 v[R][W];
+        float2 ml[R][W];
 #pragma unroll
-    for (int o = SB / 2; o >= 1; o >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o);
+        for (int q = 0; q < R; ++q) {
+            const int it = min(it0 + q * kAttnThreads, total - 1);
 #pragma unroll
-    for (int rr = 0; rr < R; ++rr) {
-        if (rr >= n) break;  // uniform over the warp
-        float acc[PER];
-#pragma unroll
-        for (int e = 0; e < PER; ++e) acc[e] = 0.f;
-#pragma unroll
-        for (int sp = 0; sp < SB; ++sp) {
-            const float wu = __shfl_sync(0xffffffffu, w, rr * SB + sp);
-            if (sp < S_b && wu != 0.f) {
-                acc[0] += __uint_as_float(v[rr][sp].x << 16) * wu;
-                acc[1] += __uint_as_float(v[rr][sp].x & 0xffff0000u) * wu;
-                if (PER == 4) {
-                    acc[PER - 2] += __uint_as_float(v[rr][sp].y << 16) * wu;
-                    acc[PER - 1] += __uint_as_float(v[rr][sp].y & 0xffff0000u) * wu;
+            for (int sp = 0; sp < W; ++sp)
+                if (sp < S_b) {
+                    const size_t row = part0 + it / CPR + (size_t)sp * stride;
+                    ml[q][sp] = __ldcg(ws.ml + row);
+                    v[q][sp] = __ldcg(reinterpret_cast<const uint4*>(ws.o_part + row * DH) + it % CPR);
                 }
-            }
         }
-        const float l = __shfl_sync(0xffffffffu, lw, rr * SB), mmax = __shfl_sync(0xffffffffu, mx, rr * SB);
-        const float inv = l > 0.f ? 1.f / l : 0.f;
-        const int pr = pr0 + rr;
-        const int tok = pr / g, hq = hk * g + pr % g;
-        __nv_bfloat16* dst = out + (((long long)b * m + tok) * Hq + hq) * DH + lane * PER;
 #pragma unroll
-        for (int e = 0; e < PER; e += 2)
-            *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16(acc[e] * inv, acc[e + 1] * inv);
-        if (lse && lane == 0)
-            lse[((long long)b * Hq + hq) * m + tok] = (mmax + log2f(l)) * 0.69314718055994531f;
+        for (int q = 0; q < R; ++q) {
+            const int it = it0 + q * kAttnThreads;
+            float mmax, l;
+            const uint4 packed = combine_parts<W>(ml[q], v[q], (1u << S_b) - 1u, mmax, l);
+            if (it >= total) break;
+            const int pr = row0 + it / CPR, tok = plan.by_g.div(pr), hq = hk * plan.g + (pr - tok * plan.g);
+            reinterpret_cast<uint4*>(out + (((long long)b * m + tok) * Hq + hq) * DH)[it % CPR] = packed;
+            if (lse && it % CPR == 0) lse[((long long)b * Hq + hq) * m + tok] = (mmax + log2f(l)) * 0.69314718055994531f;
+        }
     }
 }
 
@@ -722,6 +714,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         // stage is free long before the V stage of the same tile, and one lane that serves both in order would leave it
         // empty meanwhile ==========
         if (lane == 0) {
+            // (K and V pass through L2 once; what stays are queries, partial rows and code: 1-3 % per layer)
+            const uint64_t policy = evict_first_policy();
             int st = 0, row = (int)(row_base + (long long)t_begin * kTK);
             uint32_t ph = 1;
             for (int j = 0; j < nt; ++j, row += kTK) {
@@ -730,7 +724,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 #pragma unroll
                 for (int h = 0; h < HALVES; ++h)  // a pair block takes its 64 of the tile's 128 keys
                     tma_load_3d(sK + st * kKTile + h * kKPanel, &k_map, h * 64, hk, row + (int)rank * (kTK / 2),
-                                smem_u32(&bars.k_full[st]));
+                                smem_u32(&bars.k_full[st]), policy);
                 k_issued = j + 1;
                 if (++st == NST) st = 0, ph ^= 1u;
             }
@@ -756,17 +750,18 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             // them: 12000 keys, 8 query / 2 KV heads 15.5 -> 14.9 us per layer with V asked for behind them.  Without
             // pairs the V tiles come late then (50 rows, 40 heads 26.9 -> 27.4 us).
             if (PAIR) ok = mbar_wait(smem_u32(&bars.v_go), 0, abort_flag);
+            const uint64_t policy = evict_first_policy();
             int row = (int)(row_base + (long long)t_begin * kTK);
             for (int j = 0; j < nt; ++j, row += kTK) {
                 if (j >= NST) ok = ok && mbar_wait(smem_u32(&bars.v_empty[st]), ph, abort_flag);
                 if (!ok) break;
                 mbar_expect_tx(smem_u32(&bars.v_full[st]), kVTile);
                 if (PAIR) {  // all keys, this block's 64 of the 128 columns
-                    tma_load_3d(sV + st * kVTile, &v_map, (int)rank * 64, hk, row, smem_u32(&bars.v_full[st]));
+                    tma_load_3d(sV + st * kVTile, &v_map, (int)rank * 64, hk, row, smem_u32(&bars.v_full[st]), policy);
                 } else {
 #pragma unroll
                     for (int h = 0; h < HALVES; ++h)
-                        tma_load_3d(sV + st * kTile + h * kPanel, &v_map, h * 64, hk, row, smem_u32(&bars.v_full[st]));
+                        tma_load_3d(sV + st * kTile + h * kPanel, &v_map, h * 64, hk, row, smem_u32(&bars.v_full[st]), policy);
                 }
                 v_issued = j + 1;
                 last_st = st, last_ph = ph ^ 1u;
@@ -1182,24 +1177,23 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     }
     // ---- merging launches: whoever finishes a (sequence, KV head, row block) last combines its splits
     // (a pair's blocks count and merge on their own, each for its 128 rows)
-    if (plan.fused_merge && !direct) {  // uniform over the block; blocks without tiles left long ago
+    if (!CL && plan.fused_merge && !direct) {  // uniform over the block; blocks without tiles left long ago
         __shared__ int s_last;
         int* ticket = ws.tickets + (((size_t)b * Hkv + hk) * plan.n_rb + rb) * (PAIR ? 2 : 1) + rank;
         if (last_block_arrives(ticket, S_b, &s_last)) {
-            constexpr int NW = kAttnThreads / 32;
-            auto wide = [&](auto r_tag, auto s_tag) {
-                constexpr int R = decltype(r_tag)::value, SB = decltype(s_tag)::value;
-                for (int r = warp * R; r < rows_here; r += NW * R)
-                    merge_rows_wide<DH, R, SB>(plan, ws, b, hk, row0 + r, min(R, rows_here - r), S_b, m, Hq, Hkv, out, lse);
-            };
+            const size_t part0 = part_row0 - (size_t)split * plan.n_rb * (plan.mt * 128);
             if (S_b <= 2) {
-                wide(std::integral_constant<int, 8>{}, std::integral_constant<int, 2>{});
+                merge_block<DH, 2, 6>(plan, ws, part0, b, hk, row0, rows_here, S_b, m, Hq, out, lse);
             } else if (S_b <= 4) {
-                wide(std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{});
+                merge_block<DH, 4, 4>(plan, ws, part0, b, hk, row0, rows_here, S_b, m, Hq, out, lse);
+            } else if (S_b <= 6) {
+                merge_block<DH, 6, 3>(plan, ws, part0, b, hk, row0, rows_here, S_b, m, Hq, out, lse);
             } else if (S_b <= 8) {
-                wide(std::integral_constant<int, 2>{}, std::integral_constant<int, 8>{});
+                merge_block<DH, 8, 2>(plan, ws, part0, b, hk, row0, rows_here, S_b, m, Hq, out, lse);
+            } else if (S_b <= 16) {
+                merge_block<DH, 16, 1>(plan, ws, part0, b, hk, row0, rows_here, S_b, m, Hq, out, lse);
             } else {
-                for (int r = warp; r < rows_here; r += NW)
+                for (int r = warp; r < rows_here; r += kAttnThreads / 32)
                     merge_row<DH>(plan, ws, b, hk, row0 + r, S_b, m, Hq, Hkv, out, lse);
             }
         }
@@ -1230,33 +1224,15 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 uint4 v[kMaxCluster];
                 float2 ml[kMaxCluster];
 #pragma unroll
-                for (int s2 = 0; s2 < kMaxCluster; ++s2) {
-                    ml[s2] = make_float2(-INFINITY, 0.f), v[s2] = make_uint4(0u, 0u, 0u, 0u);
+                for (int s2 = 0; s2 < kMaxCluster; ++s2)
                     if ((parts >> s2) & 1u) {
                         ml[s2] = s_ml_in[s2 * plan.own + i];
                         v[s2] = *reinterpret_cast<const uint4*>(src + (size_t)(s2 * plan.own) * kRowBytes);
                     }
-                }
-                float mmax = ml[0].x, l = 0.f;
-#pragma unroll
-                for (int s2 = 1; s2 < kMaxCluster; ++s2) mmax = fmaxf(mmax, ml[s2].x);
-                float2 acc[4] = {};
-#pragma unroll
-                for (int s2 = 0; s2 < kMaxCluster; ++s2) {
-                    if (!((parts >> s2) & 1u)) continue;  // (uniform)
-                    const float w = ml[s2].x == -INFINITY ? 0.f : ex2(ml[s2].x - mmax);
-                    l = fmaf(ml[s2].y, w, l);
-                    const float2 w2 = make_float2(w, w);
-                    const uint32_t x[4] = {v[s2].x, v[s2].y, v[s2].z, v[s2].w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        acc[e] = __ffma2_rn(make_float2(__uint_as_float(x[e] << 16), __uint_as_float(x[e] & 0xffff0000u)), w2, acc[e]);
-                }
-                const float inv = l > 0.f ? 1.f / l : 0.f;
+                float mmax, l;
+                const uint4 packed = combine_parts<kMaxCluster>(ml, v, parts, mmax, l);
                 const int pr = rb * plan.per + r, tok = plan.by_g.div(pr), hq = hk * g + (pr - tok * g);
-                *reinterpret_cast<uint4*>(out + (((long long)b * m + tok) * Hq + hq) * DH + c * 8) =
-                    make_uint4(pack_bf16(acc[0].x * inv, acc[0].y * inv), pack_bf16(acc[1].x * inv, acc[1].y * inv),
-                               pack_bf16(acc[2].x * inv, acc[2].y * inv), pack_bf16(acc[3].x * inv, acc[3].y * inv));
+                *reinterpret_cast<uint4*>(out + (((long long)b * m + tok) * Hq + hq) * DH + c * 8) = packed;
                 if (lse && c == 0) lse[((long long)b * Hq + hq) * m + tok] = (mmax + log2f(l)) * 0.69314718055994531f;
             }
         }

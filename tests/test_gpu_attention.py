@@ -134,7 +134,9 @@ def test_ragged_batch_runs_longest_first_with_several_splits():
     (33, 8, 8, 64, 20, 6000),    # head_dim 64: deeper K/V ring, two splits for the longest sequences
     (40, 6, 2, 128, 80, 5000),   # three query heads per KV head: query rows copied by hand, not by TMA
     (60, 32, 8, 128, 8, 16384),  # few long sequences on block pairs: four and five splits merged inside the kernel
-    (60, 3, 1, 128, 37, 16384),  # short blocks: eight and nine splits per long sequence (nine: one row per warp at a time)
+    (60, 3, 1, 128, 37, 16384),  # short blocks: eight and nine splits per long sequence
+    (60, 32, 8, 128, 3, 16384),  # eleven and twelve splits
+    (8, 4, 4, 64, 3, 26000),     # more than sixteen splits: one row per warp at a time
 ])
 def test_ordered_launch_other_shapes(m, Hq, Hkv, d, B, longest):
     rng = np.random.default_rng(B + d)
