@@ -785,6 +785,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 if (lane == 0) mbar_arrive(smem_u32(&bars.v_clean));
             }
         }
+        __syncwarp();
     } else if (warp == kMmaWarp || warp == kPvWarp) {
         // ===== MMA issuers, a warp for Q.K^T and one for P.V: each walks its items in order and waits for nothing that
         // concerns the other.  The whole warp waits, one elected lane issues.  The loop's values are the same in all
@@ -1208,6 +1209,9 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(in_block(smem_u32(&s_ctl.abort), (uint32_t)r)), "r"(1u) : "memory");
         asm volatile("fence.acq_rel.cluster;" ::: "memory");  // the flag is the one thing the meeting below hands over
     }
+    // (The meetings and the release of tensor memory are instructions of whole warps, and the lanes of a warp that gives
+    // up come here one by one: each is preceded by a point where they wait for each other.)
+    __syncwarp();
     tc_fence_before();
     // (a pair releases its tensor memory together; a cluster's blocks stay until all have received what they wait for,
     // and combine meanwhile)
@@ -1254,7 +1258,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 else tc_commit(smem_u32(&bars.drain));
             }
             __syncwarp();
-            mbar_drain(smem_u32(&bars.drain), 0);
+            if (lane == 0) mbar_drain(smem_u32(&bars.drain), 0);
         }
         if (warp == kVWarp && lane == 0) {
             if (plan.q_tma) mbar_drain(smem_u32(&bars.q_full), 0);
@@ -1265,6 +1269,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             for (int j = max(0, k_issued - NST); j < k_issued; ++j)
                 mbar_drain(smem_u32(&bars.k_full[j % NST]), (uint32_t)((j / NST) & 1));
         }
+        __syncwarp();
         tc_fence_before();
         if (PAIR || CL) cluster_sync_all();
         else __syncthreads();
@@ -1275,6 +1280,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         else tmem_dealloc(tmem, kTmemCols);
     }
     if (tid == 0 && s_ctl.abort) raise_status(d_status, EAGLE2_STATUS_TIMEOUT);
+    __syncwarp();
     if (PAIR) cluster_sync_relaxed();  // neither block leaves while the other may still signal it
 }
 
