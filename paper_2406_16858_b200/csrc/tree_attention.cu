@@ -320,6 +320,10 @@ struct AttnBarriers {
     unsigned long long q_full;
     unsigned long long k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
     unsigned long long s_full[2], s_free;         // a group's scores are there / the scores' columns may be overwritten
+    // The scores of item 1, which have columns of their own, are there.  (A barrier of their own, too: s_free says that the
+    // item before has been read, so that no barrier of s_full runs two phases ahead of the group that waits for it; it says
+    // nothing of item 1.)
+    unsigned long long s_aside;
     unsigned long long p_first[2], p_full[2];     // first 32 keys' / all probabilities of a group
     unsigned long long o_done[2];                 // the group's P.V has completed
     // pair mode, used in the pair's first block: the other block's query tile / K half / V half
@@ -583,6 +587,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         } else if (tid >= 32 && tid < 34) {
             const int e = tid & 1;  // accumulator = group
             mbar_init(smem_u32(&bars.s_full[e]), 1);
+            if (e == 1) mbar_init(smem_u32(&bars.s_aside), 1);
             const uint32_t warps = (PAIR ? 2 : 1) * (kSoftmaxThreads / 64);  // one arrival per warp of a group
             mbar_init(smem_u32(&bars.p_first[e]), warps);
             mbar_init(smem_u32(&bars.p_full[e]), warps);
@@ -644,8 +649,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     if (plan.ordered) {  // item-major: the list says which (sequence, split) this block serves
         rb = take(bid, plan.by_n_rb);
         hk = take(bid, plan.by_hkv);
-        if (bid >= (int)ws.order[0]) return;  // (ordered launches set up after this point)
-        b = (int)ws.order[1 + bid];
+        if (bid >= (int)__ldcg(ws.order)) return;  // (ordered launches set up after this point)
+        b = (int)__ldcg(ws.order + 1 + bid);
         split = take(b, plan.by_splits);
     } else {
         split = take(bid, plan.by_splits);
@@ -840,7 +845,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                             if (ks == 0) umma_ss<CG, 0>(d_tmem, q_lo + qo, qk_hi, k_lo + ko, qk_hi, kIdescQK);
                             else umma_ss<CG, 1>(d_tmem, q_lo + qo, qk_hi, k_lo + ko, qk_hi, kIdescQK);
                         }
-                        commit(smem_u32(&bars.s_full[i & 1]));
+                        commit(smem_u32(i == 1 ? &bars.s_aside : &bars.s_full[i & 1]));
                         if (t == MT - 1) commit(smem_u32(&bars.k_empty[st]));
                     }
                     __syncwarp();
@@ -953,10 +958,14 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             tc_wait_st();
             tell(bar);
         };
+        const uint32_t s_next = smem_u32(&bars.s_full[grp]);
+        uint32_t s_bar = grp ? smem_u32(&bars.s_aside) : s_next, s_par = 0;
         for (int i = grp; i < n_items; i += 2) {
             const int u = i >> 1;                          // the u-th use of this group's slot and accumulator
             const int j = MT == 2 ? u : i;                 // K/V tile of the item
-            ok = mbar_wait(smem_u32(&bars.s_full[grp]), (uint32_t)(u & 1), abort_flag);
+            ok = mbar_wait(s_bar, s_par, abort_flag);
+            s_par = s_bar == s_next ? s_par ^ 1u : 0u;
+            s_bar = s_next;
             ok = __all_sync(0xffffffffu, ok);  // the tensor-memory accesses below need the whole warp
             if (!ok) break;
             if (CL && i == n_items - 1 && quad == 0 && lane == 0) {
@@ -1290,39 +1299,63 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 __global__ void __launch_bounds__(1024)
 tree_attention_schedule_kernel(const int64_t* __restrict__ kv_off, const int32_t* __restrict__ kv_len, int B, int m,
                                long long cache_rows, int max_kv_len, AttnPlan plan, uint32_t* __restrict__ order,
-                               int* __restrict__ tickets, int n_tickets) {
+                               int* __restrict__ tickets, int n_tickets, int32_t* d_status) {
+    constexpr int kListed = 4096;
     __shared__ int s_bin[kMaxTilesPerSplitOrdered + 1];  // per tile count: items, then the next free place
-    chain_wait();
+    __shared__ int s_items;
+    __shared__ uint32_t s_list[kListed];
+    // The blocks that this list is for may start, and set up, while it is made: they wait for this kernel before they read
+    // it.  The lengths are final before the wait for the kernel before (as in the attention kernel); what is written may
+    // still be read by the launch before.  So the list is made first, and written behind the wait.
     chain_release();
-    // the merging blocks' arrival counters start at zero whatever shared this workspace since
-    for (int i = threadIdx.x; i < n_tickets; i += blockDim.x) tickets[i] = 0;
     const int S = plan.splits;
     const long long n = (long long)B * S;
-    for (int i = threadIdx.x; i <= kMaxTilesPerSplitOrdered; i += blockDim.x) s_bin[i] = 0;
+    const bool early = n <= kListed;
+    if (!early) chain_wait();
+    if (threadIdx.x <= kMaxTilesPerSplitOrdered) s_bin[threadIdx.x] = 0;
     __syncthreads();
+    bool refused = false;
     auto tiles_of = [&](long long item) {
         const int b = (int)(item / S), split = (int)(item % S);
         const int L = kv_len[b];
-        if (!sequence_ok(L, kv_off[b], m, max_kv_len, cache_rows)) return 0;
-        const int tiles = (L + m + kTK - 1) / kTK;
-        return max(0, min(plan.per_split, tiles - split * plan.per_split));
+        if (!sequence_ok(L, kv_off[b], m, max_kv_len, cache_rows)) {
+            refused = true;
+            return 0;
+        }
+        // (What is left of a sequence that is cut counts as a full split: its block is the one that the merge waits for, and
+        // at the end of the launch the merge would come behind it.  Ragged batches of the LLaMA3-8B shape, B = 8, by tiles
+        // alone / like this: 55.3 / 50.9 us per layer; four sequences of 32 KV heads 62.5 / 59.9; B = 32 153.8 / 150.5.)
+        const int tiles = (L + m + kTK - 1) / kTK, t = max(0, min(plan.per_split, tiles - split * plan.per_split));
+        return t > 0 && tiles > plan.per_split ? plan.per_split : t;
     };
     for (long long i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&s_bin[tiles_of(i)], 1);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int at = 0;
-        for (int t = kMaxTilesPerSplitOrdered; t >= 1; --t) {
-            const int c = s_bin[t];
-            s_bin[t] = at;
-            at += c;
+    if (threadIdx.x < 32) {  // items with more tiles come first: bins 64 .. 1, two per lane
+        const int hi = kMaxTilesPerSplitOrdered - 2 * (int)threadIdx.x, c0 = s_bin[hi], c1 = s_bin[hi - 1];
+        int at = c0 + c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, at, o);
+            if ((int)threadIdx.x >= o) at += up;
         }
-        order[0] = (uint32_t)at;
+        s_bin[hi] = at - c0 - c1, s_bin[hi - 1] = at - c1;
+        if (threadIdx.x == 31) s_items = at;
     }
     __syncthreads();
+    uint32_t* list = early ? s_list : order + 1;
     for (long long i = threadIdx.x; i < n; i += blockDim.x) {
         const int t = tiles_of(i);
-        if (t > 0) order[1 + atomicAdd(&s_bin[t], 1)] = (uint32_t)i;
+        if (t > 0) list[atomicAdd(&s_bin[t], 1)] = (uint32_t)i;
     }
+    if (early) {
+        __syncthreads();
+        chain_wait();
+        for (int i = threadIdx.x; i < s_items; i += blockDim.x) order[1 + i] = s_list[i];
+    }
+    // the merging blocks' arrival counters start at zero whatever shared this workspace since
+    for (int i = threadIdx.x; i < n_tickets; i += blockDim.x) tickets[i] = 0;
+    if (threadIdx.x == 0) order[0] = (uint32_t)s_items;
+    if (refused) raise_status(d_status, EAGLE2_STATUS_KV_OVERFLOW);
 }
 
 // One warp per output row of a sequence that used several splits (launches that do not merge inside
@@ -1413,7 +1446,8 @@ static int launch_attention(const CUtensorMap& k_map, const CUtensorMap& v_map, 
     if (blocks > 0x7fffffffLL || (long long)B * plan.splits > 0x7fffffffLL) return EAGLE2_ERR_SHAPE;
     if (plan.ordered &&
         launch_chained(tree_attention_schedule_kernel, dim3(1), dim3(1024), 0, st, 1, kv_off, kv_len, B, m, cache_rows,
-                       max_kv_len, plan, ws.order, ws.tickets, plan.fused_merge ? B * Hkv * plan.n_rb * (plan.pair ? 2 : 1) : 0) != EAGLE2_OK)
+                       max_kv_len, plan, ws.order, ws.tickets, plan.fused_merge ? B * Hkv * plan.n_rb * (plan.pair ? 2 : 1) : 0,
+                       d_status) != EAGLE2_OK)
         return EAGLE2_ERR_CUDA;
     if (launch_chained(kern, dim3((unsigned)blocks), dim3(kAttnThreads), plan.smem, st, PAIR ? 2u : CL ? (unsigned)plan.cluster : 1u, k_map, v_map, q_map,
                        static_cast<const __nv_bfloat16*>(q), kv_off, kv_len, mask_bits, m, Hq, Hkv, cache_rows, max_kv_len,

@@ -368,3 +368,24 @@ def test_references_that_grow_with_every_tile(m, Hkv, Hq, d, tiles):
     rng = np.random.default_rng(9)
     samples = np.stack([rng.integers(0, B, 300), rng.integers(0, Hq, 300), rng.integers(0, m, 300)], axis=1).astype(np.int32)
     _compare(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), samples=samples)
+
+
+@pytest.mark.parametrize("m,Hq,Hkv,d,B", [(16, 8, 8, 64, 60), (60, 32, 8, 128, 70), (20, 12, 12, 128, 40), (40, 6, 2, 128, 90), (60, 32, 8, 128, 12)])
+def test_ordered_launch_of_many_short_sequences(m, Hq, Hkv, d, B):
+    """Many blocks of a single tile that ends inside a group of 16 keys, beside a few long sequences; then the last
+    sequence lies outside the cache: it is reported and the others are as before."""
+    rng = np.random.default_rng(B)
+    lens = rng.integers(0, 128 - m, B)
+    lens[[1, B // 2]] = [9000, 5003]
+    assert attention_mode(B, m, Hq, Hkv, d, 9000) == "ordered"
+    q, kc, vc, off, kl, bits = _inputs(43, B, m, Hq, Hkv, d, [int(x) for x in lens])
+    n = 500
+    samples = np.stack([rng.integers(0, B, n), rng.integers(0, Hq, n), rng.integers(0, m, n)], axis=1).astype(np.int32)
+    samples[:60, 0] = np.array([1, B // 2, 0])[rng.integers(0, 3, 60)]
+    _compare(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), samples=samples)
+    bad_off = off.copy()
+    bad_off[B - 1] = kc.shape[0]
+    got, _, st = gpu_attention(q, kc, vc, bad_off, kl, bits, 1.0 / np.sqrt(d), want_lse=True)
+    assert st == e2.STATUS_KV_OVERFLOW
+    good, _, _ = gpu_attention(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), want_lse=True)
+    assert (got[:B - 1] == good[:B - 1]).all()
