@@ -777,7 +777,9 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         if (has_tail && ok) {
             // (every earlier use of the last V tile's stage is over: its barrier can be waited for directly)
             last_st = __shfl_sync(0xffffffffu, last_st, 0), last_ph = __shfl_sync(0xffffffffu, last_ph, 0);
-            if (mbar_wait(smem_u32(&bars.v_full[last_st]), last_ph, abort_flag)) {
+            // (One answer for the whole warp: lanes that waited apart, some until the tile was there and some until the bound
+            // ran out, would not meet again, and the meetings of the block further down would wait for them without end.)
+            if (__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.v_full[last_st]), last_ph, abort_flag))) {
                 constexpr int PANELS = PAIR ? 1 : HALVES;
                 const int chunks = (groups_t * 16 - valid_t) * 8;
                 for (int idx = lane; idx < chunks; idx += 32)
@@ -816,7 +818,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.q_peer), 0);
                 for (int j = 0; j < nt && ok; ++j) {
                     ok = wait1(smem_u32(&bars.k_full[st]), ph);
-                    if (j == 0 && lane == 0) mbar_arrive(smem_u32(&bars.v_go));
+                    if (ok && j == 0 && lane == 0) mbar_arrive(smem_u32(&bars.v_go));
                     if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.k_peer[st]), 0);
                     if (++st == NST) st = 0, ph ^= 1u;
                 }
@@ -828,7 +830,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                     const int t = i & (MT - 1);
                     if (t == 0) {
                         ok = ok && wait1(smem_u32(&bars.k_full[st]), ph);
-                        if (PAIR && i == 0 && lane == 0) mbar_arrive(smem_u32(&bars.v_go));
+                        if (PAIR && ok && i == 0 && lane == 0) mbar_arrive(smem_u32(&bars.v_go));
                         if (PAIR) ok = ok && wait1(smem_u32(&bars.k_peer[st]), ph);
                     }
                     // (item 0 has been read before item 2 overwrites it, item i - 1 before item i; item 1 has columns of its own)
@@ -1059,6 +1061,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             ok = mbar_wait(smem_u32(&bars.o_done[grp]), (uint32_t)((n_uses - 1) & 1), abort_flag);
         if (CL) ok = ok && mbar_wait(smem_u32(&bars.peers_ready), 0, abort_flag);
         if (MT == 1) s_half[grp][r_tile] = make_float2(m_ref, l_run);
+        __syncwarp();
         ok = named_barrier_and(1, kSoftmaxThreads, ok);
         if (ok) {
             tc_fence_after();
@@ -1161,6 +1164,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         }
     }
     }  // active
+    __syncwarp();
     if (CL && !(active && warp < kTmaWarp)) {
         __syncwarp();
         cluster_wait();
