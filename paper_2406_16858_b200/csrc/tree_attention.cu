@@ -621,15 +621,6 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             if (CL) mbar_init(smem_u32(&bars.peers_ready), plan.cluster), mbar_init(smem_u32(&bars.inbox), 1 + kSoftmaxThreads / 32);
             fence_barrier_init();
         }
-        if (warp == kMmaWarp) {
-            if (PAIR) {
-                tmem_alloc2(smem_u32(&s_tmem_base), kTmemCols);
-                tmem_relinquish2();
-            } else {
-                tmem_alloc(smem_u32(&s_tmem_base), kTmemCols);
-                tmem_relinquish();
-            }
-        }
         if (warp == kTmaWarp && lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&k_map) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(&v_map) : "memory");
@@ -642,11 +633,26 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     // made visible by the fence behind their initialisation, so that the meeting need not order memory (the
     // releasing form took 0.5 us of the 1.1 us before a launch's first request).
     auto meet = [&]() {
-        tc_fence_before();
         if (PAIR) cluster_sync_all();
         else __syncthreads();
         if (CL) cluster_arrive_relaxed();
+        // Tensor memory takes another half a microsecond.  Only the warps that use it wait for it (tmem_ready); the first
+        // tiles are asked for meanwhile.
+        if (warp == kMmaWarp) {
+            if (PAIR) {
+                tmem_alloc2(smem_u32(&s_tmem_base), kTmemCols);
+                tmem_relinquish2();
+            } else {
+                tmem_alloc(smem_u32(&s_tmem_base), kTmemCols);
+                tmem_relinquish();
+            }
+        }
+    };
+    auto tmem_ready = [&]() {  // softmax and MMA warps
+        tc_fence_before();
+        asm volatile("bar.sync 2, %0;" ::"n"(kSoftmaxThreads + 64) : "memory");
         tc_fence_after();
+        return s_tmem_base;
     };
     if (plan.setup_first) set_up();
     // (such a launch also works out which tiles and rows the block serves before it waits: below)
@@ -699,7 +705,6 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         set_up();
         meet();
     }
-    const uint32_t tmem = s_tmem_base;
     volatile WaitCtl* abort_flag = &s_ctl;
     // Cluster launches: block j combines the rows [j * own, (j + 1) * own) of the row block; rows_of(j) of them exist
     // (to the next even number: row pairs travel together).  The inbox barrier counts what the other blocks' copies
@@ -803,6 +808,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         // lanes, so that descriptors and addresses stay in uniform registers, where the instruction wants them (a lane
         // on its own moves them there one by one: ~90 cycles per instruction beside busy softmax warps, which is slower
         // than the tensor pipe).
+        const uint32_t tmem = tmem_ready();
         auto wait1 = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait_spin(bar, parity, abort_flag)) != 0; };
         auto commit = [&](uint32_t bar) {
             if (PAIR) tc_commit2(bar);
@@ -914,6 +920,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         // reference maximum, row sums and accumulator, and the epilogue combines the two.  A thread owns a
         // row: its 128 scores stay in registers from the tensor-memory read to the packed probabilities, so
         // nothing is read twice and no two threads exchange anything.
+        const uint32_t tmem = tmem_ready();
         if (CL) cluster_wait();  // (the meeting of the cluster's blocks, see above)
         __shared__ float2 s_half[2][128];                 // epilogue, one row tile: [group][row] (reference, sum)
         const int grp = warp >> 2, quad = warp & 3;
@@ -1293,8 +1300,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         tc_fence_after();
     }
     if (warp == kMmaWarp) {
-        if (PAIR) tmem_dealloc2(tmem, kTmemCols);
-        else tmem_dealloc(tmem, kTmemCols);
+        if (PAIR) tmem_dealloc2(s_tmem_base, kTmemCols);
+        else tmem_dealloc(s_tmem_base, kTmemCols);
     }
     if (tid == 0 && s_ctl.abort) raise_status(d_status, EAGLE2_STATUS_TIMEOUT);
     __syncwarp();
