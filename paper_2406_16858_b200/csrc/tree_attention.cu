@@ -71,7 +71,8 @@ struct AttnPlan {
     int mt;         // 128-row tiles per block: 1 or 2
     int splits;     // KV splits per sequence (blocks of the launch)
     int per_split;  // K/V tiles per split
-    int stages;     // K/V ring depth
+    int stages;     // V ring depth
+    int k_stages;   // K ring depth
     int setup_first;  // 1: blocks set up barriers and tensor memory before they wait for the preceding
                       // kernel (worth it when no block of the launch is expected to be idle: three sequences of 40 heads
                       // 26.4 -> 25.3 us per layer, two of 8 KV heads and 444 keys 9.7 -> 8.7)
@@ -88,7 +89,7 @@ struct AttnPlan {
                       // block) to finish combines the splits' partials itself, while other blocks still run
     int tile_tok;   // query rows by TMA: tree tokens per 128-row tile
     FastDiv by_g, by_splits, by_n_rb, by_hkv, by_per_split, by_own;
-    size_t smem;
+    size_t smem, smem_most;  // shared memory of the launch, and the most that a launch of the same kernel takes
     long long wait_limit;  // bound of every device-side wait of the launch, in clock cycles
 };
 
@@ -97,11 +98,18 @@ struct AttnPlan {
 static int resident_clusters(int size);
 
 static size_t operand_tile_bytes(int d) { return (size_t)(d / 64) * kTK * 128; }  // 128 rows
-static void ring_of(AttnPlan* p, int d) {  // (the same for every plan with as many row tiles and the same head size)
+static void ring_of(AttnPlan* p, int d) {
     const size_t unit = operand_tile_bytes(d);
     int stages = (int)((220 * 1024 - p->mt * unit) / (2 * unit));
     p->stages = stages > 4 ? 4 : (stages < 2 ? 2 : stages);
-    p->smem = (p->mt + 2 * (size_t)p->stages) * unit + 1024;
+    // A K tile more where it fits (Q.K^T runs up to three items ahead of P.V), in blocks of a few tiles, whose third
+    // tile then does not wait for the first Q.K^T: 30 sequences of 32 heads, 232 keys 62.2 -> 60.2 us per layer, 24 of 40, 739
+    // keys 95.4 -> 94.2.  In longer blocks, and where one sequence is split over all SMs, the V tiles come later for it
+    // (three sequences of 40 heads, 19 tiles 25.35 -> 25.6; 10 rows at 12345 keys 18.4 -> 18.7).
+    const int more = (p->mt + 2 * (size_t)p->stages + 1) * unit <= 212 * 1024 ? 1 : 0;
+    p->k_stages = p->stages + (p->per_split <= 8 && (p->splits == 1 || p->cluster > 1) ? more : 0);
+    p->smem = (p->mt + (size_t)p->stages + p->k_stages) * unit + 1024;
+    p->smem_most = (p->mt + 2 * (size_t)p->stages + more) * unit + 1024;
 }
 constexpr int kPairStages = 4, kPairStagesOrdered = 5;
 static size_t pair_smem(int stages, int d) { return (1 + (size_t)stages) * operand_tile_bytes(d) + 1024; }
@@ -211,7 +219,7 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
     p->wait_limit = wait_limit_cycles();
     p->setup_first = B == 1;  // ragged batches leave many splits without tiles: those leave at once
     if (p->pair) {  // per block: one 128-row query tile, half-size K and V stages
-        p->stages = p->ordered ? kPairStagesOrdered : kPairStages;
+        p->stages = p->k_stages = p->ordered ? kPairStagesOrdered : kPairStages;
         p->smem = pair_smem(p->stages, d);
     }
 }
@@ -555,14 +563,14 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     // cluster launches: (reference maximum, sum) of this block's rows, and those that arrived for its share
     __shared__ __align__(16) float2 s_ml[CL ? MT * 128 : 1], s_ml_in[CL ? MT * 128 + 2 * kMaxCluster : 1];
 
-    const int g = plan.g, M = plan.M, S = plan.splits, NST = plan.stages;
+    const int g = plan.g, M = plan.M, S = plan.splits, NST = plan.stages, NSTK = plan.k_stages;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;  // 0: the block that issues the pair's MMAs
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (uniform over the warp, and known to be)
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sQ = smem_base;
     const uint32_t sK = sQ + MT * kTile;
-    const uint32_t sV = sK + (uint32_t)NST * kKTile;
+    const uint32_t sV = sK + (uint32_t)NSTK * kKTile;
     unsigned char* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
 
     // place of the block: (sequence, KV head, row block, split); an ordered launch has it from its list, below
@@ -593,7 +601,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     // ---- set-up: barriers, tensor memory (reads nothing an earlier kernel could have written); a lane per
     // ring stage, one for the rest ----
     auto set_up = [&]() {
-        if (tid < NST) {
+        if (tid < NSTK) {  // (never fewer than V stages)
             mbar_init(smem_u32(&bars.k_full[tid]), 1);
             mbar_init(smem_u32(&bars.k_empty[tid]), 1);
             mbar_init(smem_u32(&bars.v_full[tid]), 1);
@@ -733,14 +741,14 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             int st = 0, row = (int)(row_base + (long long)t_begin * kTK);
             uint32_t ph = 1;
             for (int j = 0; j < nt; ++j, row += kTK) {
-                if (j >= NST && !mbar_wait(smem_u32(&bars.k_empty[st]), ph, abort_flag)) break;
+                if (j >= NSTK && !mbar_wait(smem_u32(&bars.k_empty[st]), ph, abort_flag)) break;
                 mbar_expect_tx(smem_u32(&bars.k_full[st]), kKTile);
 #pragma unroll
                 for (int h = 0; h < HALVES; ++h)  // a pair block takes its 64 of the tile's 128 keys
                     tma_load_3d(sK + st * kKTile + h * kKPanel, &k_map, h * 64, hk, row + (int)rank * (kTK / 2),
                                 smem_u32(&bars.k_full[st]), policy);
                 k_issued = j + 1;
-                if (++st == NST) st = 0, ph ^= 1u;
+                if (++st == NSTK) st = 0, ph ^= 1u;
             }
         }
         __syncwarp();
@@ -830,7 +838,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                     ok = wait1(smem_u32(&bars.k_full[st]), ph);
                     if (ok && j == 0 && lane == 0) mbar_arrive(smem_u32(&bars.v_go));
                     if (ok && lane == 0) mbar_arrive_in(smem_u32(&bars.k_peer[st]), 0);
-                    if (++st == NST) st = 0, ph ^= 1u;
+                    if (++st == NSTK) st = 0, ph ^= 1u;
                 }
             } else {
                 if (PAIR) ok = ok && wait1(smem_u32(&bars.q_peer), 0);
@@ -861,7 +869,7 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                         if (t == MT - 1) commit(smem_u32(&bars.k_empty[st]));
                     }
                     __syncwarp();
-                    if (t == MT - 1 && ++st == NST) st = 0, ph ^= 1u;
+                    if (t == MT - 1 && ++st == NSTK) st = 0, ph ^= 1u;
                 }
             }
         } else if (PAIR && rank != 0) {
@@ -1290,8 +1298,8 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 mbar_drain(smem_u32(&bars.v_full[j % NST]), (uint32_t)((j / NST) & 1));
         }
         if (warp == kTmaWarp && lane == 0) {
-            for (int j = max(0, k_issued - NST); j < k_issued; ++j)
-                mbar_drain(smem_u32(&bars.k_full[j % NST]), (uint32_t)((j / NST) & 1));
+            for (int j = max(0, k_issued - NSTK); j < k_issued; ++j)
+                mbar_drain(smem_u32(&bars.k_full[j % NSTK]), (uint32_t)((j / NSTK) & 1));
         }
         __syncwarp();
         tc_fence_before();
@@ -1425,7 +1433,7 @@ static int resident_clusters(int size) {
     if (known) return known - 1;
     auto kern = tree_attention_kernel<128, 2, false, true>;
     AttnPlan plan;
-    plan.mt = 2;
+    plan.mt = 2, plan.per_split = plan.splits = plan.cluster = 0;
     ring_of(&plan, 128);  // what the kernel's launches take: one block per SM
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)size * 64), cfg.blockDim = dim3(kAttnThreads), cfg.dynamicSmemBytes = plan.smem;
@@ -1452,7 +1460,7 @@ static int launch_attention(const CUtensorMap& k_map, const CUtensorMap& v_map, 
                             cudaStream_t st) {
     auto kern = tree_attention_kernel<DH, MT, PAIR, CL>;
     // (always the same value for a kernel, whatever the plan: concurrent callers with other plans set it too)
-    const size_t most = PAIR ? pair_smem(kPairStagesOrdered, DH) : plan.smem;
+    const size_t most = PAIR ? pair_smem(kPairStagesOrdered, DH) : plan.smem_most;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) {
         cudaGetLastError();
         return EAGLE2_ERR_CUDA;
