@@ -39,6 +39,7 @@ namespace eagle2 {
 constexpr int kTK = 128;              // keys per K/V tile = N of the Q.K^T instruction
 constexpr int kRowsPerTile = 128;     // M of every tcgen05.mma
 constexpr int kMaxTilesPerSplit = 16; // sequences that would need longer blocks are served longest first (batches)
+constexpr int kMaxByLength = 256;      // sequences that a block can rank
 constexpr int kMaxTilesPerSplitOrdered = 64;  // a block never streams more than 8192 keys
 constexpr int kTmemCols = 512;
 constexpr int kMaxCluster = 8;
@@ -85,6 +86,7 @@ struct AttnPlan {
     int cluster;    // > 1: the blocks of a (sequence, KV head, row block) form a cluster, share out the sequence's
                     // tiles evenly and combine their partial rows through distributed shared memory
     int own;        // cluster launches: packed rows that each block of the cluster combines (even)
+    int by_length;  // 1: blocks take whole sequences, the longest first, and each finds its own by counting
     int fused_merge;  // 1 (ordered launches with several splits): the last block of a (sequence, KV head, row
                       // block) to finish combines the splits' partials itself, while other blocks still run
     int tile_tok;   // query rows by TMA: tree tokens per 128-row tile
@@ -150,7 +152,7 @@ static bool single_wave_plan(int B, int m, int Hkv, int d, int tiles, AttnPlan* 
     p->own = ((p->per + best_c - 1) / best_c + 1) / 2 * 2;
     p->splits = best_c;
     p->per_split = (tiles + best_c - 1) / best_c;
-    p->pair = p->ordered = p->fused_merge = 0;
+    p->pair = p->ordered = p->fused_merge = p->by_length = 0;
     p->wait_limit = wait_limit_cycles();
     p->setup_first = 1;
     ring_of(p, d);
@@ -189,8 +191,8 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
     p->ordered = (B > 1 && !p->pair && per_split > kMaxTilesPerSplit) ? 1 : 0;
     // An ordered launch with few (sequence, KV head) items - up to one and a half per TPC - runs on
     // pairs as well: with so few items the longest sequences decide the time, and a pair puts two SMs
-    // on each of their splits (measured per layer, ragged batches of the LLaMA3-8B shape: B = 8 86 ->
-    // 67 us, B = 12 112 -> 104 us; with more items pairs lose: B = 16 112 -> 119 us, B = 32 181 -> 216 us).
+    // on each of their splits (measured per layer, ragged batches of the LLaMA3-8B shape, single blocks / pairs: B = 8
+    // 59.4 / 49.7 us, B = 12 71.7 / 67.1; with more items pairs lose: B = 16 78.3 / 84.0, B = 20 68.6 / 70.1).
     const bool ordered_pair = p->ordered && p->mt == 2 && p->q_tma && d == 128 && 2 * items <= 3 * tpcs;
     if (ordered_pair) p->pair = 1;
     const int units = p->pair ? tpcs : sms;  // blocks (pairs) resident at once
@@ -215,9 +217,16 @@ static void attention_plan_sizes(int B, int m, int Hq, int Hkv, int d, int max_k
     p->per_split = per_split;
     p->splits = (tiles + per_split - 1) / per_split;
     p->fused_merge = (p->ordered && p->splits > 1) ? 1 : 0;
+    // More blocks than SMs, a whole sequence each: the longest first here too, but every block finds its sequence by itself
+    // (a list from another kernel costs 1.5-2 us of a layer, which a batch of equal lengths loses).  Per layer, in index order /
+    // longest first: 20 sequences of 8 KV heads, 300-1900 keys 47.1 / 35.3 us, 16 of 64/8 heads, 150-1980 keys 47.6 / 37.4,
+    // five of 40 heads, 300-1900 keys 30.2 / 26.1, 26 of head_dim 64, 253-1500 keys 25.6 / 21.5; equal lengths 0.98-1.01.  With
+    // more than four waves the end of the launch weighs little and blocks of all lengths side by side are better: 30
+    // sequences of 32 heads, 150-700 keys 67.6 / 73.0.
+    p->by_length = (B > 1 && B <= kMaxByLength && !p->ordered && p->splits == 1 && items > sms && items <= 4LL * sms) ? 1 : 0;
     ring_of(p, d);
     p->wait_limit = wait_limit_cycles();
-    p->setup_first = B == 1;  // ragged batches leave many splits without tiles: those leave at once
+    p->setup_first = B == 1 || p->by_length;  // ragged batches leave many splits without tiles: those leave at once
     if (p->pair) {  // per block: one 128-row query tile, half-size K and V stages
         p->stages = p->k_stages = p->ordered ? kPairStagesOrdered : kPairStages;
         p->smem = pair_smem(p->stages, d);
@@ -596,7 +605,25 @@ tree_attention_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     const bool early_len = plan.setup_first && !plan.ordered;
     int len_early = 0;
     long long off_early = 0;
-    if (early_len) len_early = kv_len[b], off_early = kv_off[b];
+    if (plan.by_length) {  // the b-th longest sequence, ties to the lower index
+        __shared__ int s_lens[kMaxByLength], s_place;
+        __shared__ long long s_off;
+        const int n = gridDim.x / (Hkv * plan.n_rb);
+        const int mine = tid < n ? kv_len[tid] : 0;
+        const long long off = tid < n ? kv_off[tid] : 0;
+        if (tid < n) s_lens[tid] = mine;
+        __syncthreads();
+        if (tid < n) {
+            int before = 0;
+#pragma unroll 8
+            for (int j = 0; j < n; ++j) before += s_lens[j] > mine || (s_lens[j] == mine && j < tid) ? 1 : 0;
+            if (before == b) s_place = tid, s_off = off;
+        }
+        __syncthreads();
+        b = s_place, len_early = s_lens[b], off_early = s_off;
+    } else if (early_len) {
+        len_early = kv_len[b], off_early = kv_off[b];
+    }
 
     // ---- set-up: barriers, tensor memory (reads nothing an earlier kernel could have written); a lane per
     // ring stage, one for the rest ----

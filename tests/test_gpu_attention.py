@@ -389,3 +389,22 @@ def test_ordered_launch_of_many_short_sequences(m, Hq, Hkv, d, B):
     assert st == e2.STATUS_KV_OVERFLOW
     good, _, _ = gpu_attention(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), want_lse=True)
     assert (got[:B - 1] == good[:B - 1]).all()
+
+
+@pytest.mark.parametrize("m,Hq,Hkv,d,B", [(60, 32, 8, 128, 20), (33, 32, 32, 64, 6), (20, 12, 6, 128, 50)])
+def test_whole_sequences_longest_first(m, Hq, Hkv, d, B):
+    """More blocks than SMs, a sequence each: equal lengths among them, empty ones, and one outside the cache."""
+    rng = np.random.default_rng(B)
+    lens = rng.integers(0, 700, B)
+    lens[[0, B // 2, B - 1]] = [1500, 1500, 0]
+    q, kc, vc, off, kl, bits = _inputs(44, B, m, Hq, Hkv, d, [int(x) for x in lens])
+    assert attention_mode(B, m, Hq, Hkv, d, 1500) == "no partial rows in memory"
+    n = 500
+    samples = np.stack([rng.integers(0, B, n), rng.integers(0, Hq, n), rng.integers(0, m, n)], axis=1).astype(np.int32)
+    good = _compare(q, kc, vc, off, kl, bits, 1.0 / np.sqrt(d), samples=samples)
+    bad_off = off.copy()
+    bad_off[1] = kc.shape[0]
+    got, _, st = gpu_attention(q, kc, vc, bad_off, kl, bits, 1.0 / np.sqrt(d), want_lse=True)
+    assert st == e2.STATUS_KV_OVERFLOW
+    others = np.arange(B) != 1
+    assert (gen.bf16_bits_to_f32(got)[others] == good[others]).all()
